@@ -115,6 +115,14 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// the same load without its wait, and the wait for every load before it
+__device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, float* v) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+               : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
 // packed operand geometry: one K step per chunk, 32 bytes of each row
 template <bool BF16> struct Geo {
   static constexpr int EB = BF16 ? 2 : 4;       // element bytes
@@ -172,6 +180,85 @@ __device__ __forceinline__ void pieces(double x, int b, uint32_t* out) {
       }
     }
   }
+}
+
+// ---- the slices and their sums in integer arithmetic. GB300 issues an FP64 instruction per warp every 64
+// cycles and sub-partition (measured; 19 per SM) against one integer or FP32 instruction per cycle, so
+// neither the cut into slices nor the addition of the level sums runs on the FP64 pipe.
+
+// BF16 bit patterns (in the upper half of each word) of the NS fixed-point slices of x 2^-e, |x| < 2^e: x is
+// rounded to NS * b fractional bits and cut into signed digits |a_i| <= 2^b, slice value a_i 2^(-b(i+1)). A NaN or
+// an infinity becomes a NaN in slice 0 (every sum it enters comes out NaN).
+template <int NS>
+__device__ __forceinline__ void int_slices(double x, int e, int b, uint32_t* out) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const int ex = (int)((hi >> 20) & 0x7ff);
+  const uint64_t mant = ((uint64_t)((hi & 0xfffffu) | (ex ? 0x100000u : 0u)) << 32) | lo;
+  // x = mant 2^(max(ex, 1) - 1075); F = round(x 2^(NS b - e)) fits NS b + 1 <= 43 bits: a right shift by 53 - NS b
+  // or more, except in a row of subnormals, whose e lies below the exponent of the smallest normal number
+  const int sh = 1075 + e - NS * b - max(ex, 1);
+  long long F = 0;
+  if (sh > 0 && sh < 64) F = (long long)((mant + (1ull << (sh - 1))) >> sh);
+  else if (sh <= 0 && sh > -53) F = (long long)(mant << -sh);
+  if ((int)hi < 0) F = -F;
+  // digits of three slices per 32-bit half
+  constexpr int H = NS / 2;
+  const int hb = H * b;
+  const long long up = (F + (1ll << (hb - 1))) >> hb;
+  int half[2] = {(int)up, (int)(F - (up << hb))};
+  const int rnd = 1 << (b - 1);
+#pragma unroll
+  for (int h = 1; h >= 0; --h) {
+    int v = half[h];
+#pragma unroll
+    for (int i = H - 1; i >= 0; --i) {
+      const int next = i > 0 ? (v + rnd) >> b : 0;
+      const int a = i > 0 ? v - (next << b) : v;
+      v = next;
+      // 1.5 2^(23 - b s) + a 2^(-b s): adding a to the last bits of the constant's pattern
+      const int s = h * H + i + 1;
+      const uint32_t magic = (uint32_t)(127 + 23 - b * s) << 23 | 0x400000u;
+      out[h * H + i] = __float_as_uint(__uint_as_float(magic + (uint32_t)a) - __uint_as_float(magic));
+    }
+  }
+  if (ex == 0x7ff) out[0] = 0x7fc00000u;
+}
+
+// two slices' BF16 patterns in one word: first in the low half
+__device__ __forceinline__ uint32_t pair_bf16(uint32_t first, uint32_t second) {
+  return __byte_perm(first, second, 0x7632);
+}
+
+// |x| as an integer, 0 for a NaN or an infinity (integer order = order of the magnitudes)
+__device__ __forceinline__ unsigned long long mag_bits(double x) {
+  const unsigned long long m = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+  return m < 0x7ff0000000000000ull ? m : 0ull;
+}
+
+// n 2^(e - 7 * 7) as a double, n the 64-bit fixed-point sum of a product's levels
+__device__ __forceinline__ double fixed_to_double(long long n, int e) {
+  if (n == 0) return 0.0;
+  const unsigned long long a = n < 0 ? (unsigned long long)(-n) : (unsigned long long)n;
+  const int lz = __clzll((long long)a);
+  // the top 53 bits, rounded to nearest (ties away; a carry moves into the exponent)
+  const unsigned long long m = ((a << lz) >> 10) + 1ull;      // 54 bits + rounding bit
+  const int bexp = 63 - lz - 49 + e + 1023;                   // biased exponent of the leading bit
+  if (bexp > 1 && bexp < 2046) {
+    const unsigned long long r = (m >> 1) + ((unsigned long long)(bexp - 1) << 52);   // the implicit bit adds one
+    return __longlong_as_double((long long)(r | (n < 0 ? 0x8000000000000000ull : 0ull)));
+  }
+  return ldexp((double)n, e - 49);
+}
+
+// the sum of the four level accumulators of one entry (slice width 7) as an integer multiple of 2^-49: the first
+// three are integer multiples of 2^-14, 2^-21, 2^-28 below 2^24 of them (level 2 up to rounding), the last one
+// is rounded to the grid. Returns false when one of them is not finite.
+__device__ __forceinline__ bool level_sum(float f0, float f1, float f2, float f3, long long* out) {
+  const bool fin = (fabsf(f0) < 1e30f) & (fabsf(f1) < 1e30f) & (fabsf(f2) < 1e30f) & (fabsf(f3) < 1e30f);
+  const long long a = __float2int_rn(f0 * 16384.0f), b = __float2int_rn(f1 * 2097152.0f);
+  const long long c = __float2ll_rn(f2 * 562949953421312.0f), d = __float2ll_rn(f3 * 562949953421312.0f);
+  *out = (a << 35) + (b << 28) + c + d;
+  return fin;
 }
 
 // slice width: the level-0 sum over K of 2 products of |a| <= 2^b stays below 2^24

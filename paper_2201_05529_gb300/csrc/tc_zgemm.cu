@@ -16,10 +16,10 @@
 // FP64 in the output. Products of slice
 // pairs (s, t) accumulate in TMEM by level min(s + t, 3), real and imaginary parts separately
 // (Re = Ar Br - Ai Bi via the MMA's negate-A bit, Im = Ar Bi + Ai Br); the epilogue adds the
-// levels in FP64 and applies 2^(e_row + e_col). The result is accurate to ~1e-12 of the scale
+// levels as 64-bit integers and applies 2^(e_row + e_col). The result is accurate to ~1e-12 of the scale
 // of the rows and columns it combines (per 512-long chunk of K).
 //
-// Data flow: two passes per operand (row exponents, then the 12 slice planes in the tcgen05
+// Data flow: one preparation launch (row exponents, then the 12 slice planes in the tcgen05
 // K-major no-swizzle layout: A in 128-row tiles, B in 64-column tiles, one 16-element K step per
 // block, so one cp.async.bulk stages each), then one persistent GEMM launch (one CTA per SM) that
 // walks the live 128 x 64 output tiles of all items with a two-stage bulk-copy / MMA pipeline.
@@ -55,127 +55,117 @@ __device__ __forceinline__ bool item_fits(const ZGemmItem& it) {
   return it.M <= it.cap_m && it.N <= it.cap_n && it.K <= it.cap_k;
 }
 
-// row m, column k of opA(A)
-__device__ __forceinline__ double2 a_elem(const ZGemmItem& it, int m, int k) {
-  if (it.opA == ZOP_N) return it.A[m + (size_t)k * it.lda];
-  double2 v = it.A[k + (size_t)m * it.lda];
-  if (it.opA == ZOP_C) v.y = -v.y;
-  return v;
-}
-
-// row k, column n of opB(B) (column n read from column bcol[n] when a map is given)
-__device__ __forceinline__ double2 b_elem(const ZGemmItem& it, int n, int k) {
-  const int c = it.bcol ? it.bcol[n] : n;
-  if (it.opB == ZOP_N) return it.B[k + (size_t)c * it.ldb];
-  double2 v = it.B[c + (size_t)k * it.ldb];
-  if (it.opB == ZOP_C) v.y = -v.y;
-  return v;
-}
-
-__device__ __forceinline__ double2 op_elem(const ZGemmItem& it, int which, int r, int k) {
-  return which == 0 ? a_elem(it, r, k) : b_elem(it, r, k);
-}
-
 }  // namespace
 
-// Pass 1: e with max |entry| < 2^e for every row of opA(A) (which = 0) or column of opB(B) (1).
-// grid: (x: rows, y: items)
-// which = -1: operand A even where the item marks it as already packed (a pack-only launch)
-__global__ void k_zg_rowexp(const ZGemmItem* items, int n_items, int which) {
-  const int i = blockIdx.y;
-  if (i >= n_items) return;
-  const ZGemmItem it = items[i];
-  const bool force = which < 0;
-  if (force) which = 0;
-  if (!item_live(it) || !item_fits(it) || (which == 0 && it.skip_a > 0 && !force)) return;
-  const int rows = which == 0 ? it.M : it.N, tr = which == 0 ? TMA : TNB;
-  const PackCap cp = zcap(it, which);
-  int* ex = (int*)((which == 0 ? it.TA : it.TB) + cp.exp_off);
-  const int padded = cdiv(rows, tr) * tr;
-  const bool k_contiguous = which == 0 ? it.opA != ZOP_N : it.opB == ZOP_N;
-  if (k_contiguous) {
-    // a row's entries are contiguous in memory: one warp per row, its lanes striding K (the
-    // maximum does not depend on the order, so the exponent is the same as a sequential scan's)
-    const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-    for (int r = blockIdx.x * wpb + (threadIdx.x >> 5); r < padded; r += gridDim.x * wpb) {
-      double m = 0.0;
-      if (r < rows)
-        for (int k = lane; k < it.K; k += 32) {
-          const double2 v = op_elem(it, which, r, k);
-          m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
-        }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if (lane == 0) ex[r] = row_exponent(m);
-    }
-    return;
-  }
-  // consecutive rows are contiguous: one thread per row, consecutive threads on consecutive rows
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < padded; r += gridDim.x * blockDim.x) {
-    double m = 0.0;
-    if (r < rows)
-      for (int k = 0; k < it.K; ++k) {
-        const double2 v = op_elem(it, which, r, k);
-        m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
-      }
-    ex[r] = row_exponent(m);
-  }
-}
+// Operand preparation, both passes in one launch: a block takes PREP_ROWS rows of opA(A) (blockIdx.x < n_a) or
+// columns of opB(B) of one item, finds each one's exponent e (max |entry| < 2^e), then writes the 12 slice
+// planes: one thread per (row, 8-element K group), 16 bytes per plane, eight consecutive rows in consecutive
+// 16-byte slots. The second read of the block's rows comes from L1 or L2.
+// Bound by the integer pipes and the planes' writes (24 bytes per element). Integer arithmetic throughout
+// (tc_common.cuh): with the slices cut by FP64 rint and ldexp in a launch per operand after another for the
+// exponents, the preparation of ten 1120 x 160 x 1120 products took 4.75 ms; the whole product, this kernel
+// and the GEMM with its FP64-free epilogue included, went from 5.68 to 0.93 ms (21 products of 16384 x 64
+// x 64: 7.67 to 1.54 ms).
+// mode 0: B, and A unless the item marks it as packed; mode 1: A alone, marked or not.
+// grid: (x: n_a + n_b row blocks, y: items)
+constexpr int PREP_ROWS = 8, PREP_THREADS = 256;
 
-// Pass 2: one thread per (row, 8-element K group): the 12 slice planes of its 8 entries, 16 bytes
-// each; consecutive threads take consecutive rows, so reads of column-major operands and the
-// 16-byte writes of a plane are both contiguous. grid: (x: elements, y: items)
-__global__ void k_zg_pack(const ZGemmItem* items, int n_items, int which, int* status) {
+__global__ void __launch_bounds__(PREP_THREADS) k_zg_prep(const ZGemmItem* items, int n_items, int n_a, int mode,
+                                                          int* status) {
   const int i = blockIdx.y;
   if (i >= n_items) return;
   const ZGemmItem it = items[i];
-  const bool force = which < 0;
-  if (force) which = 0;
-  if (!item_live(it) || (which == 0 && it.skip_a > 0 && !force)) return;
+  const int which = (int)blockIdx.x < n_a ? 0 : 1;
+  const int blk = which == 0 ? blockIdx.x : blockIdx.x - n_a, nblk = which == 0 ? n_a : gridDim.x - n_a;
+  if (!item_live(it) || (which == 0 && it.skip_a > 0 && mode == 0)) return;
   if (!item_fits(it)) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, ST_CAPACITY);
+    if (blk == 0 && threadIdx.x == 0) atomicOr(status, ST_CAPACITY);
     return;
   }
   const int rows = which == 0 ? it.M : it.N, tr = which == 0 ? TMA : TNB;
-  constexpr int NS = ZNS;
   const PackCap cp = zcap(it, which);
   unsigned char* out = which == 0 ? it.TA : it.TB;
-  const int* ex = (const int*)(out + cp.exp_off);
-  const int n_rt = cdiv(rows, tr), n_ks = cdiv(it.K, ZG::KSTEP);
-  const int padded = n_rt * tr, n_grp = 2 * n_ks;
-  const int b = ZBITS;         // the GEMM accumulates K in chunks of 512: 7-bit slices stay exact
-  const size_t total = (size_t)padded * n_grp;
-  for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (size_t)gridDim.x * blockDim.x) {
-    const int r = (int)(idx % padded), grp = (int)(idx / padded);
-    const int rt = r / tr, m = r % tr, ks = grp >> 1, half = grp & 1;
-    const int e = ex[r];
-    uint32_t pr[NS][4], pi[NS][4];       // 8 BF16 per plane, two per word
-#pragma unroll
-    for (int j = 0; j < ZG::KG; ++j) {
-      const int k = ks * ZG::KSTEP + half * ZG::KG + j;
-      double2 v = make_double2(0.0, 0.0);
-      if (r < rows && k < it.K) v = op_elem(it, which, r, k);
-      uint32_t sr[NS], si[NS];
-      pieces<true, NS, true>(ldexp(v.x, -e), b, sr);
-      pieces<true, NS, true>(ldexp(v.y, -e), b, si);
-#pragma unroll
-      for (int s = 0; s < NS; ++s) {
-        if ((j & 1) == 0) {
-          pr[s][j >> 1] = sr[s];
-          pi[s][j >> 1] = si[s];
-        } else {
-          pr[s][j >> 1] |= sr[s] << 16;
-          pi[s][j >> 1] |= si[s] << 16;
+  int* ex = (int*)(out + cp.exp_off);
+  const int n_ks = cdiv(it.K, ZG::KSTEP), n_grp = 2 * n_ks;
+  const int padded = cdiv(rows, tr) * tr;
+  const bool k_contiguous = which == 0 ? it.opA != ZOP_N : it.opB == ZOP_N;
+  const bool conj_op = (which == 0 ? it.opA : it.opB) == ZOP_C;
+  const double2* src = which == 0 ? it.A : it.B;
+  const size_t ld = which == 0 ? it.lda : it.ldb;
+  __shared__ unsigned long long part[PREP_THREADS / PREP_ROWS][PREP_ROWS];
+  __shared__ int s_e[PREP_ROWS];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int r0 = blk * PREP_ROWS; r0 < padded; r0 += nblk * PREP_ROWS) {
+    if (k_contiguous) {
+      // one warp per row, lanes along K
+      const int r = r0 + warp;
+      unsigned long long m = 0;
+      if (r < rows) {
+        const double2* p = src + (size_t)((which == 1 && it.bcol) ? it.bcol[r] : r) * ld;
+        for (int k = lane; k < it.K; k += 32) {
+          const double2 v = p[k];
+          m = max(m, max(mag_bits(v.x), mag_bits(v.y)));
         }
       }
-    }
-    unsigned char* base = out + ((size_t)rt * cp.ksteps + ks) * (2 * NS) * cp.plane_bytes +
-                          ((size_t)half * tr + m) * 16;
 #pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      *(uint4*)(base + (size_t)s * cp.plane_bytes) = make_uint4(pr[s][0], pr[s][1], pr[s][2], pr[s][3]);
-      *(uint4*)(base + (size_t)(NS + s) * cp.plane_bytes) = make_uint4(pi[s][0], pi[s][1], pi[s][2], pi[s][3]);
+      for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if (lane == 0) s_e[warp] = row_exponent(__longlong_as_double((long long)m));
+    } else {
+      // rows contiguous: eight rows by 32 columns per pass of the block
+      const int r = r0 + (tid % PREP_ROWS);
+      unsigned long long m = 0;
+      if (r < rows) {
+        const int c = (which == 1 && it.bcol) ? it.bcol[r] : r;
+        for (int k = tid / PREP_ROWS; k < it.K; k += PREP_THREADS / PREP_ROWS) {
+          const double2 v = src[c + (size_t)k * ld];
+          m = max(m, max(mag_bits(v.x), mag_bits(v.y)));
+        }
+      }
+      part[tid / PREP_ROWS][tid % PREP_ROWS] = m;
+      __syncthreads();
+      if (tid < PREP_ROWS) {
+        unsigned long long v = 0;
+#pragma unroll
+        for (int j = 0; j < PREP_THREADS / PREP_ROWS; ++j) v = max(v, part[j][tid]);
+        s_e[tid] = row_exponent(__longlong_as_double((long long)v));
+      }
     }
+    __syncthreads();
+    if (tid < PREP_ROWS) ex[r0 + tid] = s_e[tid];
+    const int rt = r0 / tr, m0 = r0 % tr;
+    unsigned char* tile = out + (size_t)rt * cp.ksteps * (2 * ZNS) * cp.plane_bytes;
+    for (int idx = tid; idx < PREP_ROWS * n_grp; idx += PREP_THREADS) {
+      const int rr = idx % PREP_ROWS, grp = idx / PREP_ROWS;
+      const int r = r0 + rr, k0 = grp * ZG::KG, e = s_e[rr];
+      const int c = (r < rows && which == 1 && it.bcol) ? it.bcol[r] : r;
+      const double2* p = k_contiguous ? src + (size_t)c * ld + k0 : src + c + (size_t)k0 * ld;
+      const size_t st = k_contiguous ? 1 : ld;
+      uint32_t pr[ZNS][4], pi[ZNS][4];       // 8 BF16 per plane, two per word
+#pragma unroll
+      for (int j = 0; j < ZG::KG; j += 2) {
+        double2 v[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+          v[q] = (r < rows && k0 + j + q < it.K) ? p[(size_t)(j + q) * st] : make_double2(0.0, 0.0);
+        uint32_t a0[ZNS], a1[ZNS];
+        int_slices<ZNS>(v[0].x, e, ZBITS, a0);
+        int_slices<ZNS>(v[1].x, e, ZBITS, a1);
+#pragma unroll
+        for (int s = 0; s < ZNS; ++s) pr[s][j >> 1] = pair_bf16(a0[s], a1[s]);
+        int_slices<ZNS>(conj_op ? -v[0].y : v[0].y, e, ZBITS, a0);
+        int_slices<ZNS>(conj_op ? -v[1].y : v[1].y, e, ZBITS, a1);
+#pragma unroll
+        for (int s = 0; s < ZNS; ++s) pi[s][j >> 1] = pair_bf16(a0[s], a1[s]);
+      }
+      unsigned char* base = tile + (size_t)(grp >> 1) * (2 * ZNS) * cp.plane_bytes +
+                            ((size_t)(grp & 1) * tr + m0 + rr) * 16;
+#pragma unroll
+      for (int s = 0; s < ZNS; ++s) {
+        *(uint4*)(base + (size_t)s * cp.plane_bytes) = make_uint4(pr[s][0], pr[s][1], pr[s][2], pr[s][3]);
+        *(uint4*)(base + (size_t)(ZNS + s) * cp.plane_bytes) = make_uint4(pi[s][0], pi[s][1], pi[s][2], pi[s][3]);
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -319,25 +309,21 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_zgemm(const ZGemmItem* items,
       // epilogue of the chunk: thread = row m of the tile, 8 columns per TMEM load
       const bool first = ks0 == 0;
       for (int c0 = 0; c0 < TNB; c0 += 8) {
-        double re[8], im[8];
+        long long re[8], im[8];
+        uint32_t nonfin = 0;
         {
-          float x[8], y[8];
-          tmem_ld8(tmem + lane_base + c0, x);
-          tmem_ld8(tmem + lane_base + TNB + c0, y);
+          float x[NLEV][8], y[NLEV][8];
+#pragma unroll
+          for (int L = 0; L < NLEV; ++L) {
+            tmem_ld8_nowait(tmem + lane_base + (2 * L) * TNB + c0, x[L]);
+            tmem_ld8_nowait(tmem + lane_base + (2 * L + 1) * TNB + c0, y[L]);
+          }
+          tmem_wait_ld();
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            re[j] = (double)x[j];
-            im[j] = (double)y[j];
-          }
-#pragma unroll
-          for (int L = 1; L < NLEV; ++L) {
-            tmem_ld8(tmem + lane_base + (2 * L) * TNB + c0, x);
-            tmem_ld8(tmem + lane_base + (2 * L + 1) * TNB + c0, y);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              re[j] += (double)x[j];
-              im[j] += (double)y[j];
-            }
+            const bool f = level_sum(x[0][j], x[1][j], x[2][j], x[3][j], &re[j]) &
+                           level_sum(y[0][j], y[1][j], y[2][j], y[3][j], &im[j]);
+            if (!f) nonfin |= 1u << j;
           }
         }
         if (m < it.M) {
@@ -346,14 +332,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_zgemm(const ZGemmItem* items,
             const int n = ct * TNB + c0 + j;
             if (n >= it.N) continue;
             const int e = e_m + col_exp[c0 + j];
-            double2 v = make_double2(ldexp(re[j], e), ldexp(im[j], e));
-            if (it.acc < 0) v = make_double2(-v.x, -v.y);
+            double2 v = make_double2(fixed_to_double(it.acc < 0 ? -re[j] : re[j], e),
+                                     fixed_to_double(it.acc < 0 ? -im[j] : im[j], e));
+            if (nonfin >> j & 1u) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
             double2* cp = it.C + m + (size_t)n * it.ldc;
             if (!first || it.acc < 0) {
               const double2 o = *cp;
               v = make_double2(o.x + v.x, o.y + v.y);
             }
-            bad |= !(isfinite(v.x) && isfinite(v.y));
+            bad |= mag_bits(v.x) != ((unsigned long long)__double_as_longlong(v.x) & 0x7fffffffffffffffull) ||
+                   mag_bits(v.y) != ((unsigned long long)__double_as_longlong(v.y) & 0x7fffffffffffffffull);
             *cp = v;
           }
         }
@@ -387,20 +375,16 @@ bool g_zattr_done[ZMAX_DEV] = {};
 
 void launch_zgemm_pack_a(const ZGemmItem* items, int n_items, int m_cap_max, int* status, cudaStream_t st) {
   if (n_items <= 0) return;
-  const int bx_a = std::min(1024, cdiv(std::max(1, m_cap_max), 4));     // four rows per block when a warp takes a row
-  k_zg_rowexp<<<dim3(bx_a, n_items), 128, 0, st>>>(items, n_items, -1);
-  k_zg_pack<<<dim3(128, n_items), 256, 0, st>>>(items, n_items, -1, status);
+  const int n_a = std::min(2048, cdiv(cdiv(std::max(1, m_cap_max), TMA) * TMA, PREP_ROWS));
+  k_zg_prep<<<dim3(n_a, n_items), PREP_THREADS, 0, st>>>(items, n_items, n_a, 1, status);
 }
 
 void launch_zgemm(const ZGemmItem* items, int n_items, int tile_cap, int m_cap_max, int n_cap_max, int* status,
                   cudaStream_t st) {
   if (n_items <= 0) return;
-  // four rows per block when a warp takes a row (rows contiguous in K), else 128
-  const int bx_a = std::min(1024, cdiv(std::max(1, m_cap_max), 4)), bx_b = std::min(1024, cdiv(std::max(1, n_cap_max), 4));
-  k_zg_rowexp<<<dim3(bx_a, n_items), 128, 0, st>>>(items, n_items, 0);
-  k_zg_rowexp<<<dim3(bx_b, n_items), 128, 0, st>>>(items, n_items, 1);
-  k_zg_pack<<<dim3(128, n_items), 256, 0, st>>>(items, n_items, 0, status);
-  k_zg_pack<<<dim3(64, n_items), 256, 0, st>>>(items, n_items, 1, status);
+  const int n_a = std::min(2048, cdiv(cdiv(std::max(1, m_cap_max), TMA) * TMA, PREP_ROWS));
+  const int n_b = std::min(2048, cdiv(cdiv(std::max(1, n_cap_max), TNB) * TNB, PREP_ROWS));
+  k_zg_prep<<<dim3(n_a + n_b, n_items), PREP_THREADS, 0, st>>>(items, n_items, n_a, 0, status);
   const size_t smem = (size_t)Stages<ZNS>::value * 2 * ZNS * (TMA + TNB) * ROW_BYTES + 1024;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);

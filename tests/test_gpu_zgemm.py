@@ -91,3 +91,35 @@ def test_sliced_zgemm_rejects_bad_arguments(capi):
     with pytest.raises(capi.PTError) as ei:
         capi.zgemm_sliced("N", "N", A, A, A, 4, 4, 0, scratch)
     assert ei.value.code == -1
+
+
+@pytest.mark.parametrize("m,n,k,opA,opB", [(7, 9, 15, "N", "N"), (8, 64, 16, "T", "N"), (129, 65, 33, "N", "T"),
+                                           (5, 3, 513, "H", "H")])
+def test_operand_preparation_edges(capi, m, n, k, opA, opB):
+    """Remainders of the preparation's 8-row blocks and 8-element K groups, entries over the whole exponent
+    range (subnormal rows included), and a NaN and an infinity: they make their row (column) of the product NaN
+    and leave the others as they are. Bound as above: 2^-40 K max|row| max|column| per entry."""
+    import torch
+    rng = np.random.default_rng(m + 31 * n + k)
+    OA = rng.standard_normal((1, m, k)) + 1j * rng.standard_normal((1, m, k))
+    OB = rng.standard_normal((1, k, n)) + 1j * rng.standard_normal((1, k, n))
+    OA[0, 0] *= 1e-300
+    OA[0, 1] *= 1e-320                 # subnormal
+    OB[0, :, 0] *= 1e150
+    OA[0, m - 1, k // 2] = complex(np.nan, 1.0)
+    OB[0, k - 1, n - 1] = complex(0.0, np.inf)
+    store = {"N": lambda X: X, "T": lambda X: X.transpose(0, 2, 1), "H": lambda X: X.conj().transpose(0, 2, 1)}
+    At, Bt = _colmajor(torch, store[opA](OA)), _colmajor(torch, store[opB](OB))
+    Ct = torch.zeros((1, n, m), dtype=torch.complex128, device="cuda")
+    scratch = torch.empty(capi.zgemm_scratch_bytes(m, n, k, 1), dtype=torch.uint8, device="cuda")
+    capi.zgemm_sliced(opA, opB, At, Bt, Ct, m, n, k, scratch)
+    C = Ct.cpu().numpy()[0].T
+    assert not np.isfinite(C[m - 1]).any() and not np.isfinite(C[:, n - 1]).any()
+    A, B = OA[0, :m - 1], OB[0, :, :n - 1]
+    up = np.array([600] + [1000] + [0] * (m - 3))[:, None]         # the reference in the normal range, scaled exactly
+    sc = lambda X, e: np.ldexp(X.real, e) + 1j * np.ldexp(X.imag, e)
+    ref = sc(sc(A, up) @ B, -up)
+    scale = k * np.maximum(np.abs(A.real), np.abs(A.imag)).max(1)[:, None] * \
+        np.maximum(np.abs(B.real), np.abs(B.imag)).max(0)[None, :]
+    # 4e-323: results that are themselves subnormal are rounded to multiples of 5e-324
+    assert np.all(np.abs(C[:m - 1, :n - 1] - ref) <= 2.0 ** -40 * scale + 4e-323)
