@@ -25,10 +25,6 @@ __global__ void k_truncate(Tables T, const BondWork* work, int n_work, int chi_m
                            double mtol, int rsvd = 0);
 __global__ void k_recover(Tables T, const BondWork* work, int n_work);
 __global__ void k_caps(Tables T, int n_mpos);
-__global__ void k_observe_m(Tables T, int n_chains, double2* Mbuf, const size_t* moff);
-__global__ void k_observe(Tables T, int n_chains, const double2* ops, int n_ops, int n_max,
-                          double2* obs, double2* trace, double2* Lbuf, double2* Rbuf, int ld,
-                          int use_history, const double2* Mbuf, const size_t* moff);
 __global__ void k_step_inc(int* step);
 __global__ void k_svd_load(const double2* A, int m, int n, int batch, double2* work_A,
                            size_t strideA);
@@ -165,6 +161,12 @@ void launch_rsvd_vectors(const Tables& T, const BondWork* work, int n_work, cons
 
 // set the message returned by pt_tebd_last_error(NULL) (engine.cu)
 void set_global_error(const char* msg);
+
+// readout (readout.cu): Tr(O_j rho) of every site and operator and the trace of every chain at the current
+// step; Mbuf holds 5 planes [chi_l][chi_r] per site at moff, Lbuf / Rbuf n_max + 1 vectors of ld per chain
+void launch_observe(const Tables& T, int n_chains, int n_max, int gx_m, const double2* ops, int n_ops, double2* obs,
+                    double2* trace, double2* Lbuf, double2* Rbuf, int ld, int use_history, double2* Mbuf,
+                    const size_t* moff, cudaStream_t st);
 
 // local super-operator launch (struct passed by value lives in the kernel TU)
 void launch_apply_local(const Tables& T, int site, int lam, const double2* s16, cudaStream_t st);
