@@ -115,8 +115,6 @@ struct pt_tebd {
   double2* d_omega = nullptr;         // the range finder's sketch matrix (ld_omega x l_max)
   int ld_omega = 1;
   unsigned* d_sync3 = nullptr;        // grid barrier state
-  int* d_cnt_odd = nullptr;           // per-item rotation counters
-  int* d_cnt_even = nullptr;
   SiteWork* d_sites = nullptr;
   int n_site_work = 0;
   int gx_site = 1;
@@ -285,7 +283,6 @@ void enqueue_layer(pt_tebd* h, const BondWork* work, int n, int layer) {
     ptk::launch_tc_theta(h->T, work, n, work == h->d_odd ? h->tiles_odd : h->tiles_even, (int)h->opt.precision, s);
   ptk::k_nan_guard<<<(n + 127) / 128, 128, 0, s>>>(h->T, work, n);
   ev_end(h, e);
-  int* cnt = work == h->d_odd ? h->d_cnt_odd : h->d_cnt_even;
   if (h->use_rsvd) {
     // fast path: randomized truncated SVD (tensor-core products, whole-GPU QR and l x l Jacobi)
     const ptk::RsvdLists& L = work == h->d_odd ? h->rs_odd : h->rs_even;
@@ -323,9 +320,14 @@ void enqueue_layer(pt_tebd* h, const BondWork* work, int n, int layer) {
     ev_end(h, e);
     qr(L.qb);                                           // Z = Qb Rb
     ev_begin(h, 3, &e);
-    const double tol_scale = 9.007199254740992e6;     // |cos| <= 1e-9, below the products' accuracy
-    ptk::launch_jacobi_grid(work, n, h->grid_blocks, h->opt.max_sweeps, h->d_sync3, cnt, h->T.status, s, 1, 1,
-                            1.1102230246251565e-16, 3, /*on_b=*/2, /*with_v=*/1, tol_scale);
+    // |cos| <= 2^-43: the right factor is formed from the left one (Ur = R Wr / S), so what is left unrotated enters
+    // D to first order (with 1e-9, enough where both factors are accumulated, the observables were 1e-9 off)
+    const double tol_scale = 1024.0;
+    // columns below 2^-42 ||R||, the noise of the sliced products, are left as they are: at most eps / 1024, so
+    // the truncation always discards them (their orthogonality among themselves does not matter)
+    const double floor = std::max(1.1102230246251565e-16, std::min(2.2737367544323206e-13, h->opt.eps / 1024.0));
+    ptk::launch_jacobi_grid(work, n, h->grid_blocks, lc, h->opt.max_sweeps, h->d_sync3, h->T.status, s, /*on_b=*/2,
+                            /*with_v=*/0, tol_scale, floor * floor);
     ev_end(h, e);
     ev_begin(h, 4, &e);
     // the fast path's singular values carry errors of ~1e-11 of sigma_max: gaps below the
@@ -338,7 +340,7 @@ void enqueue_layer(pt_tebd* h, const BondWork* work, int n, int layer) {
     ev_end(h, e);
   } else if (h->grid_blocks > 0) {
     // QR-preconditioned FP64 Jacobi: pivoted QR, Jacobi on R^H, then V_D = P U', U_D = D V_D / sigma
-    const int kc = work == h->d_odd ? h->kcap_odd : h->kcap_even, mc = work == h->d_odd ? h->mcap_odd : h->mcap_even;
+    const int kc = work == h->d_odd ? h->kcap_odd : h->kcap_even;
     ev_begin(h, 8, &e);
     enqueue_qr(h, work, n, rt.qr, INT_MAX);
     ev_end(h, e);
@@ -347,8 +349,8 @@ void enqueue_layer(pt_tebd* h, const BondWork* work, int n, int layer) {
     // ~1e-12 of its scale, stops its sweeps at |cos| <= 1e-9 (the last, refining sweeps of the
     // quadratic convergence are below its own accuracy)
     const double tol_scale = h->opt.precision == PT_BF16_OZAKI ? 9.007199254740992e6 /* 1e-9 / u */ : 0.0;
-    ptk::launch_jacobi_grid(work, n, h->grid_blocks, h->opt.max_sweeps, h->d_sync3, cnt, h->T.status, s, 1, 1,
-                            1.1102230246251565e-16, 3, /*on_b=*/1, /*with_v=*/0, tol_scale);
+    ptk::launch_jacobi_grid(work, n, h->grid_blocks, kc, h->opt.max_sweeps, h->d_sync3, h->T.status, s, /*on_b=*/1,
+                            /*with_v=*/0, tol_scale);
     ev_end(h, e);
   } else {
     // no co-resident whole-GPU launch possible on this device: one thread-block cluster per matrix
@@ -1141,9 +1143,7 @@ int build(pt_tebd* h) {
     h->use_rsvd = ok;
   }
   h->d_sync3 = (unsigned*)h->dalloc(sizeof(unsigned) * 4);
-  h->d_cnt_odd = (int*)h->dalloc(sizeof(int) * 2 * std::max(1, h->n_odd));
-  h->d_cnt_even = (int*)h->dalloc(sizeof(int) * 2 * std::max(1, h->n_even));
-  if (!h->d_sync3 || !h->d_cnt_odd || !h->d_cnt_even) return h->fail(PT_ERR_OOM, "Jacobi barrier state");
+  if (!h->d_sync3) return h->fail(PT_ERR_OOM, "Jacobi barrier state");
   cudaMemsetAsync(h->d_sync3, 0, sizeof(unsigned) * 4, h->stream);
   h->d_odd = odd.empty() ? nullptr : upload(h, odd);
   h->d_even = even.empty() ? nullptr : upload(h, even);
@@ -1656,7 +1656,7 @@ static size_t svd_layout(int m, int n, int batch, size_t* offs) {
   offs[2] = take(sizeof(double) * (size_t)Na * batch);        // sig
   offs[3] = take(sizeof(int) * (size_t)Na * batch);           // perm
   offs[4] = take(sizeof(int) * 8 * (size_t)batch);            // info
-  offs[5] = take(sizeof(int));                                // status
+  offs[5] = take(sizeof(int));                                // status, and the barrier's words at + 8 ints
   offs[6] = take(sizeof(BondWork) * (size_t)batch);           // work items
   offs[7] = take(sizeof(double) * (size_t)Na * batch);        // column norms
   return o;
@@ -1860,8 +1860,7 @@ int pt_svd_f64(const double* A, int m, int n, int batch, double* sigma, double* 
   cudaMemsetAsync(status, 0, sizeof(int), st);
   const int gx = (int)std::min<size_t>(256, ((size_t)m * n + 255) / 256);
   ptk::k_svd_load<<<dim3(gx, batch), 256, 0, st>>>((const double2*)A, m, n, batch, wA, sA);
-  const int cl = ptk::jacobi_cluster_size(std::max(1, std::min(16, (Na / 2 + 7) / 8)));
-  ptk::launch_jacobi_cluster(items, batch, cl, max_sweeps, status, st);
+  ptk::launch_svd_jacobi(items, batch, Ma, Na, max_sweeps, status, (unsigned*)(status + 8), st);
   const int gs = (int)std::min<size_t>(256, ((size_t)(m + n + 1) * Na + 255) / 256);
   ptk::k_svd_store<<<dim3(gs, batch), 256, 0, st>>>(wA, wV, sig, perm, m, n, batch, sA, sV, sigma,
                                                     (double2*)U, (double2*)V);

@@ -13,17 +13,23 @@ struct GridSync {
 };
 
 // Returns false when aborted (timeout here or elsewhere). The arrival counter only grows:
-// barrier k of the launch is complete once it reaches k * gridDim.x, so one atomic per CTA and
+// barrier k of the launch is complete once it reaches k * nblk, so one atomic per CTA and
 // polling of the same word suffice. The abort flag and the time limit are checked every 64 polls;
-// on expiry the CTA records ST_TIMEOUT and raises the abort flag.
-__device__ __forceinline__ bool grid_barrier(const GridSync& gs, int* status) {
+// on expiry the CTA records ST_TIMEOUT and raises the abort flag. nblk: the CTAs that take part (0: all of them).
+__device__ __forceinline__ bool grid_barrier(const GridSync& gs, int* status, unsigned nblk = 0) {
   __shared__ int ok_s;
+  if (nblk == 0) nblk = gridDim.x;
+  if (nblk == 1) {
+    __threadfence();
+    __syncthreads();
+    return true;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     int ok = 1;
     __threadfence();
     const unsigned old = atomicAdd(gs.count, 1u);
-    const unsigned target = (old / gridDim.x + 1u) * gridDim.x;
+    const unsigned target = (old / nblk + 1u) * nblk;
     volatile unsigned* vc = gs.count;
     const long long t0 = clock64();
     for (int it = 1;; ++it) {

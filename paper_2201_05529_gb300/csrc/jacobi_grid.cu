@@ -1,20 +1,39 @@
 // Whole-GPU one-sided Jacobi SVD for all bond matrices of one layer (App. A.2).
 //
-// The SVD is bound by FP64 arithmetic (1.2 TFLOP/s on GB300, ~7.9 GFLOP/s per SM), so every SM
-// must work on it even when a layer has only two bonds. One cooperative launch (one 512-thread
-// CTA per SM) processes every matrix of the layer. The columns are grouped in blocks of two and a
-// round-robin tournament runs over the blocks: in each round the block pairs of all matrices form
-// one task list, each task handled by a slot of 8 warps (two groups of 4, one warp per SM
-// sub-partition in each, the rows split across them) that runs the task's four cross pairs (and,
-// in the first round of a sweep, the pair inside each block) in sub-rounds; a grid barrier
-// separates the rounds. Partial sums are combined in a fixed order, so results are bitwise
-// reproducible. Every barrier wait has a time limit: on expiry the kernel records ST_TIMEOUT,
-// raises an abort flag that releases every other CTA, and returns.
+// What bounds it: GB300 issues one FP64 instruction per warp every 64 cycles and sub-partition, whatever the
+// number of active lanes (measured; 19 cycles per SM with all four busy), with a latency of 64 cycles, and a
+// grid barrier costs ~2400 cycles. A rotation's scalars (one lane's chain of ~30 FP64 operations) and the
+// barriers therefore cost as much as the arithmetic on columns of a few hundred rows. So:
+//   * the columns are grouped in blocks of b and a round-robin tournament runs over the blocks: one CTA holds
+//     a pair of blocks (2 b columns) in shared memory and runs its b x b cross pairs (in the first round of a
+//     sweep also the pairs inside the blocks) in sub-rounds of b disjoint pairs, so a sweep of n columns
+//     has n / b - 1 grid barriers;
+//   * the scalars of a sub-round's pairs are computed by the lanes of one extra warp at the same time. Columns
+//     carry a real scale (column = d x stored column, q = d^2), so that neither a square root nor a division is
+//     needed: with rho = tan / |gamma| (in FP32 and integers: a rotation by an angle that is 1e-7 off is still
+//     unitary and leaves 1e-7 of the pair's inner product to the next sweep) the stored columns become
+//     x - conj(mu) y and y + nu x, mu = rho q_y g, nu = rho q_x g, g = x^H y of the stored columns, and
+//     q_x, q_y are multiplied by cos^2 = 1 / (1 + tan^2). That is 9 FP64 operations before the columns can be
+//     rotated; the new norms and scales are formed while they are. A row costs 8 FP64 operations, not 12;
+//   * a CTA has two such task slots of 8 + 1 warps (named barriers), so one's scalars overlap the other's
+//     columns; tasks fill one slot of every SM before the second;
+//   * b is chosen on the device from the live dims by a cost model of these terms (choose_block), and CTAs that
+//     no round can use leave at once, so small layers pay for small barriers.
+// Before (one 512-thread CTA per SM, b = 2, columns in L2, each pair's scalars on one lane in FP64 with two sqrt /
+// rsqrt chains, 5800 cycles; now 1900), start of the calls that run it: two 256 x 256 SVDs 113 ms (clusters) -> 33,
+// the five-site chain's first eight steps 227 -> 189 ms, 16 chains' first four steps 309 -> 196 ms, the 21-site
+// chain's first four steps on the tensor-core path 905 -> 651 ms.
 //
-// on_b = 1: the matrix is R^H left by the pivoted QR (qrcp.cu); only its left vectors are wanted
-// there, so the right factor is not accumulated. on_b = 2: the l x l triangular factor of the fast
-// path's randomized range finder (rsvd.cu), both factors wanted.
-#include <climits>
+// Sums are combined in a fixed order, so results are bitwise reproducible. Every barrier wait has a time
+// limit: on expiry the kernel records ST_TIMEOUT, raises an abort flag that releases every other CTA, and
+// returns.
+//
+// on_b = 1: the matrix is R^H left by the pivoted QR (qrcp.cu); only its left vectors are wanted there, so
+// the right factor is not accumulated. on_b = 2: R^H of the l x l triangular factor R in G64 of the fast path's
+// randomized range finder (rsvd.cu), formed in V: its columns (R's rows) are graded and close to orthogonal, so ~40%
+// fewer pairs rotate than on R (CPU emulation, bonds of a nine-site chain), and the other factor follows from R and
+// the left vectors. on_b = 0: the matrix in A (the standalone SVD).
+#include <algorithm>
 
 #include "grid_sync.cuh"
 #include "kernels.h"
@@ -23,31 +42,29 @@ namespace ptk {
 
 namespace {
 
-constexpr int GRID_THREADS = 512;
-constexpr int GROUP_WARPS = 4;
-constexpr int GROUPS = GRID_THREADS / 32 / GROUP_WARPS;    // 4 pairs per CTA at a time (2 task slots)
+constexpr int JG = 2;                      // task slots per CTA
+constexpr int JW = 8;                      // column warps of a slot: JW / b per pair
+constexpr int JT = 32 * (JW + 1);          // threads of a slot: the last warp computes the scalars
+constexpr int CT = JG * JT, CW = CT / 32;  // threads and warps per CTA
+constexpr int JB = 8;                      // largest block
 constexpr int MAX_ITEMS = 1024;
+constexpr double UNIT = 1.1102230246251565e-16;
 
-template <typename R>
-__device__ __forceinline__ R wsumd(R v) {
+__device__ __forceinline__ double wsum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-template <typename R> struct Cx;
-// A: the matrix on D's shape; B: the matrix B = R^H of the pivoted QR (on_b); V: the right factor
-// (the sweeps are written for a real type R; the path instantiates them in FP64)
-template <> struct Cx<double> {
-  using T = double2;
-  static constexpr double EPS = 1.1102230246251565e-16;
-  __device__ static T* A(const BondWork& W) { return W.A; }
-  __device__ static T* B(const BondWork& W) { return W.G64; }
-  __device__ static T* V(const BondWork& W) { return W.V; }
-};
-
-__device__ __forceinline__ void named_sync(int id, int nthreads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+// Sum over the 32 lanes of two values at once (a reduce-scatter butterfly): lane 0 ends with the
+// total of a, lane 16 with the total of b; 5 shuffles and 5 adds instead of 10 and 10.
+__device__ __forceinline__ double wsum2(double a, double b, int lane) {
+  const bool hi = (lane & 16) != 0;
+  double keep = hi ? b : a;
+  keep += __shfl_xor_sync(0xffffffffu, hi ? a : b, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) keep += __shfl_xor_sync(0xffffffffu, keep, o);
+  return keep;
 }
 
 __device__ __forceinline__ void item_shape(const BondWork& W, int* Ma, int* Na) {
@@ -57,454 +74,627 @@ __device__ __forceinline__ void item_shape(const BondWork& W, int* Ma, int* Na) 
   *Na = (mD > 0 && nD > 0) ? (tr ? mD : nD) : 0;
 }
 
+__device__ __forceinline__ void slot_sync(int grp) {
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "r"(JT) : "memory");
+}
+
+__device__ __forceinline__ double2* mat_of(const BondWork& W, int on_b) {
+  return on_b == 0 ? W.A : (on_b == 1 ? W.G64 : W.V);
+}
+
+__device__ __forceinline__ void cp16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+// the first 24 bits of a positive double's significand as a float in [1, 2), and its exponent
+__device__ __forceinline__ float significand(double x, int* e) {
+  const int hi = __double2hiint(x);
+  *e = ((hi >> 20) & 0x7ff) - 1023;
+  return __int_as_float(0x3f800000 | (hi & 0xfffff) << 3 | (int)((unsigned)__double2loint(x) >> 29));
+}
+
+// f 2^k, f in [1, 2), 0 for k below -60 (k <= 1)
+__device__ __forceinline__ float scale_pow2(float f, int k) {
+  return k < -60 ? 0.f : __int_as_float(__float_as_int(f) + (k << 23));
+}
+
+constexpr int MIN_SCALE_HI = (1023 - 64) << 20;    // below 2^-64 a squared scale is multiplied into its column
+
+// columns per block: the b in {1, 2, 4, 8} that fits cols_max columns and whose sweep is shortest by the cost of
+// its terms in cycles: per sub-round the scalars and reductions (2500 cycles, shared by the tasks of an SM) and 19
+// cycles per FP64 warp instruction of the SM's tasks; per round the transfer of a task's columns and the barrier.
+// Costs estimated from the measured FP64 issue rate and barrier; the choice only moves a few percent around them.
+// One warp computes it; every lane gets the result.
+__device__ int choose_block(const int* s_Na, const int* s_Ma, int n_work, int slots, int sms, int cols_max,
+                            bool with_v, int lane) {
+  int best = 1;
+  float best_t = 3e38f;
+  for (int b = 1; b <= JB && 2 * b <= cols_max; b <<= 1) {
+    int tasks = 0, rounds = 0, rows = 0;
+    for (int w = lane; w < n_work; w += 32) {
+      if (s_Na[w] < 2) continue;
+      const int nb = (s_Na[w] + b - 1) / b, nbp = nb + (nb & 1);
+      tasks += nbp / 2;
+      rounds = max(rounds, nbp - 1);
+      // FP64 operations per pair: 4 per row for the inner product, 8 per row (and row of V) for the rotation
+      rows = max(rows, 12 * s_Ma[w] + (with_v ? 8 * s_Na[w] : 0));
+    }
+    tasks = __reduce_add_sync(0xffffffffu, tasks);
+    rounds = __reduce_max_sync(0xffffffffu, rounds);
+    rows = __reduce_max_sync(0xffffffffu, rows);
+    if (tasks == 0) return 1;
+    const float per_sm = (float)((tasks + sms - 1) / sms), waves = (float)((tasks + slots - 1) / slots);
+    const float fp = 19.f * b * (float)((rows + 31) / 32);
+    const float sub = fmaxf(waves * 2500.f + fp, per_sm * fp + 1500.f);
+    const float move = 1000.f + per_sm * b * (float)rows * 0.1f;
+    const float t = rounds * ((float)b * sub + move + (tasks > 1 ? 2500.f : 0.f)) + (b - 1) * sub;
+    if (t < best_t) {
+      best_t = t;
+      best = b;
+    }
+  }
+  return best;
+}
+
 }  // namespace
 
-// Sum over the 32 lanes of two values at once (a reduce-scatter butterfly): lane 0 ends with the
-// total of a, lane 16 with the total of b; 5 shuffles and 5 adds instead of 10 and 10.
-template <typename R>
-__device__ __forceinline__ R wsum2(R a, R b, int lane) {
-  const bool hi = (lane & 16) != 0;
-  R keep = hi ? b : a;
-  keep += __shfl_xor_sync(0xffffffffu, hi ? a : b, 16);
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) keep += __shfl_xor_sync(0xffffffffu, keep, o);
-  return keep;
-}
-
-// One column pair (i, j) of matrix w, processed by the 4 warps of group grp (rows split across
-// them). nrm holds the squared column norms: they are read here and, when the pair rotates,
-// updated by the rotation's closed form (or recomputed from the columns where that form cancels),
-// so the dot phase only forms gamma = a_i^H a_j.
-// Counts a rotation in cnt. Every warp of the group must call it.
-template <typename R>
-__device__ __forceinline__ void process_pair(typename Cx<R>::T* A, typename Cx<R>::T* V, double* nrm, int Ma,
-                                             int Na, int i, int j, double fro, double floor_eps, int grp, int gw,
-                                             int lane, R (*s_part)[GROUP_WARPS][4], R (*s_rot)[8], int* cnt_slot,
-                                             bool with_v, int* stamp, int g_round, int skip_before, R tol) {
-  using C2 = typename Cx<R>::T;
-  const R eps = Cx<R>::EPS;
-  if (i > j) { const int tt = i; i = j; j = tt; }
-  const bool real_pair = j < Na;        // uniform within the group
-  if (!real_pair) return;
-  const bool leader = gw == 0 && lane == 0;
-  R al = 0, be = 0;
-  if (leader) {
-    al = (R)__ldcg(nrm + i);
-    be = (R)__ldcg(nrm + j);
-  }
-  C2* ai = A + (size_t)i * Ma;
-  C2* aj = A + (size_t)j * Ma;
-  C2* vi = V + (size_t)i * Na;
-  C2* vj = V + (size_t)j * Na;
-  const int r0 = gw * 32 + lane;
-  // the first RC rows of each lane stay in registers for the rotation (all of them when
-  // Ma <= RC * 128); the rest, if any, are read again
-  constexpr int RC = 2, STEP = 32 * GROUP_WARPS;
-  C2 xs[RC], ys[RC];
-  const int si = __ldcg(stamp + i), sj = __ldcg(stamp + j);
-  {
-    R gr = 0, gi = 0;
-#pragma unroll
-    for (int k = 0; k < RC; ++k) {
-      const int r = r0 + k * STEP;
-      if (r < Ma) {
-        xs[k] = __ldcg(ai + r);
-        ys[k] = __ldcg(aj + r);
-        gr = fma(xs[k].x, ys[k].x, fma(xs[k].y, ys[k].y, gr));
-        gi = fma(xs[k].x, ys[k].y, fma(-xs[k].y, ys[k].x, gi));
-      }
-    }
-    for (int r = r0 + RC * STEP; r < Ma; r += STEP) {
-      const C2 x = __ldcg(ai + r), y = __ldcg(aj + r);
-      gr = fma(x.x, y.x, fma(x.y, y.y, gr));
-      gi = fma(x.x, y.y, fma(-x.y, y.x, gi));
-    }
-    // unchanged pair: neither column has rotated since this pair was checked one sweep ago (and
-    // found orthogonal, or it would carry that round's stamp), so gamma would come out the same
-    if (max(si, sj) < skip_before) return;       // uniform: every lane read the same stamps
-    const R part = wsum2(gr, gi, lane);
-    if (lane == 0) s_part[grp][gw][0] = part;
-    if (lane == 16) s_part[grp][gw][1] = part;
-  }
-  named_sync(1 + grp, 32 * GROUP_WARPS);
-  // one lane turns the partial sums (fixed order) into the rotation and shares it
-  if (leader) {
-    R flag = 0, c = 1, sv = 0, ser = 0, sei = 0, cer = 1, cei = 0;
-    R gr = 0, gi = 0;
-#pragma unroll
-    for (int k = 0; k < GROUP_WARPS; ++k) {
-      gr += s_part[grp][k][0];
-      gi += s_part[grp][k][1];
-    }
-    const R g2 = gr * gr + gi * gi;
-    const R fl2 = (R)(floor_eps * floor_eps * fro);
-    // rotate unless |gamma| <= tol sqrt(alpha beta), or a column is at the noise floor
-    // (|a|^2 <= floor_eps^2 ||A||_F^2: such columns cannot become orthogonal relative to
-    // their own norm and carry no information at this precision)
-    if (g2 > tol * tol * al * be && g2 > R(0) && fmin(al, be) > fl2) {
-      // smaller root of the rotation equation: with q = sqrt(h^2 + 4 g^2) and w = q + |h|,
-      // |s| / g = sqrt(2 / (q w)), c = w |s| / (2 g) and t g = 2 g^2 sign(h) / w (two dependent
-      // long operations instead of four)
-      const R ig = rsqrt(g2), h = be - al, ah = fabs(h);          // ig = 1 / |gamma|
-      const R q = sqrt(h * h + R(4) * g2), wq = q + ah;
-      const R sgm = rsqrt(R(0.5) * q * wq);
-      const R sgn = h >= R(0) ? R(1) : R(-1);
-      const R sg = sgn * sgm;                                     // s / |gamma|
-      c = R(0.5) * wq * sgm;
-      sv = sg * g2 * ig;
-      ser = sg * gr;                        // s e^{-i phi}: e = conj(gamma) / |gamma|
-      sei = -sg * gi;
-      const R cg_ = c * ig;
-      cer = cg_ * gr;
-      cei = -cg_ * gi;
-      __stcg(stamp + i, g_round);
-      __stcg(stamp + j, g_round);
-      const R tg = sgn * g2 * sgm * sgm * q, al2 = al - tg, be2 = be + tg;
-      if (al2 >= R(0.25) * al && be2 >= R(0.25) * be) {
-        flag = 1;
-        __stcg(nrm + i, (double)al2);
-        __stcg(nrm + j, (double)be2);
-        atomicAdd(cnt_slot, 1);
-      } else {
-        flag = 2;
-      }
-    }
-    s_rot[grp][0] = flag;
-    s_rot[grp][1] = c;
-    s_rot[grp][2] = sv;
-    s_rot[grp][3] = ser;
-    s_rot[grp][4] = sei;
-    s_rot[grp][5] = cer;
-    s_rot[grp][6] = cei;
-  }
-  named_sync(1 + grp, 32 * GROUP_WARPS);
-  if (s_rot[grp][0] == R(0)) return;
-  const R c = s_rot[grp][1], s = s_rot[grp][2], ser = s_rot[grp][3], sei = s_rot[grp][4];
-  const R cer = s_rot[grp][5], cei = s_rot[grp][6];
-  const bool renorm = s_rot[grp][0] == R(2);
-  R na = 0, nb = 0;
-  auto rotate = [&](int r, C2 x, C2 y) {
-    C2 nx, ny;
-    nx.x = c * x.x - (ser * y.x - sei * y.y);
-    nx.y = c * x.y - (ser * y.y + sei * y.x);
-    ny.x = s * x.x + (cer * y.x - cei * y.y);
-    ny.y = s * x.y + (cer * y.y + cei * y.x);
-    __stcg(ai + r, nx);
-    __stcg(aj + r, ny);
-    if (renorm) {
-      na = fma(nx.x, nx.x, fma(nx.y, nx.y, na));
-      nb = fma(ny.x, ny.x, fma(ny.y, ny.y, nb));
-    }
+// One-sided Jacobi over all matrices of a layer in FP64. with_v: accumulate the right factor V from V = I.
+// tol_scale: a pair rotates while |a_i^H a_j| > tol_scale * unit roundoff * |a_i| |a_j| (0: the row count m).
+// Columns whose squared norm is at floor2 ||A||_F^2 or below are not rotated: they cannot become orthogonal
+// relative to their own norm and carry no information at that precision. Squared column norms live in aux, squared
+// scales in sig, rotation counters in info[4..5], sweeps go to info[3]. SM: the columns fit in shared memory (cols_max
+// of them); otherwise a pair's columns are read from and written to L2 (b = 1).
+template <bool SM>
+__global__ void __launch_bounds__(CT, 1)
+    k_jacobi_grid(const BondWork* work, int n_work, int max_sweeps, GridSync gs, int* status, int on_b, int with_v,
+                  double tol_scale, double floor2, int n_grp, int dyn_bytes) {
+  extern __shared__ __align__(16) unsigned char s_raw[];
+  // of one task slot
+  struct Slot {
+    double part[JW][2];
+    double rot[JB][4];                     // mu, nu of each pair
+    double nrm[2 * JB], q[2 * JB];         // squared norms and squared scales of the task's columns
+    int flag[JB];                          // rotate
+    int redo[JB];                          // recompute the pair's norms from its columns
+    int rotc[2 * JB];                      // the column changed in this task
+    int cnt, renorm[2];
   };
-#pragma unroll
-  for (int k = 0; k < RC; ++k) {
-    const int r = r0 + k * STEP;
-    if (r < Ma) rotate(r, xs[k], ys[k]);
-  }
-  for (int r = r0 + RC * STEP; r < Ma; r += STEP) rotate(r, __ldcg(ai + r), __ldcg(aj + r));
-  for (int r = r0; with_v && r < Na; r += 32 * GROUP_WARPS) {
-    const C2 x = __ldcg(vi + r), y = __ldcg(vj + r);
-    C2 nx, ny;
-    nx.x = c * x.x - (ser * y.x - sei * y.y);
-    nx.y = c * x.y - (ser * y.y + sei * y.x);
-    ny.x = s * x.x + (cer * y.x - cei * y.y);
-    ny.y = s * x.y + (cer * y.y + cei * y.x);
-    __stcg(vi + r, nx);
-    __stcg(vj + r, ny);
-  }
-  if (!renorm) return;
-  // the rotated columns' norms, recomputed
-  const R part = wsum2(na, nb, lane);
-  if (lane == 0) s_part[grp][gw][2] = part;
-  if (lane == 16) s_part[grp][gw][3] = part;
-  named_sync(1 + grp, 32 * GROUP_WARPS);
-  if (leader) {
-    R sa = 0, sb = 0;
-#pragma unroll
-    for (int k = 0; k < GROUP_WARPS; ++k) {
-      sa += s_part[grp][k][2];
-      sb += s_part[grp][k][3];
-    }
-    __stcg(nrm + i, (double)sa);
-    __stcg(nrm + j, (double)sb);
-    atomicAdd(cnt_slot, 1);
-  }
-}
-
-// One-sided Jacobi over all matrices of a layer in FP64: on W.A (or on B = R^H in G64) with V in
-// W.V. on_b = 1: the matrix
-// is the pivoted QR's B = R^H, Na rows and info[8] columns; on_b = 2: the l x l factor in G64,
-// l = info[9]. with_v: accumulate the right factor V
-// (from V = I when init_v). finalize: write sigma, the normalised left vectors and the order.
-// floor_eps: unit roundoff that sets the noise floor; tol_scale: a pair rotates while
-// |a_i^H a_j| > tol_scale * unit roundoff * |a_i| |a_j| (0: the row count m; < 0: 4 sqrt(m), the
-// resolution of the dot products themselves, for the FP32 sweeps).
-// cnt: [n_work][2] rotation counters; sweeps go to info[sweep_slot].
-template <typename R>
-__global__ void __launch_bounds__(GRID_THREADS)
-    k_jacobi_grid(const BondWork* work, int n_work, int max_sweeps, GridSync gs, int* cnt, int* status,
-                  int init_v, int finalize, double floor_eps, int sweep_slot, int on_b, int with_v,
-                  double tol_scale) {
-  using C2 = typename Cx<R>::T;
-  __shared__ int s_Na[MAX_ITEMS];
-  __shared__ int s_Ma[MAX_ITEMS];
-  __shared__ int s_off[MAX_ITEMS + 1];      // prefix of pair counts of the active items this round
-  __shared__ unsigned char s_active[MAX_ITEMS];
-  __shared__ C2* s_A[MAX_ITEMS];
-  __shared__ C2* s_V[MAX_ITEMS];
-  __shared__ R s_part[GROUPS][GROUP_WARPS][4];
-  __shared__ R s_rot[GROUPS][8];            // rotate flag, c, s, s e^{-i phi}, c e^{-i phi}
-  __shared__ double s_fro[MAX_ITEMS];       // ||A||_F^2 per item (noise floor)
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int grp = wid / GROUP_WARPS, gw = wid % GROUP_WARPS;
-  const int slot = grp / 2, sub = grp % 2;               // a task slot = 2 groups = 8 warps
-  const int n_slots = gridDim.x * (GROUPS / 2);
-  const int my_slot = slot * gridDim.x + blockIdx.x;     // consecutive tasks go to different SMs
-  const R eps = Cx<R>::EPS;
+  __shared__ Slot s_slot[JG];
+  __shared__ int s_b, s_rounds, s_fit, s_most, s_cols;
+  const int ctid = threadIdx.x, grp = ctid / JT, tid = ctid % JT, lane = tid & 31, wid = tid >> 5, cwid = ctid >> 5;
+  Slot& S = s_slot[grp];
   if (n_work > MAX_ITEMS) {
-    if (blockIdx.x == 0 && tid == 0) atomicOr(status, ST_CAPACITY);
+    if (blockIdx.x == 0 && ctid == 0) atomicOr(status, ST_CAPACITY);
     return;
   }
-  __shared__ int s_Nf[MAX_ITEMS];           // on_b: rows of B (= columns of D); else Na
-  for (int w = tid; w < n_work; w += blockDim.x) {
+  double* s_fro = (double*)s_raw;                    // ||A||_F^2 per item
+  int* s_Na = (int*)(s_fro + n_work);                // columns that are rotated
+  int* s_Ma = s_Na + n_work;                         // rows
+  int* s_off = s_Ma + n_work;                        // [n_work + 1] prefix of the round's tasks
+  int* s_act = s_off + n_work + 1;
+  const int hdr = (8 * n_work + 4 * (4 * n_work + 1) + 15) & ~15;
+  const int slot_bytes = (dyn_bytes - hdr) / n_grp & ~15;
+  double2* s_col = (double2*)(s_raw + hdr + (size_t)grp * slot_bytes);
+  for (int w = ctid; w < n_work; w += CT) {
     int Ma, Na;
     item_shape(work[w], &Ma, &Na);
     // on_b = 1: B = R^H of the pivoted QR (G64), Na rows and k = info[8] columns (the QR's rank);
-    // on_b = 2: the range finder's small square factor (G64), l = info[9] rows and columns
+    // on_b = 2: R^H of the range finder's small square factor (in V), l = info[9] rows and columns
     const int kq = on_b == 1 ? max(0, min(work[w].info[8], Na)) : (on_b == 2 ? max(0, min(work[w].info[9], Na)) : Na);
-    s_Nf[w] = on_b == 2 ? kq : Na;
     s_Na[w] = kq;
     s_Ma[w] = on_b == 1 ? Na : (on_b == 2 ? kq : Ma);
-    s_active[w] = kq >= 2;
-    s_A[w] = on_b ? Cx<R>::B(work[w]) : Cx<R>::A(work[w]);
-    s_V[w] = Cx<R>::V(work[w]);
+    s_act[w] = kq >= 2;
   }
   __syncthreads();
-  // V = I (optional), zero counters, column norms (for the noise floor)
-  {
-    const int gt = blockIdx.x * blockDim.x + tid, ngt = gridDim.x * blockDim.x;
-    for (int w = 0; w < n_work; ++w) {
-      const int Na = s_Na[w];
-      if (init_v && with_v) {
-        C2* V = s_V[w];
-        for (size_t idx = gt; idx < (size_t)Na * Na; idx += ngt) {
-          C2 v;
-          v.x = ((idx % Na) == (idx / Na)) ? R(1) : R(0);
-          v.y = R(0);
-          __stcg(V + idx, v);
-        }
-      }
-      if (gt == 0) {
-        cnt[2 * w] = 0;
-        cnt[2 * w + 1] = 0;
-      }
-      for (int c = gt; c < Na; c += ngt) __stcg(work[w].perm + c, -1);   // rotation stamps (perm is free until the end)
+  if (cwid == 0) {
+    int rows = 0;
+    for (int w = lane; w < n_work; w += 32) rows = max(rows, s_Ma[w] + (with_v ? s_Na[w] : 0));
+    rows = __reduce_max_sync(0xffffffffu, rows);
+    const int fit = SM ? (rows > 0 ? slot_bytes / (16 * rows) : 2) : 2;
+    const int b = SM ? choose_block(s_Na, s_Ma, n_work, n_grp * gridDim.x, gridDim.x, fit, with_v != 0, lane) : 1;
+    int most = 0, cols = 0;
+    for (int w = lane; w < n_work; w += 32) {
+      const int nb = (s_Na[w] + b - 1) / b, nbp = nb + (nb & 1);
+      if (s_Na[w] >= 2) most += nbp / 2;
+      cols += s_Na[w];
     }
-    const int gwarp = wid * gridDim.x + blockIdx.x, ngwarp = gridDim.x * (blockDim.x / 32);
+    most = __reduce_add_sync(0xffffffffu, most);
+    cols = __reduce_add_sync(0xffffffffu, cols);
+    if (lane == 0) {
+      s_fit = fit;
+      s_b = b;
+      s_most = most;
+      s_cols = cols;
+    }
+  }
+  __syncthreads();
+  if (s_fit < 2) {                         // the host sized the buffer for the capacities: cannot happen
+    if (blockIdx.x == 0 && ctid == 0) atomicOr(status, ST_CAPACITY);
+    return;
+  }
+  const int b = s_b, wpp = JW / b, lw = __ffs(wpp) - 1;      // warps per pair, its logarithm
+  // CTAs that take part: as many as a round has tasks (and the passes over all columns can use)
+  const int G = max(1, min((int)gridDim.x, max(s_most, min((s_cols + 15) / 16, 152))));
+  if ((int)blockIdx.x >= G) return;
+  auto barrier = [&]() { return grid_barrier(gs, status, G); };
+  // V = I, zero counters, unit scales, column norms
+  {
+    const int gt = blockIdx.x * CT + ctid, ngt = G * CT;
+    const int gwarp = cwid * G + blockIdx.x, ngwarp = G * CW;
     int base = 0;
     for (int w = 0; w < n_work; ++w) {
+      const BondWork& W = work[w];
       const int Ma = s_Ma[w], Na = s_Na[w];
+      if (with_v)
+        for (size_t idx = gt; idx < (size_t)Na * Na; idx += ngt)
+          __stcg(W.V + idx, make_double2((idx % Na) == (idx / Na) ? 1.0 : 0.0, 0.0));
+      if (gt == 0) {
+        W.info[4] = 0;
+        W.info[5] = 0;
+      }
+      double2* A = mat_of(W, on_b);
       for (int c = gwarp - base; c < Na; c += ngwarp) {
         if (c < 0) continue;
-        const C2* a = s_A[w] + (size_t)c * Ma;
+        double2* a = A + (size_t)c * Ma;
         double s2 = 0;
         for (int r = lane; r < Ma; r += 32) {
-          const C2 x = __ldcg(a + r);
-          s2 += (double)x.x * x.x + (double)x.y * x.y;
+          double2 x = make_double2(0.0, 0.0);
+          if (on_b != 2) {
+            x = __ldcg(a + r);
+          } else {
+            if (r >= c) {
+              const double2 y = __ldcg(W.G64 + c + (size_t)r * Ma);
+              x = make_double2(y.x, -y.y);
+            }
+            __stcg(a + r, x);
+          }
+          s2 = fma(x.x, x.x, fma(x.y, x.y, s2));
         }
-        s2 = wsumd(s2);
-        if (lane == 0) __stcg(work[w].aux + c, s2);
+        s2 = wsum(s2);
+        if (lane == 0) {
+          __stcg(W.aux + c, s2);
+          __stcg(W.sig + c, 1.0);
+        }
       }
       base = (base + Na) % ngwarp;
     }
   }
-  if (!grid_barrier(gs, status)) return;
+  if (!barrier()) return;
   // ||A||_F^2 per item, summed in the same fixed order by every CTA
-  for (int w = wid; w < n_work; w += blockDim.x / 32) {
+  for (int w = cwid; w < n_work; w += CW) {
     double acc = 0;
     for (int k = lane; k < s_Na[w]; k += 32) acc += __ldcg(work[w].aux + k);
-    acc = wsumd(acc);
+    acc = wsum(acc);
     if (lane == 0) s_fro[w] = acc;
   }
-  __syncthreads();
-  int sweep = 0;
-  bool any = false;
-  for (int w = 0; w < n_work; ++w) any |= s_active[w] != 0;
-  // fixed stride of the global round index (every matrix's tournament fits in it), so that a pair
-  // that meets in round r of every sweep met one stride earlier, whichever matrices are still active
-  int stride = 1;
-  for (int w = 0; w < n_work; ++w)
-    if (s_Na[w] >= 2) {
-      const int nb = (s_Na[w] + 1) / 2, nbp = nb + (nb & 1);
-      stride = max(stride, nbp - 1);
-    }
-  while (any && sweep < max_sweeps) {
-    const int par = sweep & 1;
-    if (blockIdx.x == 0)
-      for (int w = tid; w < n_work; w += blockDim.x) cnt[2 * w + (par ^ 1)] = 0;
-    // 2-column blocks: a task pairs two blocks and runs their cross pairs (and, in round 0, the
-    // pairs inside each block) in sub-rounds separated by a barrier of the task's 8 warps; the
-    // round-robin tournament runs over blocks, so a sweep has half as many grid barriers
+  // the rounds of the next sweep: the longest tournament among the active items (0: all converged)
+  auto set_rounds = [&]() {
+    if (cwid != 0) return;
     int rounds = 0;
-    for (int w = 0; w < n_work; ++w)
-      if (s_active[w]) {
-        const int nb = (s_Na[w] + 1) / 2, nbp = nb + (nb & 1);
+    for (int w = lane; w < n_work; w += 32)
+      if (s_act[w]) {
+        const int nb = (s_Na[w] + b - 1) / b, nbp = nb + (nb & 1);
         rounds = max(rounds, nbp - 1);
       }
+    rounds = __reduce_max_sync(0xffffffffu, rounds);
+    if (lane == 0) s_rounds = rounds;
+  };
+  set_rounds();
+  __syncthreads();
+  int sweep = 0;
+  while (s_rounds > 0 && sweep < max_sweeps) {
+    const int par = sweep & 1, rounds = s_rounds;
+    if (blockIdx.x == 0)
+      for (int w = ctid; w < n_work; w += CT) work[w].info[4 + (par ^ 1)] = 0;
     for (int round = 0; round < rounds; ++round) {
-      const int g_round = sweep * stride + round;    // a pair meets in the same round of every sweep
-      if (tid == 0) {
-        int o = 0;
-        for (int w = 0; w < n_work; ++w) {
-          s_off[w] = o;
-          const int nb = (s_Na[w] + 1) / 2, nbp = nb + (nb & 1);
-          if (s_active[w] && round < nbp - 1) o += nbp / 2;
+      // prefix of the active items' task counts (warp 0)
+      if (cwid == 0) {
+        int run = 0;
+        for (int w0 = 0; w0 < n_work; w0 += 32) {
+          const int w = w0 + lane;
+          int v = 0;
+          if (w < n_work && s_act[w]) {
+            const int nb = (s_Na[w] + b - 1) / b, nbp = nb + (nb & 1);
+            if (round < nbp - 1) v = nbp / 2;
+          }
+          int inc = v;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += t;
+          }
+          if (w < n_work) s_off[w] = run + inc - v;
+          run += __shfl_sync(0xffffffffu, inc, 31);
         }
-        s_off[n_work] = o;
+        if (lane == 0) s_off[n_work] = run;
       }
       __syncthreads();
       const int total = s_off[n_work];
-      for (int t = my_slot; t < total; t += n_slots) {
+      for (int t = grp < n_grp ? grp * G + (int)blockIdx.x : total; t < total; t += n_grp * G) {
         int lo = 0, hi = n_work - 1;
         while (lo < hi) {
           const int mid = (lo + hi + 1) >> 1;
           if (s_off[mid] <= t) lo = mid;
           else hi = mid - 1;
         }
-        const int w = lo;
-        const int q = t - s_off[w];
-        const int Ma = s_Ma[w], Na = s_Na[w];
-        const int nb = (Na + 1) / 2, nbp = nb + (nb & 1);
+        const int w = lo, q = t - s_off[w];
+        const BondWork& W = work[w];
+        const int Ma = s_Ma[w], Na = s_Na[w], Vr = with_v ? Na : 0, ld = Ma + Vr;
+        const int nb = (Na + b - 1) / b, nbp = nb + (nb & 1);
         int bi, bj;
         if (q == 0) { bi = nbp - 1; bj = round; }
         else { bi = (round + q) % (nbp - 1); bj = (round - q + nbp - 1) % (nbp - 1); }
-        const int i0 = 2 * bi, j0 = 2 * bj;
-        const int n_sub = round == 0 ? 3 : 2;
-        for (int sr = 0; sr < n_sub; ++sr) {
-          int i, j;
-          if (sr == 0) { i = i0 + sub; j = j0 + sub; }
-          else if (sr == 1) { i = i0 + sub; j = j0 + 1 - sub; }
-          else { i = sub == 0 ? i0 : j0; j = i + 1; }          // pairs inside each block
-          process_pair<R>(s_A[w], s_V[w], work[w].aux, Ma, Na, i, j, s_fro[w], floor_eps, grp, gw, lane, s_part,
-                          s_rot, &cnt[2 * w + par], with_v != 0, work[w].perm, g_round,
-                          sweep > 0 ? g_round - stride : INT_MIN,
-                          (R)((tol_scale > 0 ? tol_scale : (tol_scale < 0 ? 4.0 * sqrt((double)Ma) : (double)Ma)) * eps));
-          named_sync(9 + slot, 32 * GROUP_WARPS * 2);
+        double2* A = mat_of(W, on_b);
+        // local column c: global column of block bi (c < b) or bj; -1 beyond the matrix
+        auto gcol = [&](int c) {
+          const int g = (c < b ? bi * b + c : bj * b + c - b);
+          return g < Na ? g : -1;
+        };
+        if (tid < 2 * b) {
+          const int g = gcol(tid);
+          S.nrm[tid] = g >= 0 ? __ldcg(W.aux + g) : 0.0;
+          S.q[tid] = g >= 0 ? __ldcg(W.sig + g) : 1.0;
+          S.rotc[tid] = 0;
         }
+        if (tid == 0) S.cnt = 0;
+        // the column warps share the 2 b columns evenly: JW / 2b warps per column, or two columns per warp
+        const int wpc = max(1, wpp >> 1), c0 = wpp > 1 ? wid / wpc : wid, rc0 = (wpp > 1 ? wid % wpc : 0) * 32 + lane;
+        if (SM) {
+          for (int c = c0; c < 2 * b && wid < JW; c += JW) {
+            const int g = gcol(c);
+            if (g < 0) continue;
+            const double2* a = A + (size_t)g * Ma;
+            const double2* v = W.V + (size_t)g * Na - Ma;
+            double2* dst = s_col + (size_t)c * ld;
+#pragma unroll 4
+            for (int r = rc0; r < ld; r += 32 * wpc) cp16(dst + r, (r < Ma ? a : v) + r);
+          }
+          asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+        }
+        slot_sync(grp);
+        // noise floor as the bits of a non-negative double; significand and exponent of the squared threshold
+        const long long fl2 = __double_as_longlong(floor2 * s_fro[w]);
+        const double tol = (tol_scale > 0 ? tol_scale : (double)Ma) * UNIT;
+        int et;
+        const float tm = significand(tol * tol, &et);
+        const int n_inner = round == 0 ? b - 1 : 0;
+        const int n_cross = bi < nb && bj < nb ? b : 0;       // none against the padding block
+        for (int sr = 0; sr < n_inner + n_cross; ++sr) {
+          const int p = wid >> lw, gw = wid & (wpp - 1);
+          // pair p's local columns: inside a block (round-robin over its b columns) or across the two
+          auto pair_of = [&](int pp, int* i, int* j) {
+            if (sr < n_inner) {
+              const int h = b / 2, blk = pp >= h, x = pp - blk * h;
+              int u, v;
+              if (x == 0) { u = b - 1; v = sr; }
+              else { u = (sr + x) % (b - 1); v = (sr - x + b - 1) % (b - 1); }
+              *i = blk * b + min(u, v);
+              *j = blk * b + max(u, v);
+            } else {
+              *i = pp;
+              *j = b + ((pp + sr - n_inner) & (b - 1));
+            }
+          };
+          int li = 0, lj = 0;
+          double2 *x = nullptr, *y = nullptr;
+          auto load = [](const double2* s) { return SM ? *s : __ldcg(s); };
+          auto store = [](double2* s, double2 v) {
+            if (SM) *s = v;
+            else __stcg(s, v);
+          };
+          const int r0 = gw * 32 + lane, step = wpp * 32;
+          if (wid < JW) {
+            pair_of(p, &li, &lj);
+            const int gi = gcol(li), gj = gcol(lj);
+            x = SM ? s_col + (size_t)li * ld : A + (size_t)max(gi, 0) * Ma;
+            y = SM ? s_col + (size_t)lj * ld : A + (size_t)max(gj, 0) * Ma;
+            if (gi >= 0 && gj >= 0) {
+              double gr = 0, gim = 0;
+              for (int r = r0; r < Ma; r += step) {
+                const double2 u = load(x + r), v = load(y + r);
+                gr = fma(u.x, v.x, fma(u.y, v.y, gr));
+                gim = fma(u.x, v.y, fma(-u.y, v.x, gim));
+              }
+              const double s = wsum2(gr, gim, lane);
+              if ((lane & 15) == 0) S.part[wid][lane >> 4] = s;
+            }
+            slot_sync(grp);
+          } else {
+            // lanes 2 k + comp take column warp k's partial sum; the lanes of a pair compute the same
+            const int pp = min(lane >> (1 + lw), b - 1);
+            int i, j;
+            pair_of(pp, &i, &j);
+            const bool lead = (lane & 1) == 0 && ((lane >> 1) & (wpp - 1)) == 0 && lane < 2 * JW;
+            const double al = S.nrm[i], be = S.nrm[j], qx = S.q[i], qy = S.q[j];
+            const double h = be - al, qq = qx * qy;
+            int ea, eb, eh;
+            const float am = significand(al, &ea), bm = significand(be, &eb), hm = significand(h, &eh);
+            // rotate unless |gamma| <= tol sqrt(alpha beta), or a column is at the noise floor (compared as
+            // integers; a NaN fails below)
+            bool go = gcol(i) >= 0 && gcol(j) >= 0 &&
+                      min(__double_as_longlong(al), __double_as_longlong(be)) > max(fl2, 0x0010000000000000ll - 1);
+            if (lane == 0) S.renorm[sr & 1] = 0;
+            slot_sync(grp);
+            double v = lane < 2 * JW ? S.part[lane >> 1][lane & 1] : 0.0;
+            for (int o = 2; o < 2 * wpp; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            const double other = __shfl_xor_sync(0xffffffffu, v, 1);
+            const double gr = (lane & 1) ? other : v, gm = (lane & 1) ? v : other;
+            const double g2 = qq * fma(gr, gr, gm * gm);             // |gamma|^2
+            int eg;
+            const float gs = significand(g2, &eg);
+            const int dt = et + ea + eb - eg;
+            go = go && eg > -1000 && eg < 1000 && ea < 1000 && eb < 1000 &&
+                 (dt < -4 || (dt < 4 && gs > tm * am * bm * __int_as_float((127 + max(dt, -8)) << 23)));
+            // rho = 2 sign(h) / (|h| + sqrt(h^2 + 4 |gamma|^2)), h = beta - alpha, on values scaled by 2^-E
+            const int E = max(eh, (eg + 1) >> 1);
+            const float hf = eh > -1023 ? scale_pow2(hm, eh - E) : 0.f, gf = scale_pow2(gs, eg - 2 * E);
+            const float rf = __fdividef(2.0f, hf + __fsqrt_rn(fmaf(hf, hf, 4.0f * gf)));
+            const int rb = __float_as_int(rf);
+            const double rho = __hiloint2double(((rb >> 3) + ((1023 - 127 - E) << 20)) | (__double2hiint(h) & 0x80000000),
+                                                rb << 29);
+            const double ry = rho * qy, rx = rho * qx;
+            if (lead) {
+              if (go) {
+                S.rot[pp][0] = ry * gr;
+                S.rot[pp][1] = ry * gm;
+                S.rot[pp][2] = rx * gr;
+                S.rot[pp][3] = rx * gm;
+              }
+              S.flag[pp] = go;
+            }
+            slot_sync(grp);
+            // while the columns rotate: the squared norms after a rotation by any angle, unless they cancel below a
+            // quarter (then recomputed from the columns), and the squared scales times cos^2
+            if (lead) {
+              int redo = 0;
+              if (go) {
+                const double rg = rho * g2, t2 = rho * rg, a1 = 1.0 + t2;
+                const double y0 = (double)(1.0f / (float)a1), e0 = fma(-a1, y0, 1.0);
+                const double c2 = fma(y0, fma(e0, e0, e0), y0);      // an FP32 seed, a third-order step: 1 / a1
+                const double al2 = c2 * fma(t2, be, fma(-2.0, rg, al)), be2 = c2 * fma(t2, al, fma(2.0, rg, be));
+                // a quarter of alpha: two less in the exponent field
+                redo = __double2hiint(al2) < __double2hiint(al) - (2 << 20) ||
+                       __double2hiint(be2) < __double2hiint(be) - (2 << 20);
+                if (redo) S.renorm[sr & 1] = 1;
+                S.nrm[i] = al2;
+                S.nrm[j] = be2;
+                S.q[i] = qx * c2;
+                S.q[j] = qy * c2;
+                S.rotc[i] = S.rotc[j] = 1;
+                atomicAdd(&S.cnt, 1);
+              }
+              S.redo[pp] = redo;
+            }
+          }
+          if (wid < JW) slot_sync(grp);
+          if (wid < JW && S.flag[p]) {
+            const double mr = S.rot[p][0], mi = S.rot[p][1], nr = S.rot[p][2], ni = S.rot[p][3];
+            // x <- x - conj(mu) y, y <- y + nu x
+            auto rotate = [&](double2* u, double2* v, int r) {
+              const double2 a = load(u + r), c = load(v + r);
+              double2 na, nc;
+              na.x = fma(-mr, c.x, fma(-mi, c.y, a.x));
+              na.y = fma(-mr, c.y, fma(mi, c.x, a.y));
+              nc.x = fma(nr, a.x, fma(-ni, a.y, c.x));
+              nc.y = fma(nr, a.y, fma(ni, a.x, c.y));
+              store(u + r, na);
+              store(v + r, nc);
+            };
+            if (SM) {
+              for (int r = r0; r < ld; r += step) rotate(x, y, r);
+            } else {
+              for (int r = r0; r < Ma; r += step) rotate(x, y, r);
+              for (int r = r0; r < Vr; r += step)
+                rotate(W.V + (size_t)gcol(li) * Na, W.V + (size_t)gcol(lj) * Na, r);
+            }
+          }
+          slot_sync(grp);
+          if (S.renorm[sr & 1]) {
+            // uniform in the CTA: pairs whose closed-form norms cancel get them from their columns
+            if (wid < JW && S.redo[p]) {
+              double na = 0, nb2 = 0;
+              for (int r = r0; r < Ma; r += step) {
+                const double2 u = load(x + r), v = load(y + r);
+                na = fma(u.x, u.x, fma(u.y, u.y, na));
+                nb2 = fma(v.x, v.x, fma(v.y, v.y, nb2));
+              }
+              const double s = wsum2(na, nb2, lane);
+              if ((lane & 15) == 0) S.part[wid][lane >> 4] = s;
+            }
+            slot_sync(grp);
+            if (wid < JW && S.redo[p] && gw == 0 && lane == 0) {
+              double sa = 0, sb = 0;
+              for (int k = 0; k < wpp; ++k) {
+                sa += S.part[p * wpp + k][0];
+                sb += S.part[p * wpp + k][1];
+              }
+              S.nrm[li] = sa * S.q[li];
+              S.nrm[lj] = sb * S.q[lj];
+            }
+            slot_sync(grp);
+          }
+        }
+        // changed columns, norms and scales back; a small scale is multiplied into its column
+        for (int c = c0; c < 2 * b && wid < JW; c += JW) {
+          const int g = gcol(c);
+          if (g < 0 || !S.rotc[c]) continue;
+          const bool fold = __double2hiint(S.q[c]) < MIN_SCALE_HI;
+          double2* a = A + (size_t)g * Ma;
+          double2* v = W.V + (size_t)g * Na - Ma;
+          const double2* from = s_col + (size_t)c * ld;
+          if (SM && !fold) {
+#pragma unroll 4
+            for (int r = rc0; r < ld; r += 32 * wpc) __stcg((r < Ma ? a : v) + r, from[r]);
+          } else if (fold) {
+            const double f = sqrt(S.q[c]);
+            for (int r = rc0; r < ld; r += 32 * wpc) {
+              double2* dst = (r < Ma ? a : v) + r;
+              double2 val = SM ? from[r] : __ldcg(dst);
+              val.x *= f;
+              val.y *= f;
+              __stcg(dst, val);
+            }
+          }
+        }
+        if (tid < 2 * b && S.rotc[tid]) {
+          const int g = gcol(tid);
+          __stcg(W.aux + g, S.nrm[tid]);
+          __stcg(W.sig + g, __double2hiint(S.q[tid]) < MIN_SCALE_HI ? 1.0 : S.q[tid]);
+        }
+        if (tid == 0 && S.cnt) atomicAdd(W.info + 4 + par, S.cnt);
+        slot_sync(grp);
       }
-      if (!grid_barrier(gs, status)) return;
+      if (!barrier()) return;
     }
     // sweep done: retire converged items (every CTA reads the same counters)
-    if (tid == 0)
-      for (int w = 0; w < n_work; ++w)
-        if (s_active[w] && *(volatile int*)&cnt[2 * w + par] == 0) {
-          s_active[w] = 0;
-          if (blockIdx.x == 0) work[w].info[sweep_slot] = sweep + 1;
-        }
+    for (int w = ctid; w < n_work; w += CT)
+      if (s_act[w] && *(volatile int*)(work[w].info + 4 + par) == 0) {
+        s_act[w] = 0;
+        if (blockIdx.x == 0) work[w].info[3] = sweep + 1;
+      }
     __syncthreads();
-    any = false;
-    for (int w = 0; w < n_work; ++w) any |= s_active[w] != 0;
+    set_rounds();
     ++sweep;
-    if (!grid_barrier(gs, status)) return;
+    if (!barrier()) return;
   }
-  // a preconditioning run (no finalize) that reaches its sweep cap is not an error: the FP64 sweeps
-  // that follow finish the job (and report their own non-convergence)
-  if (any && blockIdx.x == 0 && tid == 0) {
-    if (finalize) atomicOr(status, ST_SVD_NOCONV);
+  if (s_rounds > 0 && blockIdx.x == 0 && ctid == 0) {
+    atomicOr(status, ST_SVD_NOCONV);
     for (int w = 0; w < n_work; ++w)
-      if (s_active[w]) work[w].info[sweep_slot] = -sweep;
+      if (s_act[w]) work[w].info[3] = -sweep;
   }
-  if (!finalize) return;
-  // singular values: column norms, normalise the columns (left vectors), then rank by sigma
+  // singular values: column norms times the scales; normalised columns (left vectors) and V with its scales
   {
-    const int gwarp = wid * gridDim.x + blockIdx.x, ngwarp = gridDim.x * (blockDim.x / 32);
+    const int gwarp = cwid * G + blockIdx.x, ngwarp = G * CW;
     int base = 0;
     for (int w = 0; w < n_work; ++w) {
+      const BondWork& W = work[w];
       const int Ma = s_Ma[w], Na = s_Na[w];
       for (int c = gwarp - base; c < Na; c += ngwarp) {
         if (c < 0) continue;
-        C2* a = s_A[w] + (size_t)c * Ma;
-        R s2 = 0;
+        double2* a = mat_of(W, on_b) + (size_t)c * Ma;
+        const double q = __ldcg(W.sig + c), d = q == 1.0 ? 1.0 : sqrt(q);
+        double s2 = 0;
         for (int r = lane; r < Ma; r += 32) {
-          const C2 x = __ldcg(a + r);
-          s2 += x.x * x.x + x.y * x.y;
+          const double2 x = __ldcg(a + r);
+          s2 = fma(x.x, x.x, fma(x.y, x.y, s2));
         }
-        s2 = wsumd(s2);
-        const R sg = sqrt(s2);
-        if (lane == 0) __stcg(work[w].sig + c, (double)sg);
-        if (sg > R(0)) {
-          const R inv = R(1) / sg;
+        const double nrm = sqrt(wsum(s2)), sg = nrm * d;
+        __syncwarp();
+        if (lane == 0) __stcg(W.sig + c, sg);
+        if (nrm > 0.0) {
+          const double inv = 1.0 / nrm;
           for (int r = lane; r < Ma; r += 32) {
-            C2 x = __ldcg(a + r);
+            double2 x = __ldcg(a + r);
             x.x *= inv;
             x.y *= inv;
             __stcg(a + r, x);
           }
         }
+        if (with_v && d != 1.0) {
+          double2* v = W.V + (size_t)c * Na;
+          for (int r = lane; r < Na; r += 32) {
+            double2 x = __ldcg(v + r);
+            x.x *= d;
+            x.y *= d;
+            __stcg(v + r, x);
+          }
+        }
         if (lane == 0 && !(sg == sg)) {
           atomicOr(status, ST_NAN);
-          atomicOr(work[w].info + 6, FAULT_SIGMA_NAN);
+          atomicOr(W.info + 6, FAULT_SIGMA_NAN);
         }
       }
       base = (base + Na) % ngwarp;
     }
   }
-  // on_b: the columns of D beyond the QR's rank have singular value 0 (after the sigma of the
-  // k columns above, so the ranking below sees every column)
-  if (on_b) {
-    const int gt = blockIdx.x * blockDim.x + tid, ngt = gridDim.x * blockDim.x;
+  // on_b: the columns of D beyond the QR's rank have singular value 0
+  const int gt = blockIdx.x * CT + ctid, ngt = G * CT;
+  auto full = [&](int w) { return on_b == 1 ? s_Ma[w] : s_Na[w]; };
+  if (on_b == 1)
     for (int w = 0; w < n_work; ++w)
-      for (int c = s_Na[w] + gt; c < s_Nf[w]; c += ngt) __stcg(work[w].sig + c, 0.0);
-  }
-  if (!grid_barrier(gs, status)) return;
-  {
-    const int gt = blockIdx.x * blockDim.x + tid, ngt = gridDim.x * blockDim.x;
-    for (int w = 0; w < n_work; ++w) {
-      const int Na = s_Nf[w];
-      const double* sig = work[w].sig;
-      for (int c = gt; c < Na; c += ngt) {
-        // a NaN ranks as -1 so the ranks stay a permutation (perm indexes columns downstream)
-        double sc = __ldcg(sig + c);
-        if (!(sc == sc)) sc = -1.0;
-        int rk = 0;
-        for (int k = 0; k < Na; ++k) {
-          double sk = __ldcg(sig + k);
-          if (!(sk == sk)) sk = -1.0;
-          rk += (sk > sc) || (sk == sc && k < c);
-        }
-        work[w].perm[rk] = c;
+      for (int c = s_Na[w] + gt; c < full(w); c += ngt) __stcg(work[w].sig + c, 0.0);
+  if (!barrier()) return;
+  for (int w = 0; w < n_work; ++w) {
+    const int Na = full(w);
+    const double* sig = work[w].sig;
+    for (int c = gt; c < Na; c += ngt) {
+      // order by the values' bits (sign and magnitude are those of a non-negative number); a NaN ranks below
+      // every number so the ranks stay a permutation (perm indexes columns downstream)
+      auto key = [&](int k) {
+        const long long v = __double_as_longlong(__ldcg(sig + k));
+        return (v & 0x7fffffffffffffffll) > 0x7ff0000000000000ll ? -1ll : v;
+      };
+      const long long sc = key(c);
+      int rk = 0;
+      for (int k = 0; k < Na; ++k) {
+        const long long sk = key(k);
+        rk += (sk > sc) || (sk == sc && k < c);
       }
+      work[w].perm[rk] = c;
     }
   }
 }
+
+namespace {
+// dynamic shared memory of a launch over n_work items with columns of at most `rows` rows (V included), and the
+// task slots it holds (two if each has room for b = 2); the header alone: the columns stay in L2
+int jacobi_smem(int n_work, int rows, int* n_grp) {
+  constexpr long long MAX = 220 * 1024;          // 227 KB per SM less the static arrays
+  const int hdr = (8 * n_work + 4 * (4 * n_work + 1) + 15) & ~15;
+  const long long col = 16LL * rows;
+  *n_grp = JG;
+  if (hdr + JG * 4 * col <= MAX) return (int)std::min(MAX, hdr + JG * 2 * JB * col);
+  *n_grp = 1;
+  if (hdr + 2 * col <= MAX) return (int)std::min(MAX, hdr + 2 * JB * col);
+  *n_grp = JG;
+  return hdr;
+}
+}  // namespace
 
 int jacobi_grid_blocks() {
   int dev = 0, sms = 0, a = 0, b = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_jacobi_grid<double>, GRID_THREADS, 0);
-  (void)b;
-  return a >= 1 ? sms : 0;
+  cudaFuncSetAttribute(k_jacobi_grid<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_jacobi_grid<true>, CT, 220 * 1024);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_jacobi_grid<false>, CT, 32 * 1024);
+  cudaGetLastError();
+  return a >= 1 && b >= 1 ? sms : 0;
 }
 
-void launch_jacobi_grid(const BondWork* work, int n_work, int blocks, int max_sweeps, unsigned* sync3,
-                        int* cnt, int* status, cudaStream_t st, int init_v, int finalize,
-                        double floor_eps, int sweep_slot, int on_b, int with_v, double tol_scale) {
+void launch_jacobi_grid(const BondWork* work, int n_work, int blocks, int rows_cap, int max_sweeps, unsigned* sync3,
+                        int* status, cudaStream_t st, int on_b, int with_v, double tol_scale, double floor2) {
   // the barrier's arrival counter and the abort flag start at zero for every launch
-  cudaMemsetAsync(sync3, 0, sizeof(unsigned), st);
-  cudaMemsetAsync(sync3 + 2, 0, sizeof(unsigned), st);
+  cudaMemsetAsync(sync3, 0, 3 * sizeof(unsigned), st);
   GridSync gs{sync3, (int*)(sync3 + 2), GRID_WAIT_LIMIT_CYCLES};
+  int n_grp = 1;
+  const int hdr = jacobi_smem(n_work, 1 << 20, &n_grp), smem = jacobi_smem(n_work, rows_cap, &n_grp);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks, 1, 1);
-  cfg.blockDim = dim3(GRID_THREADS, 1, 1);
+  cfg.blockDim = dim3(CT, 1, 1);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeCooperative;
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_jacobi_grid<double>, work, n_work, max_sweeps, gs, cnt, status, init_v, finalize,
-                     floor_eps, sweep_slot, on_b, with_v, tol_scale);
+  cudaLaunchKernelEx(&cfg, smem > hdr ? k_jacobi_grid<true> : k_jacobi_grid<false>, work, n_work, max_sweeps, gs,
+                     status, on_b, with_v, tol_scale, floor2, n_grp, smem);
+}
+
+// Whole GPU against one cluster per matrix: two 256 x 256 matrices 113 ms in two 16-CTA clusters (32 of 152 SMs),
+// see the head of this file; the cluster kernel takes what one launch of this one does not.
+void launch_svd_jacobi(const BondWork* items, int batch, int Ma, int Na, int max_sweeps, int* status, unsigned* sync3,
+                       cudaStream_t st) {
+  const int blocks = batch <= MAX_ITEMS ? jacobi_grid_blocks() : 0;
+  if (blocks > 0) {
+    launch_jacobi_grid(items, batch, blocks, Ma + Na, max_sweeps, sync3, status, st, /*on_b=*/0, /*with_v=*/1, 0.0);
+  } else {
+    const int cl = jacobi_cluster_size(std::max(1, std::min(16, (Na / 2 + 7) / 8)));
+    launch_jacobi_cluster(items, batch, cl, max_sweeps, status, st);
+  }
 }
 
 }  // namespace ptk

@@ -54,18 +54,22 @@ int jacobi_cluster_size(int want);
 void launch_jacobi_cluster(const BondWork* work, int n_work, int cluster, int max_sweeps, int* status,
                            cudaStream_t st);
 
-// whole-GPU FP64 bond SVD (jacobi_grid.cu): blocks = one per SM (0 if not co-schedulable);
-// sync3: 3 words of device memory (arrival count, unused, abort flag); cnt: 2 ints per item
+// whole-GPU FP64 bond SVD (jacobi_grid.cu): blocks = the SM count (0 if not co-schedulable); rows_cap: the
+// largest column length at capacity (rows of the matrix, plus those of V with with_v); sync3: 3 words of device
+// memory (arrival count, unused, abort flag). Sweeps go to info[3], rotation counters in info[4..5].
 int jacobi_grid_blocks();
-// init_v: start from V = I; finalize: sigma, U, order; floor_eps: unit roundoff of the noise floor;
-// sweep_slot: info[] index for the sweep count
-// on_b: 1 = B = R^H of the pivoted QR (Na x info[8]), 2 = the range finder's l x l factor in G64
-// (l = info[9]); with_v: accumulate V; tol_scale: rotation threshold
-// in units of the unit roundoff (0: the row count)
-void launch_jacobi_grid(const BondWork* work, int n_work, int blocks, int max_sweeps, unsigned* sync3,
-                        int* cnt, int* status, cudaStream_t st, int init_v = 1, int finalize = 1,
-                        double floor_eps = 1.1102230246251565e-16, int sweep_slot = 3, int on_b = 0,
-                        int with_v = 1, double tol_scale = 0.0);
+constexpr double JACOBI_FLOOR2 = 1.232595164407831e-32;      // squared noise floor: u^2 = 2^-106
+// on_b: 0 = the matrix in A, 1 = B = R^H of the pivoted QR (Na x info[8]), 2 = R^H of the range finder's l x l
+// factor R in G64 (l = info[9]), formed and overwritten by its left vectors in V; with_v: accumulate V; tol_scale: rotation threshold in units of the unit roundoff (0: the
+// row count); floor2: columns at floor2 ||A||_F^2 or below (squared norms) are left as they are
+void launch_jacobi_grid(const BondWork* work, int n_work, int blocks, int rows_cap, int max_sweeps, unsigned* sync3,
+                        int* status, cudaStream_t st, int on_b, int with_v, double tol_scale,
+                        double floor2 = JACOBI_FLOOR2);
+
+// the standalone batched SVD's Jacobi (k_svd_load before it, k_svd_store after it) on Ma x Na matrices: the whole
+// GPU where it can be co-scheduled and a launch takes the batch, else one cluster per matrix; sync3 as above
+void launch_svd_jacobi(const BondWork* items, int batch, int Ma, int Na, int max_sweeps, int* status, unsigned* sync3,
+                       cudaStream_t st);
 
 // QR preconditioning of the bond SVD (qrcp.cu): pivoted QR of D into Y64, B = R^H into G64;
 // after the Jacobi on B: V_D = P U', U_D = D V_D / sigma
@@ -151,12 +155,14 @@ constexpr int RSVD_POWER = 2;
 void launch_rsvd_omega(double2* Om, int rows, int cols, unsigned seed, cudaStream_t st);
 // the order of a layer: plan (item lists, l into info[9]); gy1 -> QR q1; RSVD_POWER times
 // (gz1 -> QR qz, gy2 -> QR q2); gz2; gres (D - Q Z^H); tail norm; QR qb (l x l factor into G64);
-// Jacobi on it (launch_jacobi_grid, on_b = 2); truncation (k_truncate, rsvd = 1); vectors
+// Jacobi on its R^H (launch_jacobi_grid, on_b = 2); truncation (k_truncate, rsvd = 1); vectors
 void launch_rsvd_plan(const Tables& T, const BondWork* work, int n_work, const RsvdLists& L, int chi_max, int p,
                       const double2* Om, int ld_om, cudaStream_t st);
 // part: RSVD_FRO_PARTS doubles per bond (scratch of the two-pass, fixed-order sum)
 constexpr int RSVD_FRO_PARTS = 64;
 void launch_rsvd_tail_norm(const BondWork* work, int n_work, double* part, cudaStream_t st);
+// R Wr / S of the kept columns (R in G64, Wr in V, columns by perm) into RH, l x chi: Ur of R = Ur S Wr^H
+void launch_rsvd_left(const BondWork* work, int n_work, int l_cap, const int* lam_chi, cudaStream_t st);
 void launch_rsvd_vectors(const Tables& T, const BondWork* work, int n_work, const RsvdLists& L, cudaStream_t st);
 
 // set the message returned by pt_tebd_last_error(NULL) (engine.cu)

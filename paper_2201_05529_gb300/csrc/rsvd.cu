@@ -8,7 +8,7 @@
 //   Z  = D^H Q,     Qz = qr(Z)          (a power iteration: sharpens the decay by sigma^2)
 //   Y  = D Qz,      Q  = qr(Y)
 //   Z  = D^H Q = Qb Rb                  (Z = B^H for B = Q^H D, the l x n projection of D)
-//   Rb = Ur S Wr^H                      (FP64 one-sided Jacobi on the l x l factor)
+//   Rb = Ur S Wr^H                      (FP64 one-sided Jacobi on Rb^H: left vectors Wr; Ur = Rb Wr / S)
 //   D ~ Q B = (Q Wr) S (Qb Ur)^H        (left vectors Q Wr, right vectors Qb Ur)
 //
 // The four products with D (m x n) and the two that form the kept singular vectors run on the
@@ -161,7 +161,7 @@ __global__ void k_rsvd_plan_vectors(Tables T, const BondWork* work, int n_work, 
   const int l = W.info[9];
   const int chi = (Ma > 0 && l > 0) ? min(T.lam_chi[W.lam_l + 1], l) : 0;
   gu[w] = zitem(W, W.RY, max(Ma, 1), ZOP_N, W.V, max(l, 1), ZOP_N, W.A, max(Ma, 1), chi ? Ma : 0, chi, l, W.perm);
-  gv[w] = zitem(W, W.RZ, max(Na, 1), ZOP_N, W.G64, max(l, 1), ZOP_N, W.V, max(Na, 1), chi ? Na : 0, chi, l, W.perm);
+  gv[w] = zitem(W, W.RZ, max(Na, 1), ZOP_N, W.RH, max(l, 1), ZOP_N, W.V, max(Na, 1), chi ? Na : 0, chi, l, nullptr);
 }
 
 // the kept vectors now sit in order: perm = identity on the kept columns (the recovery reads
@@ -191,6 +191,7 @@ void launch_rsvd_tail_norm(const BondWork* work, int n_work, double* part, cudaS
 }
 
 void launch_rsvd_vectors(const Tables& T, const BondWork* work, int n_work, const RsvdLists& L, cudaStream_t st) {
+  launch_rsvd_left(work, n_work, L.l_cap, T.lam_chi, st);
   k_rsvd_plan_vectors<<<(n_work + 127) / 128, 128, 0, st>>>(T, work, n_work, L.gu, L.gv);
   launch_zgemm(L.gu, n_work, L.tile_cap, L.m_cap, L.l_cap, T.status, st);
   launch_zgemm(L.gv, n_work, L.tile_cap, L.m_cap, L.l_cap, T.status, st);

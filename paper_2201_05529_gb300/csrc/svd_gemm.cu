@@ -18,9 +18,11 @@ constexpr int TK = 16;   // GEMM K tile
 
 // C[m x n] = op(A)[m x k] * B[k x n], column-major; op = conjugate transpose if conjA.
 // 256 threads, each computes a 2 x 2 block of a 32 x 32 tile.
-// bcol: column c of B is column bcol[c] of the stored matrix (NULL: c)
+// bcol: column c of B is column bcol[c] of the stored matrix (NULL: c). K runs from k_from (a multiple of TK).
+// div: column c of the result is divided by div[bcol[c]] (a zero gives a zero column).
 __device__ void gemm_tile(const double2* A, int lda, bool conjA, const double2* B, int ldb, double2* C, int ldc,
-                          int m, int n, int k, int tm, int tn, const int* bcol = nullptr) {
+                          int m, int n, int k, int tm, int tn, const int* bcol = nullptr, int k_from = 0,
+                          const double* div = nullptr) {
   __shared__ double2 As[TK][TB + 1];
   __shared__ double2 Bs[TK][TB + 1];
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
@@ -29,7 +31,7 @@ __device__ void gemm_tile(const double2* A, int lda, bool conjA, const double2* 
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 2; ++j) acc[i][j] = make_double2(0.0, 0.0);
-  for (int k0 = 0; k0 < k; k0 += TK) {
+  for (int k0 = k_from; k0 < k; k0 += TK) {
     for (int e = threadIdx.x; e < TK * TB; e += blockDim.x) {
       const int kk = e / TB, mm = e % TB;
       const int row = tm * TB + mm, col = k0 + kk;
@@ -69,7 +71,14 @@ __device__ void gemm_tile(const double2* A, int lda, bool conjA, const double2* 
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const int row = tm * TB + ty * 2 + i, col = tn * TB + tx * 2 + j;
-      if (row < m && col < n) C[row + (size_t)col * ldc] = acc[i][j];
+      if (row < m && col < n) {
+        if (div) {
+          const double s = div[bcol[col]];
+          acc[i][j].x = s > 0.0 ? acc[i][j].x / s : 0.0;
+          acc[i][j].y = s > 0.0 ? acc[i][j].y / s : 0.0;
+        }
+        C[row + (size_t)col * ldc] = acc[i][j];
+      }
     }
 }
 
@@ -91,6 +100,27 @@ __global__ void __launch_bounds__(256) k_mix_gemm(const BondWork* work, int n_wo
 void launch_mix_gemm_av(const BondWork* work, int n_work, int k_cap, int m_cap, const int* lam_chi, cudaStream_t st) {
   const int tk = (k_cap + TB - 1) / TB, tmm = (m_cap + TB - 1) / TB;
   k_mix_gemm<<<dim3(tmm, tk, n_work), 256, 0, st>>>(work, n_work, lam_chi);
+}
+
+// Ur = R Wr / S on the kept columns (grid: tiles x tiles x items): R upper triangular in G64, so K starts at the
+// tile's diagonal. What the Jacobi would spend on accumulating this factor (8 of its 20 FP64 operations per row and
+// rotated pair, ~9 sweeps) is one product of 4 l^2 chi operations here.
+__global__ void __launch_bounds__(256) k_rsvd_left(const BondWork* work, int n_work, const int* lam_chi) {
+  const int w = blockIdx.z;
+  if (w >= n_work) return;
+  const BondWork& W = work[w];
+  int Ma, Na;
+  shape(W, &Ma, &Na);
+  const int l = Ma > 0 ? W.info[9] : 0;
+  const int n = min(lam_chi[W.lam_l + 1], l);
+  const int tm = blockIdx.x, tn = blockIdx.y;
+  if (tm * TB >= l || tn * TB >= n) return;
+  gemm_tile(W.G64, l, false, W.V, l, W.RH, l, l, n, l, tm, tn, W.perm, tm * TB, W.sig);
+}
+
+void launch_rsvd_left(const BondWork* work, int n_work, int l_cap, const int* lam_chi, cudaStream_t st) {
+  const int t = (l_cap + TB - 1) / TB;
+  k_rsvd_left<<<dim3(t, t, n_work), 256, 0, st>>>(work, n_work, lam_chi);
 }
 
 }  // namespace ptk

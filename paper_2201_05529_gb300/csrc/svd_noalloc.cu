@@ -54,7 +54,7 @@ Layout layout(int m, int n, int batch) {
   L.sig = o; o += align256(sizeof(double) * Na * batch);
   L.perm = o; o += align256(sizeof(int) * Na * batch);
   L.info = o; o += align256(sizeof(int) * 8 * (size_t)batch);
-  L.status = o; o += align256(sizeof(int));
+  L.status = o; o += align256(sizeof(int));      // and the barrier's words at + 8 ints
   L.items = o; o += align256(sizeof(BondWork) * (size_t)batch);
   L.aux = o; o += align256(sizeof(double) * Na * batch);
   L.total = o;
@@ -129,9 +129,8 @@ int pt_svd_f64_noalloc(const double* A, int m, int n, int batch, double* sigma, 
   k_noalloc_setup<<<(batch + 127) / 128, 128, 0, st>>>(base, L, m, n, batch);
   const int gx = (int)std::min<size_t>(256, ((size_t)m * n + 255) / 256);
   ptk::k_svd_load<<<dim3(gx, batch), 256, 0, st>>>((const double2*)A, m, n, batch, (double2*)(base + L.A), sA);
-  const int cl = ptk::jacobi_cluster_size(std::max(1, std::min(16, (Na / 2 + 7) / 8)));
-  ptk::launch_jacobi_cluster((const BondWork*)(base + L.items), batch, cl, max_sweeps,
-                             (int*)(base + L.status), st);
+  ptk::launch_svd_jacobi((const BondWork*)(base + L.items), batch, Ma, Na, max_sweeps, (int*)(base + L.status),
+                         (unsigned*)(base + L.status) + 8, st);
   const int gs = (int)std::min<size_t>(256, ((size_t)(m + n + 1) * Na + 255) / 256);
   ptk::k_svd_store<<<dim3(gs, batch), 256, 0, st>>>((const double2*)(base + L.A), (const double2*)(base + L.V),
                                                     (const double*)(base + L.sig), (const int*)(base + L.perm), m,

@@ -1,0 +1,47 @@
+"""The batched FP64 one-sided Jacobi SVD (pt_svd_f64) against its definition at the sizes where the whole-GPU kernel
+changes its work: single columns, odd counts, block edges (1, 2, 4 or 8 columns per block), a mix that fills
+several blocks, wide matrices, columns too long for shared memory, matrices of very small and large scale, graded,
+rank-deficient and repeated singular values. Bounds: |A - U S V^H| and |U^H U - I| within 1e-13 max(m, n) (rotations
+unitary to rounding, at most a few thousand per column), sigma against LAPACK within 1e-13 max(m, n) of sigma_1."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("m,n,batch,scale", [(1, 1, 1, 1.0), (5, 1, 2, 1.0), (2, 2, 3, 1.0), (3, 3, 1, 1e-60), (9, 7, 4, 1e60),
+                                             (17, 16, 2, 1.0), (33, 33, 1, 1.0), (20, 50, 3, 1.0), (129, 65, 9, 1.0),
+                                             (256, 130, 2, 1.0), (7200, 3, 1, 1.0)])
+def test_jacobi_svd_against_definition(m, n, batch, scale):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2201_05529_gb300 as pkg
+    pkg.build()
+    capi = pkg.load()
+    capi.use_torch_allocator()
+    rng = np.random.default_rng(m * 1009 + n)
+    A = rng.standard_normal((batch, m, n)) + 1j * rng.standard_normal((batch, m, n))
+    A[0] *= np.exp(-12.0 * np.arange(n) / max(1, n))[None, :]            # graded
+    if batch > 1 and n > 2:
+        A[1][:, 2] = A[1][:, 0] - A[1][:, 1]                             # rank-deficient
+    if batch > 2 and min(m, n) > 3:
+        q1 = np.linalg.qr(A[2] if m >= n else A[2].T)[0]
+        A[2] = (q1 if m >= n else q1.T) * 1.0                            # all singular values equal
+    A = A * scale
+    k = min(m, n)
+    At = torch.from_numpy(A).cuda()
+    S = torch.zeros((batch, k), dtype=torch.float64, device="cuda")
+    U = torch.zeros((batch, m, k), dtype=torch.complex128, device="cuda")
+    V = torch.zeros((batch, n, k), dtype=torch.complex128, device="cuda")
+    capi.svd_f64(At, S, U, V, torch.empty(capi.svd_scratch_bytes(m, n, batch), dtype=torch.uint8, device="cuda"))
+    S, U, V = S.cpu().numpy(), U.cpu().numpy(), V.cpu().numpy()
+    tol = 1e-13 * max(m, n)
+    for b in range(batch):
+        s = np.linalg.svd(A[b], compute_uv=False)
+        assert np.all(np.diff(S[b]) <= 0)
+        assert np.abs(S[b] - s).max() <= tol * s[0]
+        assert np.abs((U[b] * S[b]) @ V[b].conj().T - A[b]).max() <= tol * s[0]
+        r = int((s > 1e-10 * s[0]).sum())                                # vectors of the null space are arbitrary in U
+        assert np.abs(U[b][:, :r].conj().T @ U[b][:, :r] - np.eye(r)).max() <= 1e-13 * max(m, n)
+        assert np.abs(V[b].conj().T @ V[b] - np.eye(k)).max() <= tol
