@@ -1797,7 +1797,7 @@ int pt_zgemm_sliced(int opA, int opB, int m, int n, int k, const double* A, int 
   }
   cudaMemcpyAsync(items, h.data(), sizeof(ptk::ZGemmItem) * batch, cudaMemcpyHostToDevice, st);
   cudaMemsetAsync(status, 0, sizeof(int), st);
-  ptk::launch_zgemm(items, batch, ptk::zgemm_tile_cap(m, n) * batch, m, n, status, st);
+  ptk::launch_zgemm(items, batch, ptk::zgemm_tile_cap(m, n) * batch, m, n, status, st, k);
   int hs = 0;
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, st);

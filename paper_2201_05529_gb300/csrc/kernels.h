@@ -116,15 +116,27 @@ struct ZGemmItem {
   int* flag;               // set to 1 when a product entry is not finite (NULL: not reported)
   int acc;                 // 0: C = opA(A) opB(B); -1: C = C - opA(A) opB(B)
   int skip_a;              // 1: A's slice planes and row exponents are already in TA (packed earlier)
+  int skip_b;              // 1: B's are already in TB, or another item of the launch writes them there
+  const double2* A2;       // rows a_split .. M - 1 of opA(A) come from A2 (same op and leading dimension); NULL: all from A
+  int a_split;
+  long long split;         // > 0: each K chunk's product goes to C + chunk * split (chunks of zgemm9_chunks)
 };
 size_t zgemm_pack_bytes(int rows_cap, int k_cap, int which);
 // the A operands' slice planes and row exponents alone (for items whose later products skip them)
 void launch_zgemm_pack_a(const ZGemmItem* items, int n_items, int m_cap_max, int* status, cudaStream_t st);
 int zgemm_tile_cap(int m_cap, int n_cap);
 // tile_cap: total output tiles of the item list at capacity (the persistent grid's upper bound);
-// m_cap_max / n_cap_max: the largest M and N capacities (pack grid sizes)
+// m_cap_max / n_cap_max: the largest M and N capacities (pack grid sizes); k_cap_max: the largest K capacity where it
+// is at most 64 (the preparation then takes more rows per block)
 void launch_zgemm(const ZGemmItem* items, int n_items, int tile_cap, int m_cap_max, int n_cap_max, int* status,
-                  cudaStream_t st);
+                  cudaStream_t st, int k_cap_max = 1 << 30);
+// the same product from nine slices, for uses that need an FP64 product's accuracy (2^-60 of max|row| max|column| per
+// term, one FP64 rounding per 256-long chunk of K, the chunks added in FP64). Its operands' packed sizes, the
+// number of K chunks; unit_cap: output tiles (128 x 32), times the chunks where items are split
+size_t zgemm9_pack_bytes(int rows_cap, int k_cap, int which);
+int zgemm9_chunks(int k);
+void launch_zgemm9(const ZGemmItem* items, int n_items, long long unit_cap, int m_cap_max, int n_cap_max, int k_cap_max,
+                   int* status, cudaStream_t st);
 // the most items one launch_zgemm takes
 int zgemm_max_items();
 

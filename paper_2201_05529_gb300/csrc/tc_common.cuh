@@ -68,6 +68,16 @@ __device__ __forceinline__ uint64_t smem_desc(const void* p, uint32_t lbo, uint3
   return d;                        // base offset 0, layout type 0 = SWIZZLE_NONE
 }
 
+// the same for rows of 32 bytes (one K step) in the 32-byte swizzle: eight rows of 32 bytes per 256-byte atom
+// (SBO), the two 16-byte halves of rows 4 .. 7 exchanged
+__device__ __forceinline__ uint64_t smem_desc_sw32(const void* p) {
+  return smem_desc(p, 16, 256) | (uint64_t)6 << 61;
+}
+// byte offset of half h (16 bytes) of row m in that layout
+__device__ __forceinline__ uint32_t sw32_offset(int m, int h) {
+  return (uint32_t)(m * 32 + ((h ^ (m >> 2 & 1)) * 16));
+}
+
 // instruction descriptor for kind::tf32 (ab_fmt = 2) or kind::f16 with bf16 inputs (ab_fmt = 1):
 // FP32 accumulator, K-major A and B, N >> 3 at bit 17, M >> 4 at bit 24
 __device__ __forceinline__ uint32_t instr_desc(uint32_t ab_fmt, int M, int N) {
@@ -78,6 +88,21 @@ __device__ __forceinline__ uint32_t instr_desc(uint32_t ab_fmt, int M, int N) {
   d |= (uint32_t)(N >> 3) << 17;
   d |= (uint32_t)(M >> 4) << 24;
   return d;
+}
+
+// slice pairs (s, u), s + u < NS, by accumulator level L = min(s + u, NLEV - 1): pair i of level L
+__host__ __device__ constexpr int pair_count(int L, int NS, int NLEV) {
+  int n = 0;
+  for (int t = L; t < (L == NLEV - 1 ? NS : L + 1); ++t) n += t + 1;
+  return n;
+}
+__host__ __device__ constexpr int pair_s(int L, int i) {
+  while (i > L) i -= ++L;          // the deeper levels that share the last accumulator
+  return i;
+}
+__host__ __device__ constexpr int pair_u(int L, int i) {
+  while (i > L) i -= ++L;
+  return L - i;
 }
 
 template <bool BF16>
@@ -96,6 +121,75 @@ __device__ __forceinline__ void mma(uint32_t tmem_d, uint64_t adesc, uint64_t bd
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(en)
         : "memory");
   }
+}
+
+// The MMAs of one K step of a complex product of NS x NS slices (Re += Ar Br - Ai Bi, Im += Ar Bi + Ai Br) into the
+// accumulators dre = tmem + 2 L TN, dim = dre + TN of the levels.
+template <bool BF16, int NS, int NLEV, int TN, uint32_t A_PLANE, uint32_t B_PLANE>
+__device__ __forceinline__ void mma_slices(uint32_t tmem, uint64_t a0, uint64_t b0, uint32_t idesc, bool acc) {
+  constexpr int MOST = pair_count(NLEV - 1, NS, NLEV);
+  auto a = [&](int plane) { return a0 + (uint64_t)(plane * (A_PLANE >> 4)); };
+  auto b = [&](int plane) { return b0 + (uint64_t)(plane * (B_PLANE >> 4)); };
+#pragma unroll
+  for (int i = 0; i < MOST; ++i)
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+      for (int L = NLEV - 1; L >= 0; --L) {
+        if (i >= pair_count(L, NS, NLEV)) continue;
+        const int s = pair_s(L, i), u = pair_u(L, i);
+        const uint32_t dre = tmem + (2 * L) * TN, dim = dre + TN;
+        const bool en = acc || i > 0 || r > 0;
+        if (r == 0) {
+          mma<BF16>(dre, a(s), b(u), idesc, en);
+          mma<BF16>(dim, a(s), b(NS + u), idesc, en);
+        } else {
+          mma<BF16>(dre, a(NS + s), b(NS + u), idesc | NEG_A, en);
+          mma<BF16>(dim, a(NS + s), b(u), idesc, en);
+        }
+      }
+}
+
+// The same with B's planes as (-Bi, Br, Bi) per slice, adjacent: one MMA of 2 TN columns forms Ar Br and Ar Bi, another
+// -Ai Bi and Ai Br, so half as many MMAs. An MMA of 128 rows costs 53 cycles at up to 64 columns, whatever the
+// accumulators of its neighbours, and 66 at 128 (measured; the operands' layout does not matter).
+// The whole warp runs it and `one` lane issues: the descriptors then stay in uniform registers (issued by a branch
+// of one lane, every operand is moved there first and an MMA takes ~110 cycles).
+__device__ __forceinline__ void mma_bf16_one(bool one, uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, bool acc) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %4, 0;\n setp.ne.u32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc ? 1u : 0u), "r"(one ? 1u : 0u)
+      : "memory");
+}
+
+template <int NS, int NLEV, int TN, uint32_t A_PLANE, uint32_t B_PLANE>
+__device__ __forceinline__ void mma_slices_stacked(bool one, uint32_t tmem, uint64_t a0, uint64_t b0, uint32_t idesc,
+                                                   bool acc) {
+  constexpr int MOST = pair_count(NLEV - 1, NS, NLEV);
+  auto a = [&](int plane) { return a0 + (uint64_t)(plane * (A_PLANE >> 4)); };
+  auto b = [&](int plane) { return b0 + (uint64_t)(plane * (B_PLANE >> 4)); };
+#pragma unroll
+  for (int i = 0; i < MOST; ++i)
+#pragma unroll
+    for (int L = NLEV - 1; L >= 0; --L) {
+      if (i >= pair_count(L, NS, NLEV)) continue;
+      const int s = pair_s(L, i), u = pair_u(L, i);
+      const uint32_t d = tmem + 2 * L * TN;
+      mma_bf16_one(one, d, a(s), b(3 * u + 1), idesc, acc || i > 0);
+      mma_bf16_one(one, d, a(NS + s), b(3 * u), idesc, true);
+    }
+}
+
+// one lane of a converged warp
+__device__ __forceinline__ bool elect_one() {
+  uint32_t one;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(one));
+  return one != 0;
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
@@ -139,12 +233,15 @@ struct PackCap {
   size_t plane_bytes, exp_off, total;
 };
 
-__host__ __device__ __forceinline__ PackCap pack_cap(int rows_cap, int k_cap, int tile_rows, int kstep, int ns) {
+// planes: per K step and row tile, 2 ns unless given
+__host__ __device__ __forceinline__ PackCap pack_cap(int rows_cap, int k_cap, int tile_rows, int kstep, int ns,
+                                                     int planes = 0) {
+  if (planes == 0) planes = 2 * ns;
   PackCap c;
   c.tiles = cdiv(rows_cap, tile_rows);
   c.ksteps = cdiv(k_cap, kstep);
   c.plane_bytes = (size_t)tile_rows * ROW_BYTES;
-  c.exp_off = (size_t)c.tiles * c.ksteps * 2 * ns * c.plane_bytes;
+  c.exp_off = (size_t)c.tiles * c.ksteps * planes * c.plane_bytes;
   c.total = c.exp_off + sizeof(int) * (size_t)c.tiles * tile_rows;
   return c;
 }
@@ -187,38 +284,43 @@ __device__ __forceinline__ void pieces(double x, int b, uint32_t* out) {
 // neither the cut into slices nor the addition of the level sums runs on the FP64 pipe.
 
 // BF16 bit patterns (in the upper half of each word) of the NS fixed-point slices of x 2^-e, |x| < 2^e: x is
-// rounded to NS * b fractional bits and cut into signed digits |a_i| <= 2^b, slice value a_i 2^(-b(i+1)). A NaN or
-// an infinity becomes a NaN in slice 0 (every sum it enters comes out NaN).
+// rounded to NS * b fractional bits and cut into signed digits |a_i| <= 2^b, slice value a_i 2^(-b(i+1)) (NS a multiple
+// of three, NS b <= 63). A NaN or an infinity becomes a NaN in slice 0 (every sum it enters comes out NaN).
 template <int NS>
 __device__ __forceinline__ void int_slices(double x, int e, int b, uint32_t* out) {
   const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
   const int ex = (int)((hi >> 20) & 0x7ff);
   const uint64_t mant = ((uint64_t)((hi & 0xfffffu) | (ex ? 0x100000u : 0u)) << 32) | lo;
-  // x = mant 2^(max(ex, 1) - 1075); F = round(x 2^(NS b - e)) fits NS b + 1 <= 43 bits: a right shift by 53 - NS b
-  // or more, except in a row of subnormals, whose e lies below the exponent of the smallest normal number
+  // |x| = mant 2^(max(ex, 1) - 1075); F = round(|x| 2^(NS b - e)) < 2^(NS b): a shift to the right by 53 - NS b or more,
+  // except in a row of subnormals, whose e lies below the exponent of the smallest normal number
   const int sh = 1075 + e - NS * b - max(ex, 1);
-  long long F = 0;
-  if (sh > 0 && sh < 64) F = (long long)((mant + (1ull << (sh - 1))) >> sh);
-  else if (sh <= 0 && sh > -53) F = (long long)(mant << -sh);
-  if ((int)hi < 0) F = -F;
-  // digits of three slices per 32-bit half
-  constexpr int H = NS / 2;
-  const int hb = H * b;
-  const long long up = (F + (1ll << (hb - 1))) >> hb;
-  int half[2] = {(int)up, (int)(F - (up << hb))};
+  uint64_t F = 0;
+  if (sh > 0 && sh < 64) F = (mant + (1ull << (sh - 1))) >> sh;
+  else if (sh <= 0 && sh > -53) F = mant << -sh;
+  // 32-bit parts of three digits, the last part first; the sign goes onto the digits
+  constexpr int P = NS / 3;
+  const int pb = 3 * b;
+  const uint32_t sign = hi & 0x80000000u;
   const int rnd = 1 << (b - 1);
 #pragma unroll
-  for (int h = 1; h >= 0; --h) {
-    int v = half[h];
+  for (int h = P - 1; h >= 0; --h) {
+    int v;
+    if (h > 0) {
+      const uint64_t up = (F + (1ull << (pb - 1))) >> pb;
+      v = (int)((long long)F - (long long)(up << pb));
+      F = up;
+    } else {
+      v = (int)F;
+    }
 #pragma unroll
-    for (int i = H - 1; i >= 0; --i) {
+    for (int i = 2; i >= 0; --i) {
       const int next = i > 0 ? (v + rnd) >> b : 0;
       const int a = i > 0 ? v - (next << b) : v;
       v = next;
       // 1.5 2^(23 - b s) + a 2^(-b s): adding a to the last bits of the constant's pattern
-      const int s = h * H + i + 1;
+      const int s = h * 3 + i + 1;
       const uint32_t magic = (uint32_t)(127 + 23 - b * s) << 23 | 0x400000u;
-      out[h * H + i] = __float_as_uint(__uint_as_float(magic + (uint32_t)a) - __uint_as_float(magic));
+      out[h * 3 + i] = __float_as_uint(__uint_as_float(magic + (uint32_t)a) - __uint_as_float(magic)) ^ sign;
     }
   }
   if (ex == 0x7ff) out[0] = 0x7fc00000u;
@@ -235,30 +337,33 @@ __device__ __forceinline__ unsigned long long mag_bits(double x) {
   return m < 0x7ff0000000000000ull ? m : 0ull;
 }
 
-// n 2^(e - 7 * 7) as a double, n the 64-bit fixed-point sum of a product's levels
-__device__ __forceinline__ double fixed_to_double(long long n, int e) {
+// n 2^(e - lsb) as a double, n the 64-bit fixed-point sum of a product's levels
+__device__ __forceinline__ double fixed_to_double(long long n, int e, int lsb) {
   if (n == 0) return 0.0;
   const unsigned long long a = n < 0 ? (unsigned long long)(-n) : (unsigned long long)n;
   const int lz = __clzll((long long)a);
   // the top 53 bits, rounded to nearest (ties away; a carry moves into the exponent)
-  const unsigned long long m = ((a << lz) >> 10) + 1ull;      // 54 bits + rounding bit
-  const int bexp = 63 - lz - 49 + e + 1023;                   // biased exponent of the leading bit
+  const unsigned long long m = ((a << lz) >> 10) + 1ull;      // 53 bits and the rounding bit
+  const int bexp = 63 - lz - lsb + e + 1023;                  // biased exponent of the leading bit
   if (bexp > 1 && bexp < 2046) {
     const unsigned long long r = (m >> 1) + ((unsigned long long)(bexp - 1) << 52);   // the implicit bit adds one
     return __longlong_as_double((long long)(r | (n < 0 ? 0x8000000000000000ull : 0ull)));
   }
-  return ldexp((double)n, e - 49);
+  return ldexp((double)n, e - lsb);
 }
 
-// the sum of the four level accumulators of one entry (slice width 7) as an integer multiple of 2^-49: the first
-// three are integer multiples of 2^-14, 2^-21, 2^-28 below 2^24 of them (level 2 up to rounding), the last one
-// is rounded to the grid. Returns false when one of them is not finite.
-__device__ __forceinline__ bool level_sum(float f0, float f1, float f2, float f3, long long* out) {
-  const bool fin = (fabsf(f0) < 1e30f) & (fabsf(f1) < 1e30f) & (fabsf(f2) < 1e30f) & (fabsf(f3) < 1e30f);
-  const long long a = __float2int_rn(f0 * 16384.0f), b = __float2int_rn(f1 * 2097152.0f);
-  const long long c = __float2ll_rn(f2 * 562949953421312.0f), d = __float2ll_rn(f3 * 562949953421312.0f);
-  *out = (a << 35) + (b << 28) + c + d;
-  return fin;
+// the sum of levels FROM .. TO of an entry's accumulators (slice width 7) as an integer multiple of 2^-LSB: level L holds
+// integer multiples of 2^(-7 (L + 2)) below 2^24 of them. LAST > 0: the last level, shared by several, is rounded to
+// multiples of 2^-LAST, which fit 32 bits.
+template <int FROM, int TO, int LSB, int LAST, int NLEV>
+__device__ __forceinline__ long long level_sum(const float (&f)[NLEV][8], int j) {
+  long long n = 0;
+#pragma unroll
+  for (int L = FROM; L <= TO; ++L) {
+    const int u = LAST > 0 && L == TO ? LAST : 7 * (L + 2);
+    n += (long long)__float2int_rn(f[L][j] * __uint_as_float((uint32_t)(127 + u) << 23)) * (1ll << (LSB - u));
+  }
+  return n;
 }
 
 // slice width: the level-0 sum over K of 2 products of |a| <= 2^b stays below 2^24

@@ -258,7 +258,7 @@ void launch_site_tc(const Tables& T, const SiteWork* work, int n_work, ZGemmItem
   if (n_work <= 0) return;
   k_site_tc_plan<<<(n_work + 127) / 128, 128, 0, st>>>(T, work, n_work, items);
   k_site_tc_gather<<<dim3(gx, n_work), 256, 0, st>>>(T, work, n_work, items);
-  launch_zgemm(items, n_work, tile_cap, m_cap_max, n_cap_max, T.status, st);
+  launch_zgemm(items, n_work, tile_cap, m_cap_max, n_cap_max, T.status, st, /*k_cap_max=*/n_cap_max);    // K, N: 4 kappa
   k_site_tc_scatter<<<dim3(gx, n_work), 256, 0, st>>>(T, work, n_work, items);
 }
 

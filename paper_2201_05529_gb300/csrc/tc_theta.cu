@@ -317,7 +317,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_theta(Tables T, const Bond
       bool ok = true;
       uint32_t loaded = g, waited = g, committed = 0;
       bool any_commit = false;
-      bool init[4] = {false, false, false, false};
       // prologue: the first STAGES - 1 steps (their stages were freed by the previous tile's end)
       for (int ks = 0; ks < n_ks && ks < STAGES - 1; ++ks) {
         load(ks, g + ks);
@@ -331,24 +330,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_theta(Tables T, const Bond
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const unsigned char* sa = smem + (gg % STAGES) * STAGE;
         const unsigned char* sb = sa + A_STAGE;
-#pragma unroll
-        for (int i = 0; i < NS; ++i) {
-#pragma unroll
-          for (int j = 0; j < NS - i; ++j) {
-            const int L = (i + j) < NLEV - 1 ? (i + j) : NLEV - 1;
-            const uint32_t dre = tmem + (2 * L) * TNB, dim = dre + TNB;
-            const uint64_t ar = smem_desc(sa + i * A_PLANE, LBO_A, SBO);
-            const uint64_t ai = smem_desc(sa + (NS + i) * A_PLANE, LBO_A, SBO);
-            const uint64_t br = smem_desc(sb + j * B_PLANE, LBO_B, SBO);
-            const uint64_t bi = smem_desc(sb + (NS + j) * B_PLANE, LBO_B, SBO);
-            // Re += Ar Br - Ai Bi, Im += Ar Bi + Ai Br
-            mma<BF16>(dre, ar, br, idesc, init[L]);
-            mma<BF16>(dre, ai, bi, idesc | NEG_A, true);
-            mma<BF16>(dim, ar, bi, idesc, init[L]);
-            mma<BF16>(dim, ai, br, idesc, true);
-            init[L] = true;
-          }
-        }
+        // Re += Ar Br - Ai Bi, Im += Ar Bi + Ai Br
+        mma_slices<BF16, NS, NLEV, TNB, A_PLANE, B_PLANE>(tmem, smem_desc(sa, LBO_A, SBO), smem_desc(sb, LBO_B, SBO),
+                                                          idesc, ks > 0);
         mma_commit(&bar_empty[gg % STAGES]);
         committed = gg;
         any_commit = true;
