@@ -49,6 +49,33 @@ int hqr_grid_fits(int total_cols_cap, int n_items, int blocks);
 void launch_hqr_grid(const Tables& T, const BondWork* work, int n_work, int blocks, unsigned* sync3,
                      cudaStream_t st);
 
+// blocked QR with the explicit Q (qr_block.cu): panels by clusters, the rest as nine-slice tensor-core products.
+// One QRBlk per matrix: its workspace at capacity m_cap x n_cap (qr_block_bytes lays it out from base; base NULL:
+// the size only); q is written by the call from the live dims
+struct ZGemmItem;
+struct QRBlk {
+  QRItem q;
+  double2 *Wp, *X, *S;
+  unsigned char *TA, *TB, *TA2, *TB2;
+  int m_cap, n_cap;
+};
+struct QRBlkList {
+  QRBlk* blk = nullptr;    // device, n_items
+  ZGemmItem* ops = nullptr;    // device, qr_block_ops(n_items, n_cap)
+  int n_items = 0, m_cap = 1, n_cap = 1;
+  int cluster = 0;         // qr_block_cluster(n_items, m_cap)
+};
+int qr_block_cluster(int n_items, int m_cap);
+size_t qr_block_bytes(int m, int n, QRBlk* B, char* base);
+size_t qr_block_ops(int n_items, int n_cap);
+// the whole factorisation of small matrices, one CTA each (items' live shapes at most m_cap x n_cap)
+int qr_small_fits(int m_cap, int n_cap);
+void launch_qr_small(const QRItem* items, int n_items, int m_cap, int n_cap, int* status, cudaStream_t st);
+// list: the matrices (n_items of them), or NULL: the outer blocks of the layer's bonds (matrix 2 w: B_L of bond w,
+// 2 w + 1: B_R^H)
+void launch_qr_block(const Tables& T, const BondWork* work, const QRItem* list, const QRBlkList& L, int* status,
+                     cudaStream_t st);
+
 // cluster-parallel FP64 bond SVD (jacobi_cluster.cu)
 int jacobi_cluster_size(int want);
 void launch_jacobi_cluster(const BondWork* work, int n_work, int cluster, int max_sweeps, int* status,
