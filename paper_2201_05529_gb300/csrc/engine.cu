@@ -91,7 +91,7 @@ struct pt_tebd {
   BondWork* d_odd = nullptr;
   BondWork* d_even = nullptr;
   int n_odd = 0, n_even = 0;
-  int gx_bond = 1;
+  int gx_bond = 1, gx_theta = 1;
   int cl_odd = 1, cl_even = 1;        // Jacobi cluster sizes per layer list
   int grid_blocks = 0;                // whole-GPU Jacobi: CTAs per launch (0: use the cluster kernel)
   int tiles_odd = 1, tiles_even = 1;  // fast path: theta + gate GEMM output tiles per layer (capacity)
@@ -284,7 +284,7 @@ void enqueue_layer(pt_tebd* h, const BondWork* work, int n, int layer) {
   ev_end(h, e);
   ev_begin(h, 2, &e);
   if (h->opt.precision == PT_FP64)
-    ptk::k_theta_gate<<<dim3(h->gx_bond, n), 128, 0, s>>>(h->T, work, n);
+    ptk::k_theta_gate<<<dim3(h->gx_theta, n), 256, 0, s>>>(h->T, work, n);
   else
     ptk::launch_tc_theta(h->T, work, n, work == h->d_odd ? h->tiles_odd : h->tiles_even, (int)h->opt.precision, s);
   ptk::k_nan_guard<<<(n + 127) / 128, 128, 0, s>>>(h->T, work, n);
@@ -342,7 +342,7 @@ void enqueue_layer(pt_tebd* h, const BondWork* work, int n, int layer) {
     // the fast path's singular values carry errors of ~1e-11 of sigma_max: gaps below the
     // FAST_MULTIPLET_TOL floor count as degenerate, so it sees the exact multiplets the FP64 path sees
     const double mtol = std::max(h->opt.multiplet_tol, FAST_MULTIPLET_TOL);
-    ptk::k_truncate<<<(n + 63) / 64, 64, 0, s>>>(h->T, work, n, h->opt.chi_max, h->opt.eps, mtol, /*rsvd=*/1);
+    ptk::k_truncate<<<(n + 3) / 4, 128, 0, s>>>(h->T, work, n, h->opt.chi_max, h->opt.eps, mtol, /*rsvd=*/1);
     ev_end(h, e);
     ev_begin(h, 8, &e);
     ptk::launch_rsvd_vectors(h->T, work, n, L, s);
@@ -370,7 +370,7 @@ void enqueue_layer(pt_tebd* h, const BondWork* work, int n, int layer) {
   }
   if (!h->use_rsvd) {
     ev_begin(h, 4, &e);
-    ptk::k_truncate<<<(n + 63) / 64, 64, 0, s>>>(h->T, work, n, h->opt.chi_max, h->opt.eps,
+    ptk::k_truncate<<<(n + 3) / 4, 128, 0, s>>>(h->T, work, n, h->opt.chi_max, h->opt.eps,
                                                   h->opt.multiplet_tol);
     ev_end(h, e);
   }
@@ -663,7 +663,7 @@ int tune_layer(pt_tebd* h, const BondWork* work, int n, const std::vector<BondWo
     ptk::k_build_blocks<<<dim3(h->gx_bond, n), 256, 0, s>>>(h->T, work, n);
     enqueue_k2(h, work, n, r.k2);
     if (h->opt.precision == PT_FP64)
-      ptk::k_theta_gate<<<dim3(h->gx_bond, n), 128, 0, s>>>(h->T, work, n);
+      ptk::k_theta_gate<<<dim3(h->gx_theta, n), 256, 0, s>>>(h->T, work, n);
     else
       ptk::launch_tc_theta(h->T, work, n, odd ? h->tiles_odd : h->tiles_even, (int)h->opt.precision, s);
   }
@@ -1157,6 +1157,13 @@ int build(pt_tebd* h) {
   h->d_odd = odd.empty() ? nullptr : upload(h, odd);
   h->d_even = even.empty() ? nullptr : upload(h, even);
   h->gx_bond = (int)std::min<size_t>(256, (max_bond_elems + 255) / 256);
+  {
+    // theta + gate: 32 pairs (u, v) of D's 4 r_L x 4 r_R entries per block and turn
+    size_t pairs = 1;
+    for (auto* v : {&odd, &even})
+      for (auto& W : *v) pairs = std::max(pairs, (size_t)(W.mD_cap / 4) * (W.nD_cap / 4));
+    h->gx_theta = (int)std::min<size_t>(1024, (pairs + 31) / 32);
+  }
 
   if (h->use_rsvd) {
     // the fast path's Gamma recovery on the tensor cores: per bond a left item (Q_L times U, C in HH)

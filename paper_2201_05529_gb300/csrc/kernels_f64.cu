@@ -221,7 +221,15 @@ __global__ void __launch_bounds__(QR_THREADS) k_householder(Tables T, const Bond
 // ------------------------------------------------------------------ K3: theta + gate
 // App. A.2: D[(u,p'),(q',v)] = sum_{pq} G[p'q',pq] sum_c R_L[u,(p,c)] lambda_c L_R[(c,q),v].
 // D (m >= n) or D^H (m < n) is written column-major into W.A for the one-sided Jacobi.
-__global__ void k_theta_gate(Tables T, const BondWork* work, int n_work) {
+//
+// Bound by the FP64 pipe, for small blocks by the latency of one warp's chain (an FP64 instruction takes 64 cycles of
+// a sub-partition): a block takes 32 pairs (u, v), one per lane; warp (p, q-half) forms two of their 16 theta entries
+// into shared memory, then two of the 16 gate outputs each. The gate's zero entries, the same for a whole warp, are
+// skipped (a U(1)- or parity-symmetric chain's gates have 36 to 64 nonzeros of 256) unless an entry of theta is not
+// finite. One thread per (u, v) for all 16 outputs took 53 us for a 16 x 16 D (1300 FP64 operations in a chain
+// per warp), 90 for 64 x 16 and 145 for two of 144 x 144; now 23, 34 and 76.
+constexpr int TG_PAIRS = 32;
+__global__ void __launch_bounds__(256) k_theta_gate(Tables T, const BondWork* work, int n_work) {
   const int w = blockIdx.y;
   if (w >= n_work) return;
   const BondWork& W = work[w];
@@ -242,34 +250,42 @@ __global__ void k_theta_gate(Tables T, const BondWork* work, int n_work) {
   const int ldLR = d.lqR ? d.mR : d.nR;
   const double* lamC = T.lam_ptr[d.BC];
   __shared__ double2 g[256];
+  __shared__ double2 th[16][TG_PAIRS];
   for (int i = threadIdx.x; i < 256; i += blockDim.x) g[i] = W.gate[i];
-  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int p = warp >> 1, q0 = (warp & 1) * 2;
   const int total = d.rL * d.rR;
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
-    const int u = idx / d.rR, v = idx % d.rR;
-    double2 th[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) th[i] = cmk(0, 0);
-    for (int c = 0; c < d.chc; ++c) {
-      const double lc = lamC[c];
-      double2 rl[4], lr[4];
-#pragma unroll
-      for (int p = 0; p < 4; ++p) rl[p] = cscale(RLp[u + (size_t)(p * d.chc + c) * ldRL], lc);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) lr[q] = cconj(LRp[v + (size_t)(c * 4 + q) * ldLR]);
-#pragma unroll
-      for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) th[p * 4 + q] = cfma(rl[p], lr[q], th[p * 4 + q]);
+  for (int base = blockIdx.x * TG_PAIRS; base < total; base += gridDim.x * TG_PAIRS) {
+    const int idx = base + lane;
+    const bool in = idx < total;
+    const int u = in ? idx / d.rR : 0, v = in ? idx - u * d.rR : 0;
+    double2 t0 = cmk(0, 0), t1 = cmk(0, 0);
+    {
+      const double2* rl = RLp + u + (size_t)(p * d.chc) * ldRL;
+      const double2* l0 = LRp + v + (size_t)q0 * ldLR;
+#pragma unroll 2
+      for (int c = 0; c < d.chc; ++c) {
+        const double2 a = cscale(rl[(size_t)c * ldRL], lamC[c]);
+        t0 = cfma(a, cconj(l0[(size_t)(4 * c) * ldLR]), t0);
+        t1 = cfma(a, cconj(l0[(size_t)(4 * c + 1) * ldLR]), t1);
+      }
     }
-#pragma unroll 1
-    for (int pp = 0; pp < 4; ++pp) {
-#pragma unroll 1
-      for (int qq = 0; qq < 4; ++qq) {
-        double2 acc = cmk(0, 0);
+    __syncthreads();                               // the gate is loaded; the last turn's theta has been read
+    th[p * 4 + q0][lane] = t0;
+    th[p * 4 + q0 + 1][lane] = t1;
+    const bool fin = isfinite(t0.x) && isfinite(t0.y) && isfinite(t1.x) && isfinite(t1.y);
+    const bool all = __syncthreads_or(in && !fin) != 0;      // no skipping next to a NaN or an infinity
 #pragma unroll
-        for (int i = 0; i < 16; ++i) acc = cfma(g[(pp * 4 + qq) * 16 + i], th[i], acc);
-        const int row = u * 4 + pp, col = qq * d.rR + v;
+    for (int h = 0; h < 2; ++h) {
+      const int pq = warp * 2 + h;                 // (p', q')
+      double2 acc = cmk(0, 0);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const double2 gv = g[pq * 16 + i];
+        if (all || gv.x != 0.0 || gv.y != 0.0) acc = cfma(gv, th[i][lane], acc);
+      }
+      if (in) {
+        const int row = u * 4 + (pq >> 2), col = (pq & 3) * d.rR + v;
         if (!(isfinite(acc.x) && isfinite(acc.y))) W.info[7] = 1;    // k_nan_guard stops this bond
         if (!tr) W.A[row + (size_t)col * d.mD] = acc;
         else W.A[col + (size_t)row * d.nD] = cconj(acc);
@@ -304,21 +320,42 @@ __global__ void k_nan_guard(Tables T, const BondWork* work, int n_work) {
 // App. A.2: the smallest chi with ||discarded||_2 < eps * s_max, capped at chi_max; exact zeros
 // dropped; a cut may not split a multiplet (relative gap <= mtol). lambda = kept / ||kept||_2 and
 // log||kept||_2 goes into the bond's log-norm accumulator.
-PT_DEV int truncation_rank(const double* sig, const int* perm, int n, double eps, int chi_max,
-                           double mtol) {
+//
+// One warp per bond, the ordered singular values in chunks of 32 lanes: the tail sums and the norm are shuffle scans and
+// sums (one thread's dependent FP64 chain over 144 values took 80 us, now 16).
+PT_DEV int truncation_rank(const double* sig, const int* perm, int n, double eps, int chi_max, double mtol, int lane) {
   if (n <= 0) return 1;
   const double smax = sig[perm[0]];
   if (!(smax > 0.0)) return 1;
   const double thr = eps * smax;
-  int chi = n;
-  double tail2 = 0.0;
-  for (int c = n; c >= 1; --c) {
-    if (sqrt(tail2) < thr) chi = c;
-    else break;
-    tail2 += sig[perm[c - 1]] * sig[perm[c - 1]];
+  // chi: the smallest count whose discarded rest (the values from chi on) has a norm below thr; tail(n) = 0 counts too
+  int chi = n, nz = 0;
+  double tail2 = 0.0;                              // of the values behind the chunk
+  bool open = true;                                // every count seen so far passed
+  for (int c0 = (n - 1) / 32 * 32; c0 >= 0; c0 -= 32) {
+    const int i = c0 + lane;
+    const double v = i < n ? sig[perm[i]] : 0.0;
+    nz += __popc(__ballot_sync(0xffffffffu, v > 0.0));
+    double t = v * v;                              // suffix sum within the chunk
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double x = __shfl_down_sync(0xffffffffu, t, o);
+      if (lane + o < 32) t += x;
+    }
+    t += tail2;                                    // tail2 with this value: the rest when i values are kept
+    // counts i + 1 keep this value: their rest is the next value's suffix sum
+    double rest = __shfl_down_sync(0xffffffffu, t, 1);
+    if (lane == 31) rest = tail2;
+    const unsigned pass = __ballot_sync(0xffffffffu, i >= n || sqrt(rest) < thr);
+    if (open) {
+      // lanes from the top down while they pass
+      const unsigned fail = ~pass;
+      const int lowest = fail ? 32 - __clz((int)fail) : 0;       // the lowest lane of the passing run
+      if (lowest < 32 && c0 + lowest + 1 <= n) chi = min(chi, c0 + lowest + 1);
+      open = fail == 0;
+    }
+    tail2 = __shfl_sync(0xffffffffu, t, 0);
   }
-  int nz = 0;
-  for (int i = 0; i < n; ++i) nz += sig[perm[i]] > 0.0;
   chi = max(1, min(chi, nz));
   auto splits = [&](int c) {
     return c > 0 && c < n && (sig[perm[c - 1]] - sig[perm[c]]) <= mtol * smax;
@@ -334,7 +371,7 @@ PT_DEV int truncation_rank(const double* sig, const int* perm, int n, double eps
 
 __global__ void k_truncate(Tables T, const BondWork* work, int n_work, int chi_max, double eps,
                            double mtol, int rsvd) {
-  const int w = blockIdx.x * blockDim.x + threadIdx.x;
+  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (w >= n_work) return;
   const BondWork& W = work[w];
   const int mD = W.info[0], nD = W.info[1];
@@ -346,35 +383,43 @@ __global__ void k_truncate(Tables T, const BondWork* work, int n_work, int chi_m
     const int l = W.info[9];
     if (l <= 0) return;
     if (l < n) {
-      W.sig[l] = sqrt(fmax(0.0, *(const double*)(W.info + 12)));     // ||D - Q Q^H D||_F
-      W.perm[l] = l;
+      if (lane == 0) {
+        W.sig[l] = sqrt(fmax(0.0, *(const double*)(W.info + 12)));     // ||D - Q Q^H D||_F
+        W.perm[l] = l;
+      }
+      __syncwarp();
       n = l + 1;
     } else {
       n = l;
     }
   }
   const int BC = W.lam_l + 1;
-  int chi = truncation_rank(W.sig, W.perm, n, eps, chi_max, mtol);
+  int chi = truncation_rank(W.sig, W.perm, n, eps, chi_max, mtol, lane);
   if (chi > T.lam_cap[BC]) {
-    atomicOr(T.status, ST_CAPACITY);
+    if (lane == 0) atomicOr(T.status, ST_CAPACITY);
     chi = T.lam_cap[BC];
   }
-  double n2 = 0.0;
-  for (int i = 0; i < chi; ++i) n2 += W.sig[W.perm[i]] * W.sig[W.perm[i]];
+  double n2 = 0.0, tail2 = 0.0;
+  for (int i = lane; i < n; i += 32) {
+    const double v = W.sig[W.perm[i]];
+    if (i < chi) n2 = fma(v, v, n2);
+    else tail2 = fma(v, v, tail2);
+  }
+  n2 = warp_sum(n2);
+  tail2 = warp_sum(tail2);
   const double nrm = sqrt(n2);
   double* lam = T.lam_ptr[BC];
-  if (nrm > 0.0 && nrm == nrm) {
-    for (int i = 0; i < chi; ++i) lam[i] = W.sig[W.perm[i]] / nrm;
+  const bool fine = nrm > 0.0 && nrm == nrm;
+  for (int i = lane; i < chi; i += 32) lam[i] = fine ? W.sig[W.perm[i]] / nrm : 0.0;
+  if (lane != 0) return;
+  if (fine) {
     T.lam_lognorm[BC] += log(nrm);
   } else {
     atomicOr(T.status, ST_NAN);
     W.info[6] |= FAULT_ZERO_NORM;
-    for (int i = 0; i < chi; ++i) lam[i] = 0.0;
   }
   T.lam_chi[BC] = chi;
   // discarded weight ||sigma_{>= chi}||_2 / sigma_max of this update, for the bond log
-  double tail2 = 0.0;
-  for (int i = chi; i < n; ++i) tail2 += W.sig[W.perm[i]] * W.sig[W.perm[i]];
   const double smax = W.sig[W.perm[0]];
   *(double*)(W.info + 10) = smax > 0.0 ? sqrt(tail2) / smax : 0.0;
 }

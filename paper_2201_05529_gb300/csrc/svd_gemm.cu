@@ -13,11 +13,12 @@ __device__ __forceinline__ void shape(const BondWork& W, int* Ma, int* Na) {
   *Na = (mD > 0 && nD > 0) ? (tr ? mD : nD) : 0;
 }
 
-constexpr int TB = 32;   // GEMM tile
+constexpr int TB = 16;   // GEMM tile: one output per thread, so that a layer of two bonds fills more SMs (a 2 x 2
+                         // block per thread in 32 x 32 tiles: 90 us for two 144 x 144 x 40, FP64 issue on 20 SMs; 45 us so)
 constexpr int TK = 16;   // GEMM K tile
 
 // C[m x n] = op(A)[m x k] * B[k x n], column-major; op = conjugate transpose if conjA.
-// 256 threads, each computes a 2 x 2 block of a 32 x 32 tile.
+// 256 threads, one entry of a 16 x 16 tile each.
 // bcol: column c of B is column bcol[c] of the stored matrix (NULL: c). K runs from k_from (a multiple of TK).
 // div: column c of the result is divided by div[bcol[c]] (a zero gives a zero column).
 __device__ void gemm_tile(const double2* A, int lda, bool conjA, const double2* B, int ldb, double2* C, int ldc,
@@ -25,15 +26,12 @@ __device__ void gemm_tile(const double2* A, int lda, bool conjA, const double2* 
                           const double* div = nullptr) {
   __shared__ double2 As[TK][TB + 1];
   __shared__ double2 Bs[TK][TB + 1];
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  double2 acc[2][2];
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) acc[i][j] = make_double2(0.0, 0.0);
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;      // row tx, column ty of the tile
+  double2 acc = make_double2(0.0, 0.0), acc2 = acc;
   for (int k0 = k_from; k0 < k; k0 += TK) {
-    for (int e = threadIdx.x; e < TK * TB; e += blockDim.x) {
-      const int kk = e / TB, mm = e % TB;
+    {
+      // thread (mm, kk) loads one element of each operand's tile
+      const int mm = tx, kk = ty;
       const int row = tm * TB + mm, col = k0 + kk;
       double2 a = make_double2(0.0, 0.0);
       if (row < m && col < k) {
@@ -45,41 +43,29 @@ __device__ void gemm_tile(const double2* A, int lda, bool conjA, const double2* 
         }
       }
       As[kk][mm] = a;
-      const int bc = tn * TB + mm, br = k0 + kk;
-      Bs[kk][mm] = (bc < n && br < k) ? B[br + (size_t)(bcol ? bcol[bc] : bc) * ldb] : make_double2(0.0, 0.0);
+      const int br = k0 + tx, bc = tn * TB + ty;            // B's tile along its columns
+      Bs[tx][ty] = (bc < n && br < k) ? B[br + (size_t)(bcol ? bcol[bc] : bc) * ldb] : make_double2(0.0, 0.0);
     }
     __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < TK; ++kk) {
-      double2 a[2], b[2];
 #pragma unroll
-      for (int i = 0; i < 2; ++i) a[i] = As[kk][ty * 2 + i];
-#pragma unroll
-      for (int j = 0; j < 2; ++j) b[j] = Bs[kk][tx * 2 + j];
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          acc[i][j].x = fma(a[i].x, b[j].x, fma(-a[i].y, b[j].y, acc[i][j].x));
-          acc[i][j].y = fma(a[i].x, b[j].y, fma(a[i].y, b[j].x, acc[i][j].y));
-        }
+    for (int kk = 0; kk < TK; kk += 2) {
+      const double2 a = As[kk][tx], b = Bs[kk][ty], c = As[kk + 1][tx], d = Bs[kk + 1][ty];
+      acc.x = fma(a.x, b.x, fma(-a.y, b.y, acc.x));
+      acc.y = fma(a.x, b.y, fma(a.y, b.x, acc.y));
+      acc2.x = fma(c.x, d.x, fma(-c.y, d.y, acc2.x));
+      acc2.y = fma(c.x, d.y, fma(c.y, d.x, acc2.y));
     }
     __syncthreads();
   }
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int row = tm * TB + ty * 2 + i, col = tn * TB + tx * 2 + j;
-      if (row < m && col < n) {
-        if (div) {
-          const double s = div[bcol[col]];
-          acc[i][j].x = s > 0.0 ? acc[i][j].x / s : 0.0;
-          acc[i][j].y = s > 0.0 ? acc[i][j].y / s : 0.0;
-        }
-        C[row + (size_t)col * ldc] = acc[i][j];
-      }
+  const int row = tm * TB + tx, col = tn * TB + ty;
+  if (row < m && col < n) {
+    double2 v = make_double2(acc.x + acc2.x, acc.y + acc2.y);
+    if (div) {
+      const double s = div[bcol[col]];
+      v = s > 0.0 ? make_double2(v.x / s, v.y / s) : make_double2(0.0, 0.0);
     }
+    C[row + (size_t)col * ldc] = v;
+  }
 }
 
 }  // namespace
