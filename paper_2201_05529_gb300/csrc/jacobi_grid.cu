@@ -6,8 +6,11 @@
 // barriers therefore cost as much as the arithmetic on columns of a few hundred rows. So:
 //   * the columns are grouped in blocks of b and a round-robin tournament runs over the blocks: one CTA holds
 //     a pair of blocks (2 b columns) in shared memory and runs its b x b cross pairs (in the first round of a
-//     sweep also the pairs inside the blocks) in sub-rounds of b disjoint pairs, so a sweep of n columns
-//     has n / b - 1 grid barriers;
+//     sweep also the pairs inside the blocks) in sub-rounds of b disjoint pairs;
+//   * a task waits for its two blocks only: each block carries the number of rounds it has been through (in perm, free
+//     until the end), stored after its columns and polled by the next task that needs it. A grid barrier per round
+//     instead, with its column transfers, took 8000 of the 14000 cycles of a round with b = 2; grid barriers remain
+//     at the end of a sweep;
 //   * the scalars of a sub-round's pairs are computed by the lanes of one extra warp at the same time. Columns
 //     carry a real scale (column = d x stored column, q = d^2), so that neither a square root nor a division is
 //     needed: with rho = tan / |gamma| (in FP32 and integers: a rotation by an angle that is 1e-7 off is still
@@ -20,9 +23,10 @@
 //   * b is chosen on the device from the live dims by a cost model of these terms (choose_block), and CTAs that
 //     no round can use leave at once, so small layers pay for small barriers.
 // Before (one 512-thread CTA per SM, b = 2, columns in L2, each pair's scalars on one lane in FP64 with two sqrt /
-// rsqrt chains, 5800 cycles; now 1900), start of the calls that run it: two 256 x 256 SVDs 113 ms (clusters) -> 33,
-// the five-site chain's first eight steps 227 -> 189 ms, 16 chains' first four steps 309 -> 196 ms, the 21-site
-// chain's first four steps on the tensor-core path 905 -> 651 ms.
+// rsqrt chains, 5800 cycles; now 1900) -> with a grid barrier per round -> with the blocks' own counters and a pair's two
+// norms, scales and factors on two lanes: two 256 x 256 SVDs 112 ms (clusters) -> 31.6 -> 27.9, the three-site chain's
+// first eight steps 51.8 -> 34.6 -> 33.5 ms, the five-site chain's 219 -> 180 -> 150 ms, the 21-site chain's first four
+// on the tensor-core path 905 -> 651 (451 with the other kernels' later changes) -> 438 ms.
 //
 // Sums are combined in a fixed order, so results are bitwise reproducible. Every barrier wait has a time
 // limit: on expiry the kernel records ST_TIMEOUT, raises an abort flag that releases every other CTA, and
@@ -94,16 +98,34 @@ __device__ __forceinline__ float significand(double x, int* e) {
   return __int_as_float(0x3f800000 | (hi & 0xfffff) << 3 | (int)((unsigned)__double2loint(x) >> 29));
 }
 
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // f 2^k, f in [1, 2), 0 for k below -60 (k <= 1)
 __device__ __forceinline__ float scale_pow2(float f, int k) {
   return k < -60 ? 0.f : __int_as_float(__float_as_int(f) + (k << 23));
+}
+
+// shared-memory tables of a launch over n items
+__host__ __device__ constexpr int header_bytes(int n) { return (48 * n + 4 * (4 * n + 1) + 15) & ~15; }
+
+__device__ __forceinline__ int load_acquire(const int* p) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void store_relaxed(int* p, int v) {
+  asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 constexpr int MIN_SCALE_HI = (1023 - 64) << 20;    // below 2^-64 a squared scale is multiplied into its column
 
 // columns per block: the b in {1, 2, 4, 8} that fits cols_max columns and whose sweep is shortest by the cost of
 // its terms in cycles: per sub-round the scalars and reductions (2500 cycles, shared by the tasks of an SM) and 19
-// cycles per FP64 warp instruction of the SM's tasks; per round the transfer of a task's columns and the barrier.
+// cycles per FP64 warp instruction of the SM's tasks; per round the transfer of a task's columns and its waits.
 // Costs estimated from the measured FP64 issue rate and barrier; the choice only moves a few percent around them.
 // One warp computes it; every lane gets the result.
 __device__ int choose_block(const int* s_Na, const int* s_Ma, int n_work, int slots, int sms, int cols_max,
@@ -111,10 +133,11 @@ __device__ int choose_block(const int* s_Na, const int* s_Ma, int n_work, int sl
   int best = 1;
   float best_t = 3e38f;
   for (int b = 1; b <= JB && 2 * b <= cols_max; b <<= 1) {
-    int tasks = 0, rounds = 0, rows = 0;
+    int tasks = 0, rounds = 0, rows = 0, most_nb = 0;
     for (int w = lane; w < n_work; w += 32) {
       if (s_Na[w] < 2) continue;
       const int nb = (s_Na[w] + b - 1) / b, nbp = nb + (nb & 1);
+      most_nb = max(most_nb, nb);
       tasks += nbp / 2;
       rounds = max(rounds, nbp - 1);
       // FP64 operations per pair: 4 per row for the inner product, 8 per row (and row of V) for the rotation
@@ -123,12 +146,14 @@ __device__ int choose_block(const int* s_Na, const int* s_Ma, int n_work, int sl
     tasks = __reduce_add_sync(0xffffffffu, tasks);
     rounds = __reduce_max_sync(0xffffffffu, rounds);
     rows = __reduce_max_sync(0xffffffffu, rows);
+    most_nb = __reduce_max_sync(0xffffffffu, most_nb);
     if (tasks == 0) return 1;
     const float per_sm = (float)((tasks + sms - 1) / sms), waves = (float)((tasks + slots - 1) / slots);
     const float fp = 19.f * b * (float)((rows + 31) / 32);
     const float sub = fmaxf(waves * 2500.f + fp, per_sm * fp + 1500.f);
     const float move = 1000.f + per_sm * b * (float)rows * 0.1f;
-    const float t = rounds * ((float)b * sub + move + (tasks > 1 ? 2500.f : 0.f)) + (b - 1) * sub;
+    // one block only: no cross pairs
+    const float t = most_nb < 2 ? (b - 1) * sub : rounds * ((float)b * sub + move + 2500.f) + (b - 1) * sub;
     if (t < best_t) {
       best_t = t;
       best = b;
@@ -158,7 +183,7 @@ __global__ void __launch_bounds__(CT, 1)
     int flag[JB];                          // rotate
     int redo[JB];                          // recompute the pair's norms from its columns
     int rotc[2 * JB];                      // the column changed in this task
-    int cnt, renorm[2];
+    int cnt, renorm[2], lost[2];
   };
   __shared__ Slot s_slot[JG];
   __shared__ int s_b, s_rounds, s_fit, s_most, s_cols;
@@ -169,11 +194,16 @@ __global__ void __launch_bounds__(CT, 1)
     return;
   }
   double* s_fro = (double*)s_raw;                    // ||A||_F^2 per item
-  int* s_Na = (int*)(s_fro + n_work);                // columns that are rotated
+  double2** s_A = (double2**)(s_fro + n_work);       // the items' buffers (the work list itself is behind two loads)
+  double2** s_V = s_A + n_work;
+  double** s_aux = (double**)(s_V + n_work);
+  double** s_sig = s_aux + n_work;
+  int** s_ver = (int**)(s_sig + n_work);
+  int* s_Na = (int*)(s_ver + n_work);                // columns that are rotated
   int* s_Ma = s_Na + n_work;                         // rows
-  int* s_off = s_Ma + n_work;                        // [n_work + 1] prefix of the round's tasks
+  int* s_off = s_Ma + n_work;                        // [n_work + 1] prefix of the sweep's tasks per round
   int* s_act = s_off + n_work + 1;
-  const int hdr = (8 * n_work + 4 * (4 * n_work + 1) + 15) & ~15;
+  const int hdr = header_bytes(n_work);
   const int slot_bytes = (dyn_bytes - hdr) / n_grp & ~15;
   double2* s_col = (double2*)(s_raw + hdr + (size_t)grp * slot_bytes);
   for (int w = ctid; w < n_work; w += CT) {
@@ -185,6 +215,11 @@ __global__ void __launch_bounds__(CT, 1)
     s_Na[w] = kq;
     s_Ma[w] = on_b == 1 ? Na : (on_b == 2 ? kq : Ma);
     s_act[w] = kq >= 2;
+    s_A[w] = mat_of(work[w], on_b);
+    s_V[w] = work[w].V;
+    s_aux[w] = work[w].aux;
+    s_sig[w] = work[w].sig;
+    s_ver[w] = work[w].perm;
   }
   __syncthreads();
   if (cwid == 0) {
@@ -255,6 +290,7 @@ __global__ void __launch_bounds__(CT, 1)
         if (lane == 0) {
           __stcg(W.aux + c, s2);
           __stcg(W.sig + c, 1.0);
+          __stcg(W.perm + c, 0);           // rounds of block c (blocks are fewer than columns)
         }
       }
       base = (base + Na) % ngwarp;
@@ -268,17 +304,33 @@ __global__ void __launch_bounds__(CT, 1)
     acc = wsum(acc);
     if (lane == 0) s_fro[w] = acc;
   }
-  // the rounds of the next sweep: the longest tournament among the active items (0: all converged)
+  // the rounds of the next sweep, the longest tournament among the active items (0: all converged), and the prefix of
+  // the active items' task counts
   auto set_rounds = [&]() {
     if (cwid != 0) return;
-    int rounds = 0;
-    for (int w = lane; w < n_work; w += 32)
-      if (s_act[w]) {
+    int rounds = 0, run = 0;
+    for (int w0 = 0; w0 < n_work; w0 += 32) {
+      const int w = w0 + lane;
+      int v = 0;
+      if (w < n_work && s_act[w]) {
         const int nb = (s_Na[w] + b - 1) / b, nbp = nb + (nb & 1);
         rounds = max(rounds, nbp - 1);
+        v = nbp / 2;
       }
+      int inc = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+      }
+      if (w < n_work) s_off[w] = run + inc - v;
+      run += __shfl_sync(0xffffffffu, inc, 31);
+    }
     rounds = __reduce_max_sync(0xffffffffu, rounds);
-    if (lane == 0) s_rounds = rounds;
+    if (lane == 0) {
+      s_off[n_work] = run;
+      s_rounds = rounds;
+    }
   };
   set_rounds();
   __syncthreads();
@@ -287,30 +339,9 @@ __global__ void __launch_bounds__(CT, 1)
     const int par = sweep & 1, rounds = s_rounds;
     if (blockIdx.x == 0)
       for (int w = ctid; w < n_work; w += CT) work[w].info[4 + (par ^ 1)] = 0;
-    for (int round = 0; round < rounds; ++round) {
-      // prefix of the active items' task counts (warp 0)
-      if (cwid == 0) {
-        int run = 0;
-        for (int w0 = 0; w0 < n_work; w0 += 32) {
-          const int w = w0 + lane;
-          int v = 0;
-          if (w < n_work && s_act[w]) {
-            const int nb = (s_Na[w] + b - 1) / b, nbp = nb + (nb & 1);
-            if (round < nbp - 1) v = nbp / 2;
-          }
-          int inc = v;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += t;
-          }
-          if (w < n_work) s_off[w] = run + inc - v;
-          run += __shfl_sync(0xffffffffu, inc, 31);
-        }
-        if (lane == 0) s_off[n_work] = run;
-      }
-      __syncthreads();
-      const int total = s_off[n_work];
+    const int total = s_off[n_work];
+    bool gone = false;                     // a wait ran out (this slot or another CTA): to the barrier, which fails
+    for (int round = 0; round < rounds && !gone; ++round) {
       for (int t = grp < n_grp ? grp * G + (int)blockIdx.x : total; t < total; t += n_grp * G) {
         int lo = 0, hi = n_work - 1;
         while (lo < hi) {
@@ -319,22 +350,47 @@ __global__ void __launch_bounds__(CT, 1)
           else hi = mid - 1;
         }
         const int w = lo, q = t - s_off[w];
-        const BondWork& W = work[w];
         const int Ma = s_Ma[w], Na = s_Na[w], Vr = with_v ? Na : 0, ld = Ma + Vr;
         const int nb = (Na + b - 1) / b, nbp = nb + (nb & 1);
+        if (round >= nbp - 1) continue;    // this item's tournament is over
         int bi, bj;
         if (q == 0) { bi = nbp - 1; bj = round; }
         else { bi = (round + q) % (nbp - 1); bj = (round - q + nbp - 1) % (nbp - 1); }
-        double2* A = mat_of(W, on_b);
+        double2 *A = s_A[w], *V = s_V[w];
+        double *aux = s_aux[w], *sig = s_sig[w];
         // local column c: global column of block bi (c < b) or bj; -1 beyond the matrix
         auto gcol = [&](int c) {
           const int g = (c < b ? bi * b + c : bj * b + c - b);
           return g < Na ? g : -1;
         };
+        // both blocks have been through the rounds before this one
+        const int need = sweep * (nbp - 1) + round;
+        int* ver = s_ver[w];
+        if (wid == JW && lane < 2) {
+          const int blk = lane == 0 ? bi : bj;
+          bool lost = false;
+          if (blk < nb && need > 0) {
+            const long long t0 = clock64();
+            for (int it = 1; load_acquire(ver + blk) < need; ++it) {
+              if ((it & 63) != 0) continue;
+              if (*(volatile int*)gs.abort) lost = true;
+              else if (clock64() - t0 > gs.limit) {
+                atomicOr(status, ST_TIMEOUT);
+                atomicExch(gs.abort, 1);
+                lost = true;
+              }
+              if (lost) break;
+            }
+          }
+          S.lost[lane] = lost;
+        }
+        slot_sync(grp);
+        gone = S.lost[0] || S.lost[1];
+        if (gone) break;
         if (tid < 2 * b) {
           const int g = gcol(tid);
-          S.nrm[tid] = g >= 0 ? __ldcg(W.aux + g) : 0.0;
-          S.q[tid] = g >= 0 ? __ldcg(W.sig + g) : 1.0;
+          S.nrm[tid] = g >= 0 ? __ldcg(aux + g) : 0.0;
+          S.q[tid] = g >= 0 ? __ldcg(sig + g) : 1.0;
           S.rotc[tid] = 0;
         }
         if (tid == 0) S.cnt = 0;
@@ -345,7 +401,7 @@ __global__ void __launch_bounds__(CT, 1)
             const int g = gcol(c);
             if (g < 0) continue;
             const double2* a = A + (size_t)g * Ma;
-            const double2* v = W.V + (size_t)g * Na - Ma;
+            const double2* v = V + (size_t)g * Na - Ma;
             double2* dst = s_col + (size_t)c * ld;
 #pragma unroll 4
             for (int r = rc0; r < ld; r += 32 * wpc) cp16(dst + r, (r < Ma ? a : v) + r);
@@ -405,7 +461,8 @@ __global__ void __launch_bounds__(CT, 1)
             const int pp = min(lane >> (1 + lw), b - 1);
             int i, j;
             pair_of(pp, &i, &j);
-            const bool lead = (lane & 1) == 0 && ((lane >> 1) & (wpp - 1)) == 0 && lane < 2 * JW;
+            const bool first = ((lane >> 1) & (wpp - 1)) == 0 && lane < 2 * JW;
+            const bool lead = first && (lane & 1) == 0, lead_odd = first && (lane & 1) != 0;
             const double al = S.nrm[i], be = S.nrm[j], qx = S.q[i], qy = S.q[j];
             const double h = be - al, qq = qx * qy;
             int ea, eb, eh;
@@ -415,6 +472,8 @@ __global__ void __launch_bounds__(CT, 1)
             bool go = gcol(i) >= 0 && gcol(j) >= 0 &&
                       min(__double_as_longlong(al), __double_as_longlong(be)) > max(fl2, 0x0010000000000000ll - 1);
             if (lane == 0) S.renorm[sr & 1] = 0;
+            // computed here, while the column warps form the inner products, not after the barrier
+            asm volatile("" ::"d"(h), "d"(qq), "f"(am), "f"(bm), "f"(hm), "r"(ea + eb + et), "r"(eh), "r"((int)go));
             slot_sync(grp);
             double v = lane < 2 * JW ? S.part[lane >> 1][lane & 1] : 0.0;
             for (int o = 2; o < 2 * wpp; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -429,43 +488,41 @@ __global__ void __launch_bounds__(CT, 1)
             // rho = 2 sign(h) / (|h| + sqrt(h^2 + 4 |gamma|^2)), h = beta - alpha, on values scaled by 2^-E
             const int E = max(eh, (eg + 1) >> 1);
             const float hf = eh > -1023 ? scale_pow2(hm, eh - E) : 0.f, gf = scale_pow2(gs, eg - 2 * E);
-            const float rf = __fdividef(2.0f, hf + __fsqrt_rn(fmaf(hf, hf, 4.0f * gf)));
+            const float rf = __fdividef(2.0f, hf + sqrt_approx(fmaf(hf, hf, 4.0f * gf)));
             const int rb = __float_as_int(rf);
             const double rho = __hiloint2double(((rb >> 3) + ((1023 - 127 - E) << 20)) | (__double2hiint(h) & 0x80000000),
                                                 rb << 29);
-            const double ry = rho * qy, rx = rho * qx;
-            if (lead) {
+            // the even lanes form mu and then column i's norm and scale, the odd lanes nu and column j's
+            const bool odd = lane & 1;
+            const double own = odd ? qy : qx, f = rho * (odd ? qx : qy);
+            if (lead || lead_odd) {
               if (go) {
-                S.rot[pp][0] = ry * gr;
-                S.rot[pp][1] = ry * gm;
-                S.rot[pp][2] = rx * gr;
-                S.rot[pp][3] = rx * gm;
+                S.rot[pp][odd ? 2 : 0] = f * gr;
+                S.rot[pp][odd ? 3 : 1] = f * gm;
               }
-              S.flag[pp] = go;
+              if (lead) S.flag[pp] = go;
             }
             slot_sync(grp);
             // while the columns rotate: the squared norms after a rotation by any angle, unless they cancel below a
             // quarter (then recomputed from the columns), and the squared scales times cos^2
-            if (lead) {
-              int redo = 0;
-              if (go) {
-                const double rg = rho * g2, t2 = rho * rg, a1 = 1.0 + t2;
-                const double y0 = (double)(1.0f / (float)a1), e0 = fma(-a1, y0, 1.0);
-                const double c2 = fma(y0, fma(e0, e0, e0), y0);      // an FP32 seed, a third-order step: 1 / a1
-                const double al2 = c2 * fma(t2, be, fma(-2.0, rg, al)), be2 = c2 * fma(t2, al, fma(2.0, rg, be));
-                // a quarter of alpha: two less in the exponent field
-                redo = __double2hiint(al2) < __double2hiint(al) - (2 << 20) ||
-                       __double2hiint(be2) < __double2hiint(be) - (2 << 20);
-                if (redo) S.renorm[sr & 1] = 1;
-                S.nrm[i] = al2;
-                S.nrm[j] = be2;
-                S.q[i] = qx * c2;
-                S.q[j] = qy * c2;
-                S.rotc[i] = S.rotc[j] = 1;
-                atomicAdd(&S.cnt, 1);
-              }
-              S.redo[pp] = redo;
+            int redo = 0;
+            if ((lead || lead_odd) && go) {
+              const double rg = rho * g2, t2 = rho * rg, a1 = 1.0 + t2;
+              const double y0 = (double)(1.0f / (float)a1), e0 = fma(-a1, y0, 1.0);
+              const double c2 = fma(y0, fma(e0, e0, e0), y0);        // an FP32 seed, a third-order step: 1 / a1
+              const double mine = odd ? be : al, his = odd ? al : be;
+              const double nrm = c2 * fma(t2, his, fma(odd ? 2.0 : -2.0, rg, mine));
+              // a quarter: two less in the exponent field
+              redo = __double2hiint(nrm) < __double2hiint(mine) - (2 << 20);
+              const int at = odd ? j : i;
+              S.nrm[at] = nrm;
+              S.q[at] = own * c2;
+              S.rotc[at] = 1;
+              if (lead) atomicAdd(&S.cnt, 1);
             }
+            redo |= __shfl_xor_sync(0xffffffffu, redo, 1);
+            if (first && redo) S.renorm[sr & 1] = 1;
+            if (lead) S.redo[pp] = redo;
           }
           if (wid < JW) slot_sync(grp);
           if (wid < JW && S.flag[p]) {
@@ -486,7 +543,7 @@ __global__ void __launch_bounds__(CT, 1)
             } else {
               for (int r = r0; r < Ma; r += step) rotate(x, y, r);
               for (int r = r0; r < Vr; r += step)
-                rotate(W.V + (size_t)gcol(li) * Na, W.V + (size_t)gcol(lj) * Na, r);
+                rotate(V + (size_t)gcol(li) * Na, V + (size_t)gcol(lj) * Na, r);
             }
           }
           slot_sync(grp);
@@ -521,7 +578,7 @@ __global__ void __launch_bounds__(CT, 1)
           if (g < 0 || !S.rotc[c]) continue;
           const bool fold = __double2hiint(S.q[c]) < MIN_SCALE_HI;
           double2* a = A + (size_t)g * Ma;
-          double2* v = W.V + (size_t)g * Na - Ma;
+          double2* v = V + (size_t)g * Na - Ma;
           const double2* from = s_col + (size_t)c * ld;
           if (SM && !fold) {
 #pragma unroll 4
@@ -539,14 +596,19 @@ __global__ void __launch_bounds__(CT, 1)
         }
         if (tid < 2 * b && S.rotc[tid]) {
           const int g = gcol(tid);
-          __stcg(W.aux + g, S.nrm[tid]);
-          __stcg(W.sig + g, __double2hiint(S.q[tid]) < MIN_SCALE_HI ? 1.0 : S.q[tid]);
+          __stcg(aux + g, S.nrm[tid]);
+          __stcg(sig + g, __double2hiint(S.q[tid]) < MIN_SCALE_HI ? 1.0 : S.q[tid]);
         }
-        if (tid == 0 && S.cnt) atomicAdd(W.info + 4 + par, S.cnt);
         slot_sync(grp);
+        if (tid == 0) {
+          if (S.cnt) atomicAdd(work[w].info + 4 + par, S.cnt);
+          __threadfence();                 // the slot's columns, norms and scales (thread 0 has them through the barrier)
+          if (bi < nb) store_relaxed(ver + bi, need + 1);
+          if (bj < nb) store_relaxed(ver + bj, need + 1);
+        }
       }
-      if (!barrier()) return;
     }
+    if (!barrier()) return;                // every rotation of the sweep has been counted
     // sweep done: retire converged items (every CTA reads the same counters)
     for (int w = ctid; w < n_work; w += CT)
       if (s_act[w] && *(volatile int*)(work[w].info + 4 + par) == 0) {
@@ -641,7 +703,7 @@ namespace {
 // task slots it holds (two if each has room for b = 2); the header alone: the columns stay in L2
 int jacobi_smem(int n_work, int rows, int* n_grp) {
   constexpr long long MAX = 220 * 1024;          // 227 KB per SM less the static arrays
-  const int hdr = (8 * n_work + 4 * (4 * n_work + 1) + 15) & ~15;
+  const int hdr = header_bytes(n_work);
   const long long col = 16LL * rows;
   *n_grp = JG;
   if (hdr + JG * 4 * col <= MAX) return (int)std::min(MAX, hdr + JG * 2 * JB * col);
@@ -657,6 +719,7 @@ int jacobi_grid_blocks() {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaFuncSetAttribute(k_jacobi_grid<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+  cudaFuncSetAttribute(k_jacobi_grid<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, header_bytes(MAX_ITEMS));
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_jacobi_grid<true>, CT, 220 * 1024);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_jacobi_grid<false>, CT, 32 * 1024);
   cudaGetLastError();
