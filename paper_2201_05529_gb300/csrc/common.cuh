@@ -106,6 +106,7 @@ struct BondWork {
   double* sig;             // [max(k_cap, mR_cap)] singular values (unsorted); B_R^H reflector scalars
   double* aux;             // [max(k_cap, nL_cap)] column norms scratch; B_L reflector scalars
   int* perm;               // [k_cap] perm[rank] = column
+  int* rounds;             // [k_cap] the Jacobi's rounds per block of columns
   void* TA;                // fast path: packed split planes of the theta operands (tc_theta.cu)
   void* TB;
   double2* G64;            // [k_cap^2] B = R^H of the pivoted QR; fast path: the range finder's l x l factor

@@ -1006,10 +1006,13 @@ int build(pt_tebd* h) {
       W.sig = (double*)h->dalloc(sizeof(double) * sa);
       W.aux = (double*)h->dalloc(sizeof(double) * sa);
       W.perm = (int*)h->dalloc(sizeof(int) * W.k_cap);
+      W.rounds = (int*)h->dalloc(sizeof(int) * W.k_cap);
       W.info = (int*)h->dalloc(sizeof(int) * 16);
-      if (!W.QL || !W.RL || !W.QR || !W.LR || !W.HH || !W.A || !W.V || !W.sig || !W.aux || !W.perm || !W.info)
+      if (!W.QL || !W.RL || !W.QR || !W.LR || !W.HH || !W.A || !W.V || !W.sig || !W.aux || !W.perm || !W.rounds ||
+          !W.info)
         return h->fail(PT_ERR_OOM, "bond scratch");
       cudaMemsetAsync(W.info, 0, sizeof(int) * 16, h->stream);
+      cudaMemsetAsync(W.perm, 0, sizeof(int) * W.k_cap, h->stream);      // column indices from the start
       if (h->opt.precision != PT_FP64) {
         W.TA = h->dalloc(ptk::tc_pack_bytes(W, 0, (int)h->opt.precision));
         W.TB = h->dalloc(ptk::tc_pack_bytes(W, 1, (int)h->opt.precision));
@@ -1935,6 +1938,7 @@ int pt_svd_f64(const double* A, int m, int n, int batch, double* sigma, double* 
     W.V = wV + b * sV;
     W.sig = sig + (size_t)b * Na;
     W.perm = perm + (size_t)b * Na;
+    W.rounds = (int*)(sigma + (size_t)b * Na);        // free until the results are written
     W.info = info + 8 * (size_t)b;
     W.aux = (double*)(base + offs[7]) + (size_t)b * Na;
     W.mD_cap = m;
@@ -1948,6 +1952,7 @@ int pt_svd_f64(const double* A, int m, int n, int batch, double* sigma, double* 
   cudaMemcpyAsync(items, hw.data(), sizeof(BondWork) * batch, cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(info, hinfo.data(), sizeof(int) * hinfo.size(), cudaMemcpyHostToDevice, st);
   cudaMemsetAsync(status, 0, sizeof(int), st);
+  cudaMemsetAsync(perm, 0, sizeof(int) * (size_t)Na * batch, st);      // column indices also if the Jacobi gives up early
   const int gx = (int)std::min<size_t>(256, ((size_t)m * n + 255) / 256);
   ptk::k_svd_load<<<dim3(gx, batch), 256, 0, st>>>((const double2*)A, m, n, batch, wA, sA);
   ptk::launch_svd_jacobi(items, batch, Ma, Na, max_sweeps, status, (unsigned*)(status + 8), st);
@@ -1979,6 +1984,14 @@ int pt_svd_f64(const double* A, int m, int n, int batch, double* sigma, double* 
   if (hs & ST_NAN) {
     g_err = "pt_svd_f64: NaN";
     return PT_ERR_NAN;
+  }
+  if (hs & ST_TIMEOUT) {
+    g_err = "pt_svd_f64: a barrier wait ran out of time";
+    return PT_ERR_DEVICE_TIMEOUT;
+  }
+  if (hs & ST_CAPACITY) {
+    g_err = "pt_svd_f64: capacity";
+    return PT_ERR_CAPACITY;
   }
   return PT_OK;
 }

@@ -7,8 +7,8 @@
 //   * the columns are grouped in blocks of b and a round-robin tournament runs over the blocks: one CTA holds
 //     a pair of blocks (2 b columns) in shared memory and runs its b x b cross pairs (in the first round of a
 //     sweep also the pairs inside the blocks) in sub-rounds of b disjoint pairs;
-//   * a task waits for its two blocks only: each block carries the number of rounds it has been through (in perm, free
-//     until the end), stored after its columns and polled by the next task that needs it. A grid barrier per round
+//   * a task waits for its two blocks only: each block carries the number of rounds it has been through
+//     (BondWork::rounds), stored after its columns and polled by the next task that needs it. A grid barrier per round
 //     instead, with its column transfers, took 8000 of the 14000 cycles of a round with b = 2; grid barriers remain
 //     at the end of a sweep;
 //   * the scalars of a sub-round's pairs are computed by the lanes of one extra warp at the same time. Columns
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(CT, 1)
     s_V[w] = work[w].V;
     s_aux[w] = work[w].aux;
     s_sig[w] = work[w].sig;
-    s_ver[w] = work[w].perm;
+    s_ver[w] = work[w].rounds;
   }
   __syncthreads();
   if (cwid == 0) {
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(CT, 1)
         if (lane == 0) {
           __stcg(W.aux + c, s2);
           __stcg(W.sig + c, 1.0);
-          __stcg(W.perm + c, 0);           // rounds of block c (blocks are fewer than columns)
+          __stcg(W.rounds + c, 0);         // of block c (blocks are fewer than columns)
         }
       }
       base = (base + Na) % ngwarp;

@@ -62,7 +62,7 @@ Layout layout(int m, int n, int batch) {
 }
 
 // Fill the per-matrix work descriptors in the workspace on the device (no host staging buffers).
-__global__ void k_noalloc_setup(unsigned char* base, Layout L, int m, int n, int batch) {
+__global__ void k_noalloc_setup(unsigned char* base, Layout L, int m, int n, int batch, double* sigma) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b == 0) *(int*)(base + L.status) = 0;
   if (b >= batch) return;
@@ -73,6 +73,8 @@ __global__ void k_noalloc_setup(unsigned char* base, Layout L, int m, int n, int
   W.sig = (double*)(base + L.sig) + b * Na;
   W.aux = (double*)(base + L.aux) + b * Na;
   W.perm = (int*)(base + L.perm) + b * Na;
+  for (int i = 0; i < (int)Na; ++i) W.perm[i] = 0;      // column indices also if the Jacobi gives up early
+  W.rounds = (int*)(sigma + b * Na);                    // free until the results are written
   W.info = (int*)(base + L.info) + 8 * b;
   W.mD_cap = m;
   W.nD_cap = n;
@@ -126,7 +128,7 @@ int pt_svd_f64_noalloc(const double* A, int m, int n, int batch, double* sigma, 
   cudaStream_t st = (cudaStream_t)cuda_stream;
   const int Ma = m > n ? m : n, Na = m < n ? m : n;
   const size_t sA = (size_t)Ma * Na, sV = (size_t)Na * Na;
-  k_noalloc_setup<<<(batch + 127) / 128, 128, 0, st>>>(base, L, m, n, batch);
+  k_noalloc_setup<<<(batch + 127) / 128, 128, 0, st>>>(base, L, m, n, batch, sigma);
   const int gx = (int)std::min<size_t>(256, ((size_t)m * n + 255) / 256);
   ptk::k_svd_load<<<dim3(gx, batch), 256, 0, st>>>((const double2*)A, m, n, batch, (double2*)(base + L.A), sA);
   ptk::launch_svd_jacobi((const BondWork*)(base + L.items), batch, Ma, Na, max_sweeps, (int*)(base + L.status),
@@ -143,6 +145,7 @@ int pt_svd_f64_noalloc(const double* A, int m, int n, int batch, double* sigma, 
   if (e != cudaSuccess) return fail(PT_ERR_CUDA, std::string("sync: ") + cudaGetErrorString(e));
   if (hs & ST_SVD_NOCONV) return fail(PT_ERR_SVD_NOCONV, "Jacobi did not converge within max_sweeps");
   if (hs & ST_NAN) return fail(PT_ERR_NAN, "NaN in the singular values");
+  if (hs & ST_TIMEOUT) return fail(PT_ERR_DEVICE_TIMEOUT, "a grid barrier wait ran out of time");
   return PT_OK;
 }
 
