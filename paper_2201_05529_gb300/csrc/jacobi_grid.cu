@@ -409,6 +409,39 @@ __global__ void __launch_bounds__(CT, 1)
           asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
         }
         slot_sync(grp);
+        if (round == 0) {
+          // once a sweep the norms from the columns (2 b of them, wpc warps or half a warp's turn each): a closed-form
+          // norm keeps the rounding error of the norms it came from, which a column that has shrunk by several
+          // rotations to the level of rounding does not bear
+          double na = 0, nb2 = 0;
+          if (wid < JW) {
+            const int g0 = gcol(c0), g1 = wpp > 1 ? -1 : gcol(c0 + JW);
+            auto norm2 = [&](int c, int g) {
+              const double2* a = SM ? s_col + (size_t)c * ld : A + (size_t)g * Ma;
+              double v = 0;
+              for (int r = rc0; r < Ma; r += 32 * wpc) {
+                const double2 u = SM ? a[r] : __ldcg(a + r);
+                v = fma(u.x, u.x, fma(u.y, u.y, v));
+              }
+              return v;
+            };
+            if (g0 >= 0) na = norm2(c0, g0);
+            if (g1 >= 0) nb2 = norm2(c0 + JW, g1);
+            __syncwarp();
+            const double s = wsum2(na, nb2, lane);
+            if ((lane & 15) == 0) S.part[wid][lane >> 4] = s;
+          }
+          slot_sync(grp);
+          if (tid < 2 * b) {
+            double s = 0;
+            if (wpp > 1)
+              for (int k = 0; k < wpc; ++k) s += S.part[tid * wpc + k][0];
+            else
+              s = S.part[tid & (JW - 1)][tid / JW];
+            S.nrm[tid] = s * S.q[tid];
+          }
+          slot_sync(grp);
+        }
         // noise floor as the bits of a non-negative double; significand and exponent of the squared threshold
         const long long fl2 = __double_as_longlong(floor2 * s_fro[w]);
         const double tol = (tol_scale > 0 ? tol_scale : (double)Ma) * UNIT;
@@ -594,7 +627,7 @@ __global__ void __launch_bounds__(CT, 1)
             }
           }
         }
-        if (tid < 2 * b && S.rotc[tid]) {
+        if (tid < 2 * b && gcol(tid) >= 0 && (round == 0 || S.rotc[tid])) {
           const int g = gcol(tid);
           __stcg(aux + g, S.nrm[tid]);
           __stcg(sig + g, __double2hiint(S.q[tid]) < MIN_SCALE_HI ? 1.0 : S.q[tid]);

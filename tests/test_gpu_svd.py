@@ -45,3 +45,29 @@ def test_jacobi_svd_against_definition(m, n, batch, scale):
         r = int((s > 1e-10 * s[0]).sum())                                # vectors of the null space are arbitrary in U
         assert np.abs(U[b][:, :r].conj().T @ U[b][:, :r] - np.eye(r)).max() <= 1e-13 * max(m, n)
         assert np.abs(V[b].conj().T @ V[b] - np.eye(k)).max() <= tol
+
+
+@pytest.mark.parametrize("m,n,r", [(97, 130, 24), (128, 32, 8), (256, 256, 64), (64, 64, 1), (31, 31, 30)])
+def test_jacobi_svd_of_low_rank(m, n, r):
+    """Matrices of exact rank r: the columns of the null space shrink to rounding level over many rotations, which
+    closed-form norms alone do not follow. The rest of the spectrum stays within 100 max(m, n) u of sigma_1."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2201_05529_gb300 as pkg
+    pkg.build()
+    capi = pkg.load()
+    capi.use_torch_allocator()
+    rng = np.random.default_rng(m + n + r)
+    k = min(m, n)
+    A = (rng.standard_normal((1, m, r)) + 1j * rng.standard_normal((1, m, r))) @ rng.standard_normal((r, n))
+    S = torch.zeros((1, k), dtype=torch.float64, device="cuda")
+    U = torch.zeros((1, m, k), dtype=torch.complex128, device="cuda")
+    V = torch.zeros((1, n, k), dtype=torch.complex128, device="cuda")
+    capi.svd_f64_noalloc(torch.from_numpy(A).cuda(), S, U, V)
+    S, U, V = S.cpu().numpy()[0], U.cpu().numpy()[0], V.cpu().numpy()[0]
+    s = np.linalg.svd(A[0], compute_uv=False)
+    tol = 1e-13 * max(m, n)
+    assert np.abs(S - s).max() <= tol * s[0]
+    assert S[r:].max() <= 100 * max(m, n) * 1.2e-16 * s[0]
+    assert np.abs((U * S) @ V.conj().T - A[0]).max() <= tol * s[0]
