@@ -1724,12 +1724,13 @@ static size_t svd_layout(int m, int n, int batch, size_t* offs) {
   offs[5] = take(sizeof(int));                                // status, and the barrier's words at + 8 ints
   offs[6] = take(sizeof(BondWork) * (size_t)batch);           // work items
   offs[7] = take(sizeof(double) * (size_t)Na * batch);        // column norms
+  offs[8] = take(ptk::svd_qr_fits(Ma, Na, batch) ? ptk::svd_qr_layout(Ma, Na, batch, nullptr, nullptr) : 0);
   return o;
 }
 
 size_t pt_svd_scratch_bytes(int m, int n, int batch) {
   if (m < 1 || n < 1 || batch < 1) return 0;
-  size_t offs[8];
+  size_t offs[9];
   return svd_layout(m, n, batch, offs);
 }
 
@@ -1918,7 +1919,7 @@ int pt_svd_f64(const double* A, int m, int n, int batch, double* sigma, double* 
   }
   if (max_sweeps <= 0) max_sweeps = 60;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  size_t offs[8];
+  size_t offs[9];
   svd_layout(m, n, batch, offs);
   char* base = (char*)scratch;
   double2* wA = (double2*)(base + offs[0]);
@@ -1930,49 +1931,57 @@ int pt_svd_f64(const double* A, int m, int n, int batch, double* sigma, double* 
   BondWork* items = (BondWork*)(base + offs[6]);
   const int Ma = std::max(m, n), Na = std::min(m, n);
   const size_t sA = (size_t)Ma * Na, sV = (size_t)Na * Na;
+  ptk::SvdQr sq{};
+  ptk::SvdQrHost hq;
   std::vector<BondWork> hw(batch);
   std::vector<int> hinfo(8 * (size_t)batch, 0);
-  for (int b = 0; b < batch; ++b) {
-    BondWork W{};
-    W.A = wA + b * sA;
-    W.V = wV + b * sV;
-    W.sig = sig + (size_t)b * Na;
-    W.perm = perm + (size_t)b * Na;
-    W.rounds = (int*)(sigma + (size_t)b * Na);        // free until the results are written
-    W.info = info + 8 * (size_t)b;
-    W.aux = (double*)(base + offs[7]) + (size_t)b * Na;
-    W.mD_cap = m;
-    W.nD_cap = n;
-    W.k_cap = Na;
-    hw[b] = W;
-    hinfo[8 * b + 0] = m;
-    hinfo[8 * b + 1] = n;
-    hinfo[8 * b + 2] = m < n ? 1 : 0;
-  }
-  cudaMemcpyAsync(items, hw.data(), sizeof(BondWork) * batch, cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(info, hinfo.data(), sizeof(int) * hinfo.size(), cudaMemcpyHostToDevice, st);
-  cudaMemsetAsync(status, 0, sizeof(int), st);
-  cudaMemsetAsync(perm, 0, sizeof(int) * (size_t)Na * batch, st);      // column indices also if the Jacobi gives up early
-  const int gx = (int)std::min<size_t>(256, ((size_t)m * n + 255) / 256);
-  ptk::k_svd_load<<<dim3(gx, batch), 256, 0, st>>>((const double2*)A, m, n, batch, wA, sA);
-  ptk::launch_svd_jacobi(items, batch, Ma, Na, max_sweeps, status, (unsigned*)(status + 8), st);
-  const int gs = (int)std::min<size_t>(256, ((size_t)(m + n + 1) * Na + 255) / 256);
-  ptk::k_svd_store<<<dim3(gs, batch), 256, 0, st>>>(wA, wV, sig, perm, m, n, batch, sA, sV, sigma,
-                                                    (double2*)U, (double2*)V);
-  // the host copies of items/info must outlive the async copies above
-  cudaError_t es = cudaStreamSynchronize(st);
-  if (es != cudaSuccess) {
-    g_err = std::string("pt_svd_f64: ") + cudaGetErrorString(es);
-    return PT_ERR_CUDA;
-  }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) {
-    g_err = std::string("pt_svd_f64: ") + cudaGetErrorString(e);
-    return PT_ERR_CUDA;
-  }
+  // one attempt, after the two QRs (pre) or directly; the status bits it leaves
+  auto attempt = [&](bool pre, int* hs) {
+    if (pre) ptk::svd_qr_layout(Ma, Na, batch, &sq, base + offs[8]);
+    for (int b = 0; b < batch; ++b) {
+      BondWork W{};
+      W.A = pre ? sq.T + b * sV : wA + b * sA;
+      W.V = wV + b * sV;
+      W.sig = sig + (size_t)b * Na;
+      W.perm = perm + (size_t)b * Na;
+      W.rounds = (int*)(sigma + (size_t)b * Na);        // free until the results are written
+      W.info = info + 8 * (size_t)b;
+      W.aux = (double*)(base + offs[7]) + (size_t)b * Na;
+      W.mD_cap = m;
+      W.nD_cap = n;
+      W.k_cap = Na;
+      hw[b] = W;
+      hinfo[8 * b + 0] = pre ? Na : m;
+      hinfo[8 * b + 1] = pre ? Na : n;
+      hinfo[8 * b + 2] = !pre && m < n ? 1 : 0;
+    }
+    cudaMemcpyAsync(items, hw.data(), sizeof(BondWork) * batch, cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(info, hinfo.data(), sizeof(int) * hinfo.size(), cudaMemcpyHostToDevice, st);
+    cudaMemsetAsync(status, 0, sizeof(int), st);
+    // column indices also if the Jacobi gives up early
+    cudaMemsetAsync(perm, 0, sizeof(int) * (size_t)Na * batch, st);
+    if (pre) {
+      ptk::launch_svd_qr((const double2*)A, m, n, batch, items, wA, wV, sig, perm, sq, &hq, max_sweeps, status,
+                         (unsigned*)(status + 8), sigma, (double2*)U, (double2*)V, st);
+    } else {
+      const int gx = (int)std::min<size_t>(256, ((size_t)m * n + 255) / 256);
+      ptk::k_svd_load<<<dim3(gx, batch), 256, 0, st>>>((const double2*)A, m, n, batch, wA, sA);
+      ptk::launch_svd_jacobi(items, batch, Ma, Na, max_sweeps, status, (unsigned*)(status + 8), st);
+      const int gs = (int)std::min<size_t>(256, ((size_t)(m + n + 1) * Na + 255) / 256);
+      ptk::k_svd_store<<<dim3(gs, batch), 256, 0, st>>>(wA, wV, sig, perm, m, n, batch, sA, sV, sigma,
+                                                        (double2*)U, (double2*)V);
+    }
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(hs, status, sizeof(int), cudaMemcpyDeviceToHost, st);
+    // the host copies of the lists must outlive the async copies above
+    const cudaError_t es = cudaStreamSynchronize(st);
+    return e == cudaSuccess ? es : e;
+  };
+  const bool pre = ptk::svd_qr_fits(Ma, Na, batch);
   int hs = 0;
-  e = cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  cudaError_t e = attempt(pre, &hs);
+  // an infinity turns into NaN in a reflector, not everywhere in a rotation: such input gets the direct call's answer
+  if (e == cudaSuccess && pre && (hs & (ST_NAN | ST_SVD_NOCONV)) != 0) e = attempt(false, &hs);
   if (e != cudaSuccess) {
     g_err = std::string("pt_svd_f64: ") + cudaGetErrorString(e);
     return PT_ERR_CUDA;

@@ -1,5 +1,7 @@
 // Kernel declarations shared by the engine and the kernel translation units.
 #pragma once
+#include <vector>
+
 #include "common.cuh"
 
 namespace ptk {
@@ -98,6 +100,26 @@ void launch_jacobi_grid(const BondWork* work, int n_work, int blocks, int rows_c
 void launch_svd_jacobi(const BondWork* items, int batch, int Ma, int Na, int max_sweeps, int* status, unsigned* sync3,
                        cudaStream_t st);
 
+// the standalone SVD after two QRs (svd_qr.cu): its workspaces (of size svd_qr_layout), the host copies of its lists
+// (kept until the stream is synchronised); items: n x n matrices in SvdQr::T with V in wV
+struct SvdQr {
+  double2 *Y, *T, *M, *Vp;
+  double *tau, *nrm;
+  int *pcol, *prow;
+  QRItem* qr;
+  QRBlk* blk;
+  struct ZGemmItem *mul, *ops;
+  char* blk_ws;
+  unsigned char* pack;
+  size_t per_blk, per_a, per_b;
+};
+struct SvdQrHost;
+bool svd_qr_fits(int Ma, int Na, int batch);
+size_t svd_qr_layout(int Ma, int Na, int batch, SvdQr* out, char* base);
+void launch_svd_qr(const double2* A, int m, int n, int batch, const BondWork* items, double2* wA, double2* wV,
+                   double* sig, int* perm, const SvdQr& s, SvdQrHost* h, int max_sweeps, int* status,
+                   unsigned* sync3, double* sigma, double2* U, double2* V, cudaStream_t st);
+
 // QR preconditioning of the bond SVD (qrcp.cu): pivoted QR of D into Y64, B = R^H into G64;
 // after the Jacobi on B: V_D = P U', U_D = D V_D / sigma
 int qrcp_cluster_size(int want, int m_cap, int n_cap);
@@ -147,6 +169,11 @@ struct ZGemmItem {
   const double2* A2;       // rows a_split .. M - 1 of opA(A) come from A2 (same op and leading dimension); NULL: all from A
   int a_split;
   long long split;         // > 0: each K chunk's product goes to C + chunk * split (chunks of zgemm9_chunks)
+};
+struct SvdQrHost {
+  std::vector<QRItem> qr;
+  std::vector<QRBlk> blk;
+  std::vector<ZGemmItem> mul;
 };
 size_t zgemm_pack_bytes(int rows_cap, int k_cap, int which);
 // the A operands' slice planes and row exponents alone (for items whose later products skip them)
