@@ -96,13 +96,14 @@ struct pt_tebd {
   int grid_blocks = 0;                // whole-GPU Jacobi: CTAs per launch (0: use the cluster kernel)
   int tiles_odd = 1, tiles_even = 1;  // fast path: theta + gate GEMM output tiles per layer (capacity)
   std::vector<int*> bond_info;        // per bond (odd list, then even list): its info words
-  int qr_cluster = 1;                 // CTAs per matrix of the global-memory cluster pivoted QR
   int qr_smem_cluster = 0;            // >0: the cluster shared-memory pivoted QR fits (CTAs per matrix)
-  bool qr_grid_odd = false, qr_grid_even = false;   // the whole-GPU pivoted QR fits the layer
+  bool qr_grid_odd = false, qr_grid_even = false;   // choice 0 is taken for the layer
   bool hqr_odd = false, hqr_even = false;            // the whole-GPU outer-block QR/LQ fits the layer
   // the kernels each layer runs (chosen by the autotuner, forced, or by the default order)
   struct Route {
-    int qr = 2;      // pivoted QR of the SVD: 0 whole GPU, 1 cluster shared memory, 2 cluster global memory
+    // pivoted QR of the SVD: 1 the largest cluster per matrix, 2 clusters by the number of matrices; 0, the name of a
+  // whole-GPU kernel that 1 took the place of (saved choices hold it), runs as 1
+  int qr = 2;
     int k2 = 1;      // outer-block QR/LQ: 0 whole GPU, 1 one CTA per block
     float ms_qr[3] = {-1, -1, -1}, ms_k2[2] = {-1, -1};   // tuner timings (ms; -1: not a candidate)
     bool tuned = false, cached = false;
@@ -257,16 +258,13 @@ void enqueue_k2(pt_tebd* h, const BondWork* work, int n, int k2) {
   else ptk::k_householder<<<dim3(n, 2), ptk::QR_THREADS_, 0, h->stream>>>(h->T, work, n);
 }
 
-// pivoted QR of the SVD: 0 whole GPU, 1 cluster shared memory, 2 cluster global memory; it stops at
+// pivoted QR of the SVD: 0, 1 the largest cluster, 2 clusters by the number of matrices; it stops at
 // D's noise level (FP64 rounding, or the sliced tensor-core product's) or after kmax reflectors
 void enqueue_qr(pt_tebd* h, const BondWork* work, int n, int qr, int kmax) {
   const int kc = work == h->d_odd ? h->kcap_odd : h->kcap_even, mc = work == h->d_odd ? h->mcap_odd : h->mcap_even;
   const double tau2 = h->opt.precision == PT_BF16_OZAKI ? 8.271806125530277e-25    // (2^-40)^2
                                                         : 1.232595164407831e-32;   // (2^-53)^2
-  if (qr == 0) ptk::launch_qrcp_grid(work, n, h->grid_blocks, h->d_sync3, tau2, kmax, h->T.status, h->stream);
-  else
-    ptk::launch_qrcp_precondition(work, n, h->qr_cluster, qr == 1 ? h->qr_smem_cluster : 0, kc, mc, tau2, kmax,
-                                  h->T.status, h->stream);
+  ptk::launch_qrcp_precondition(work, n, qr == 2 ? 0 : h->qr_smem_cluster, kc, mc, tau2, kmax, h->T.status, h->stream);
 }
 
 // multiplet floor of the fast path (relative to sigma_max): above its singular values' accuracy
@@ -670,7 +668,6 @@ int tune_layer(pt_tebd* h, const BondWork* work, int n, const std::vector<BondWo
   std::vector<int> qrc{2};
   if (h->use_rsvd) qrc.clear();                      // the fast path's SVD has no pivoted QR
   else if (h->qr_smem_cluster > 0) qrc.insert(qrc.begin(), 1);
-  if (!h->use_rsvd && (odd ? h->qr_grid_odd : h->qr_grid_even)) qrc.insert(qrc.begin(), 0);
   for (int c : qrc) {
     float best = 1e30f;
     for (int rep = 0; rep < 2; ++rep)
@@ -752,13 +749,13 @@ int choose_routes(pt_tebd* h, const std::vector<BondWork>& odd, const std::vecto
   cudaMemcpyAsync(&h->tune_status, T.status, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
   cudaStreamSynchronize(h->stream);
   if (h->tune_status != 0) {
-    auto defaults = [&](pt_tebd::Route& r, bool qr_grid, bool hqr) {
-      r.qr = qr_grid ? 0 : (h->qr_smem_cluster > 0 ? 1 : 2);
+    auto defaults = [&](pt_tebd::Route& r, bool hqr) {
+      r.qr = 2;
       r.k2 = hqr ? 0 : 1;
       r.tuned = false;
     };
-    defaults(h->route_odd, h->qr_grid_odd, h->hqr_odd);
-    defaults(h->route_even, h->qr_grid_even, h->hqr_even);
+    defaults(h->route_odd, h->hqr_odd);
+    defaults(h->route_even, h->hqr_even);
   }
   // back to the initial state
   upload_initial_gamma_lambda(h);
@@ -1081,22 +1078,18 @@ int build(pt_tebd* h) {
     dims(odd, &h->kcap_odd, &h->mcap_odd);
     dims(even, &h->kcap_even, &h->mcap_even);
     int k = std::max(h->kcap_odd, h->kcap_even);
-    h->qr_cluster = ptk::qrcp_cluster_size(std::max(1, std::min(16, (k + 31) / 32)),
-                                           std::max(h->mcap_odd, h->mcap_even), k);
     h->qr_smem_cluster = ptk::qrcp_smem_cluster(std::max(h->mcap_odd, h->mcap_even), k);
   }
   // bond SVDs: the whole-GPU cooperative kernels when the device can co-schedule them, else one
   // thread-block cluster per matrix
   h->grid_blocks = std::max(h->n_odd, h->n_even) <= 1024 ? ptk::jacobi_grid_blocks() : 0;
   {
-    // which kernels fit each layer: the whole-GPU pivoted QR where the layer's columns fit one per
-    // warp; the cluster shared-memory one where a matrix fits 200 KB per CTA; the global-memory one
-    // always; the whole-GPU outer-block QR where every block's columns fit the CTAs' share
-    const bool ok = h->grid_blocks > 0 && ptk::qrcp_grid_ok();
+    // choice 0 of the pivoted QR is taken where a layer's columns fit one to a warp, 16 warps to an SM
     auto fits = [&](const std::vector<BondWork>& v, int mc) {
       int tot = 0;
       for (auto& W : v) tot += W.k_cap;
-      return ok && !v.empty() && ptk::qrcp_grid_fits((int)v.size(), mc, tot, h->grid_blocks);
+      return h->grid_blocks > 0 && !v.empty() && v.size() <= 256 && mc <= 256 &&
+             (tot + h->grid_blocks - 1) / h->grid_blocks <= 16;
     };
     h->qr_grid_odd = fits(odd, h->mcap_odd);
     h->qr_grid_even = fits(even, h->mcap_even);
@@ -1110,13 +1103,9 @@ int build(pt_tebd* h) {
     };
     h->hqr_odd = hfits(odd);
     h->hqr_even = hfits(even);
-    // default order (no tuning): whole GPU, then cluster shared memory, then cluster global memory
-    auto defaults = [&](pt_tebd::Route& r, bool qr_grid, bool hqr) {
-      r.qr = qr_grid ? 0 : (h->qr_smem_cluster > 0 ? 1 : 2);
-      r.k2 = hqr ? 0 : 1;
-    };
-    defaults(h->route_odd, h->qr_grid_odd, h->hqr_odd);
-    defaults(h->route_even, h->qr_grid_even, h->hqr_even);
+    // default (no tuning): clusters by the number of matrices, the whole-GPU outer QR where it fits
+    h->route_odd.k2 = h->hqr_odd ? 0 : 1;
+    h->route_even.k2 = h->hqr_even ? 0 : 1;
   }
   if (h->opt.precision == PT_BF16_OZAKI && h->grid_blocks > 0 && ptk::hqr_items_ok()) {
     // the fast path's randomized truncated SVD: item lists per layer, the sketch matrix

@@ -122,17 +122,13 @@ void launch_svd_qr(const double2* A, int m, int n, int batch, const BondWork* it
 
 // QR preconditioning of the bond SVD (qrcp.cu): pivoted QR of D into Y64, B = R^H into G64;
 // after the Jacobi on B: V_D = P U', U_D = D V_D / sigma
-int qrcp_cluster_size(int want, int m_cap, int n_cap);
+// cluster size for which matrices up to m_cap x n_cap stay in shared memory (0: none)
 int qrcp_smem_cluster(int m_cap, int n_cap);
-// whole-GPU variant (cooperative, one CTA per SM): usable when qrcp_grid_ok() and the layer fits
-int qrcp_grid_ok();
-int qrcp_grid_fits(int n_work, int m_cap, int total_cols_cap, int blocks);
 // tau2: squared relative noise level of D at which the pivoted QR stops (rank-revealing);
 // kmax: stop after at most kmax reflectors (the autotuner times a prefix; otherwise INT_MAX)
-void launch_qrcp_grid(const BondWork* work, int n_work, int blocks, unsigned* sync3, double tau2, int kmax,
-                      int* status, cudaStream_t st);
-void launch_qrcp_precondition(const BondWork* work, int n_work, int cluster, int smem_cluster, int k_cap, int m_cap,
-                              double tau2, int kmax, int* status, cudaStream_t st);
+// cluster: CTAs per matrix (0: by the number of matrices; columns that do not fit shared memory stay in L2)
+void launch_qrcp_precondition(const BondWork* work, int n_work, int cluster, int k_cap, int m_cap, double tau2,
+                              int kmax, int* status, cudaStream_t st);
 // after the truncation: V_D and U_D on the kept columns (lam_chi: the tables' bond dims)
 void launch_qrcp_finish(const BondWork* work, int n_work, int k_cap, int m_cap, const int* lam_chi,
                         cudaStream_t st);
