@@ -18,6 +18,8 @@
 //     x - conj(mu) y and y + nu x, mu = rho q_y g, nu = rho q_x g, g = x^H y of the stored columns, and
 //     q_x, q_y are multiplied by cos^2 = 1 / (1 + tan^2). That is 9 FP64 operations before the columns can be
 //     rotated; the new norms and scales are formed while they are. A row costs 8 FP64 operations, not 12;
+//   * inner products are summed over lanes and warps in 64-bit fixed point (to_fixed below): the butterflies were six of
+//     the eighteen FP64 instructions that a warp with one row per lane issues per pair;
 //   * a CTA has two such task slots of 8 + 1 warps (named barriers), so one's scalars overlap the other's
 //     columns; tasks fill one slot of every SM before the second;
 //   * b is chosen on the device from the live dims by a cost model of these terms (choose_block), and CTAs that
@@ -41,6 +43,7 @@
 
 #include "grid_sync.cuh"
 #include "kernels.h"
+#include "tc_common.cuh"
 
 namespace ptk {
 
@@ -96,6 +99,34 @@ __device__ __forceinline__ float significand(double x, int* e) {
   const int hi = __double2hiint(x);
   *e = ((hi >> 20) & 0x7ff) - 1023;
   return __int_as_float(0x3f800000 | (hi & 0xfffff) << 3 | (int)((unsigned)__double2loint(x) >> 29));
+}
+
+// Sums over the lanes and warps as 64-bit fixed-point numbers. With E = pair_exponent, |x| |y| < 2^E for the stored
+// columns, so by Cauchy-Schwarz every partial inner product is below 2^E too and so are sums of their magnitudes: at 57
+// fractional bits below 2^E the sums need no further headroom, their error (2^-57 of |x| |y| per lane) is below that of
+// FP64 sums, and 5 bits remain for norms that are off (closed forms between two exact ones).
+__device__ __forceinline__ int exponent_of(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) - 1023; }
+
+__device__ __forceinline__ int pair_exponent(double al, double be, double qx, double qy) {
+  return (exponent_of(al) + exponent_of(be) - exponent_of(qx) - exponent_of(qy) + 3) >> 1;
+}
+
+// x in units of 2^(E - 57), truncated; 0 if not finite or out of range
+__device__ __forceinline__ long long to_fixed(double x, int E) {
+  const long long b = __double_as_longlong(x);
+  const int e = exponent_of(x), sh = e - E + 5;
+  long long m = (b & 0xfffffffffffffll) | 0x10000000000000ll;
+  m = sh >= 0 ? m << min(sh, 63) : m >> min(-sh, 63);
+  if (sh > 9 || e < -1022 || e > 1023) m = 0;
+  return b < 0 ? -m : m;
+}
+
+// the sum of v over the lanes, in every lane: 21 + 21 + 22 bits by the integer reduction of a warp
+__device__ __forceinline__ long long lane_sum(long long v) {
+  const unsigned l0 = __reduce_add_sync(0xffffffffu, (unsigned)v & 0x1fffffu);
+  const unsigned l1 = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 21) & 0x1fffffu);
+  const int l2 = (int)__reduce_add_sync(0xffffffffu, (unsigned)(int)(v >> 42));
+  return (long long)l0 + ((long long)l1 << 21) + ((long long)l2 << 42);
 }
 
 __device__ __forceinline__ float sqrt_approx(float x) {
@@ -485,8 +516,10 @@ __global__ void __launch_bounds__(CT, 1)
                 gr = fma(u.x, v.x, fma(u.y, v.y, gr));
                 gim = fma(u.x, v.y, fma(-u.y, v.x, gim));
               }
-              const double s = wsum2(gr, gim, lane);
-              if ((lane & 15) == 0) S.part[wid][lane >> 4] = s;
+              const int E = pair_exponent(S.nrm[li], S.nrm[lj], S.q[li], S.q[lj]);
+              __syncwarp();
+              const long long sr_ = lane_sum(to_fixed(gr, E)), si_ = lane_sum(to_fixed(gim, E));
+              if (lane < 2) S.part[wid][lane] = __longlong_as_double(lane == 0 ? sr_ : si_);
             }
             slot_sync(grp);
           } else {
@@ -498,6 +531,7 @@ __global__ void __launch_bounds__(CT, 1)
             const bool lead = first && (lane & 1) == 0, lead_odd = first && (lane & 1) != 0;
             const double al = S.nrm[i], be = S.nrm[j], qx = S.q[i], qy = S.q[j];
             const double h = be - al, qq = qx * qy;
+            const int pe = pair_exponent(al, be, qx, qy);
             int ea, eb, eh;
             const float am = significand(al, &ea), bm = significand(be, &eb), hm = significand(h, &eh);
             // rotate unless |gamma| <= tol sqrt(alpha beta), or a column is at the noise floor (compared as
@@ -506,10 +540,12 @@ __global__ void __launch_bounds__(CT, 1)
                       min(__double_as_longlong(al), __double_as_longlong(be)) > max(fl2, 0x0010000000000000ll - 1);
             if (lane == 0) S.renorm[sr & 1] = 0;
             // computed here, while the column warps form the inner products, not after the barrier
-            asm volatile("" ::"d"(h), "d"(qq), "f"(am), "f"(bm), "f"(hm), "r"(ea + eb + et), "r"(eh), "r"((int)go));
+            asm volatile("" ::"d"(h), "d"(qq), "f"(am), "f"(bm), "f"(hm), "r"(ea + eb + et), "r"(eh), "r"(pe),
+                         "r"((int)go));
             slot_sync(grp);
-            double v = lane < 2 * JW ? S.part[lane >> 1][lane & 1] : 0.0;
-            for (int o = 2; o < 2 * wpp; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            long long vf = lane < 2 * JW ? __double_as_longlong(S.part[lane >> 1][lane & 1]) : 0ll;
+            for (int o = 2; o < 2 * wpp; o <<= 1) vf += __shfl_xor_sync(0xffffffffu, vf, o);
+            const double v = tcx::fixed_to_double(vf, pe, 57);
             const double other = __shfl_xor_sync(0xffffffffu, v, 1);
             const double gr = (lane & 1) ? other : v, gm = (lane & 1) ? v : other;
             const double g2 = qq * fma(gr, gr, gm * gm);             // |gamma|^2
