@@ -32,6 +32,7 @@ namespace {
 constexpr int NB = 32;                     // panel width
 constexpr int PT = 512;                    // threads of a panel CTA
 constexpr int PW = PT / 32;
+constexpr int PANEL_T = PT + 32;           // and a warp for the scalars
 constexpr int SMALL_N = 32;                // columns of a matrix that one CTA factors whole
 constexpr int MAX_C = 16;                  // CTAs per cluster
 constexpr int PANEL_SMEM = 200 * 1024;     // panel rows of one CTA (227 KB less the exchange buffers)
@@ -45,6 +46,14 @@ __device__ __forceinline__ double wsum2(double a, double b, int lane) {
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) keep += __shfl_xor_sync(0xffffffffu, keep, o);
   return keep;
+}
+
+// sums of a and b over the L lanes of a group (half: the upper half of it), in every lane
+__device__ __forceinline__ double2 group_sum(double a, double b, int L, bool half) {
+  double s = (half ? b : a) + __shfl_xor_sync(0xffffffffu, half ? a : b, L >> 1);
+  for (int o = L >> 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  const double other = __shfl_xor_sync(0xffffffffu, s, L >> 1);
+  return half ? make_double2(other, s) : make_double2(s, other);
 }
 
 __device__ __forceinline__ bool live(const QRItem& q) { return q.m > 0 && q.n > 0 && q.n <= q.m; }
@@ -138,18 +147,19 @@ __global__ void k_qrb_plan(Tables T, const BondWork* work, const QRItem* list, Q
 }
 
 // Panel p of every matrix: one cluster per matrix. Dynamic shared memory: the CTA's rows of the panel, column-major.
-// Per column j: the warps form s_k = sum_{r > j} conj(x_r) a_k,r (x = column j) of their columns k >= j (k mod 16) and
-// send them, with row j from its owner, to every CTA; after the cluster barrier two warps add the parts (lane = column),
-// one warp forms the reflector's scalars and w_k = tau u^H a_k of all columns at once, and every warp updates its
-// columns. An FP64 instruction takes 64 cycles of a sub-partition whatever its lanes, so what is done once per column
-// is done by one warp for all 32 columns, not by each warp for its own: 15000 cycles per reflector besides the rows'
-// arithmetic before, ~6000 so.
-__global__ void __launch_bounds__(PT, 1) k_qr_panel(const QRBlk* blk, int n_items, int p, int rc_cap, int* status) {
+// Per column j: L lanes per column k >= j form s_k = sum_{r > j} conj(x_r) a_k,r (x = column j) and send it, with row j
+// from its owner, to every CTA; after the cluster barrier the same lanes add the parts while an extra warp forms the
+// reflector's scalars from those of s_j; then they apply w_k = tau u^H a_k to their column. An FP64 instruction takes 64
+// cycles of a sub-partition whatever its lanes: so columns share warps where there are many (L = 4 or 8: fewer
+// reduction steps than a warp per column has), the scalars' square roots go to two lanes of one instruction and start from
+// FP32. Cycles per reflector besides the rows' arithmetic: 15000 with all of it done by every warp for its own columns ->
+// 6000 with one warp for the sums over CTAs and the scalars of all columns -> 4000 so.
+__global__ void __launch_bounds__(PANEL_T, 1) k_qr_panel(const QRBlk* blk, int n_items, int p, int rc_cap, int* status) {
   extern __shared__ __align__(16) double2 s_p[];
   __shared__ double2 s_part[2][MAX_C][NB];
   __shared__ double2 s_row[2][NB];
-  __shared__ double2 s_w[NB], s_u, s_scale[NB], s_ph;
-  __shared__ double s_tot[2][NB], s_a2, s_aabs, s_taus[NB];
+  __shared__ double2 s_u, s_cr, s_scale[NB];
+  __shared__ double s_ti, s_taus[NB];
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), C = (int)cl.num_blocks();
   const int i = blockIdx.x / C;
@@ -164,129 +174,154 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel(const QRBlk* blk, int n_item
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int lo = min(rows, rank * rc), mine = min(rows, lo + rc) - lo;
   double2* A = q.A + row0 + (size_t)row0 * q.m;
-  for (int k = warp; k < nc; k += PW)
+  for (int k = warp; k < nc; k += PANEL_T / 32)
     for (int r = lane; r < mine; r += 32) s_p[(size_t)k * rc + r] = A[lo + r + (size_t)k * q.m];
   // R above the panel: rows 0 .. row0 - 1 of its columns are final
-  for (int idx = rank * PT + tid; idx < row0 * nc; idx += C * PT) {
+  for (int idx = rank * PANEL_T + tid; idx < row0 * nc; idx += C * PANEL_T) {
     const int r = idx % row0, k = idx / row0;
     q.R[r + (size_t)(row0 + k) * q.n] = q.A[r + (size_t)(row0 + k) * q.m];
   }
   cl.sync();
+  const int grp_rows = min(rc, rows);
   for (int j = 0; j < nc; ++j) {
     const int par = j & 1, own = j / rc, jl = j - lo;          // row j's CTA; row j's local index
     const double2* x = s_p + (size_t)j * rc;
     const int from = max(0, jl + 1);                           // first local row below j
-    const int k0 = j + ((warp - j) & (PW - 1)), k1 = k0 + PW;  // this warp's columns
-    if (k0 < nc) {
-      const double2* y0 = s_p + (size_t)k0 * rc;
-      const double2* y1 = s_p + (size_t)(k1 < nc ? k1 : k0) * rc;
-      double a0 = 0, b0 = 0, a1 = 0, b1 = 0;
-      if (k1 < nc) {
-        for (int r = from + lane; r < mine; r += 32) {
-          const double2 u = x[r], v = y0[r], w = y1[r];
-          a0 = fma(u.x, v.x, fma(u.y, v.y, a0));
-          b0 = fma(u.x, v.y, fma(-u.y, v.x, b0));
-          a1 = fma(u.x, w.x, fma(u.y, w.y, a1));
-          b1 = fma(u.x, w.y, fma(-u.y, w.x, b1));
-        }
-      } else {
-        for (int r = from + lane; r < mine; r += 32) {
-          const double2 u = x[r], v = y0[r];
-          a0 = fma(u.x, v.x, fma(u.y, v.y, a0));
-          b0 = fma(u.x, v.y, fma(-u.y, v.x, b0));
-        }
-      }
-      __syncwarp();
-      // four sums in one reduce-scatter: lanes 0, 8, 16, 24 end with re 0, im 0, re 1, im 1
-      const bool h16 = lane & 16, h8 = lane & 8;
-      double c0 = h16 ? a1 : a0, c1 = h16 ? b1 : b0;
-      if (k1 < nc) {
-        c0 += __shfl_xor_sync(0xffffffffu, h16 ? a0 : a1, 16);
-        c1 += __shfl_xor_sync(0xffffffffu, h16 ? b0 : b1, 16);
-      } else {
-        c0 = a0 + __shfl_xor_sync(0xffffffffu, a0, 16);
-        c1 = b0 + __shfl_xor_sync(0xffffffffu, b0, 16);
-      }
-      double d = (h8 ? c1 : c0) + __shfl_xor_sync(0xffffffffu, h8 ? c0 : c1, 8);
+    // lanes per column: the instructions of a sub-partition, eight per row and four per reduction step; the same in
+    // every CTA, and so that one pass of the 16 warps takes all columns
+    int lg = 5;
+    {
+      const int nk = nc - j;
+      int best = 0x7fffffff;
 #pragma unroll
-      for (int o = 4; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-      const double2 t0 = make_double2(__shfl_sync(0xffffffffu, d, 0), __shfl_sync(0xffffffffu, d, 8));
-      const double2 t1 = make_double2(__shfl_sync(0xffffffffu, d, 16), __shfl_sync(0xffffffffu, d, 24));
-      const int to = lane & 15;
-      const int k = lane < 16 ? k0 : k1;
-      if (to < C && k < nc) {
-        *cl.map_shared_rank(&s_part[par][rank][k], to) = lane < 16 ? t0 : t1;
-        if (rank == own) *cl.map_shared_rank(&s_row[par][k], to) = s_p[(size_t)k * rc + jl];
+      for (int t = 2; t <= 5; ++t) {
+        const int warps = ((((nk << t) + 31) >> 5) + 3) >> 2;
+        const int c = warps * (8 * ((grp_rows + (1 << t) - 1) >> t) + 4 * t + 8);
+        if (c < best && (nk << t) <= 32 * PW) {
+          best = c;
+          lg = t;
+        }
+      }
+    }
+    const int L = 1 << lg, ln = lane & (L - 1);
+    const int k = warp < PW ? j + ((warp * 32 + lane) >> lg) : nc;         // this group's column
+    const bool on = k < nc, half = ln >= (L >> 1);
+    double2* y = s_p + (size_t)(on ? k : j) * rc;
+    if (__any_sync(0xffffffffu, on)) {
+      double a0 = 0, b0 = 0;
+      if (on) {
+        int r = from + ln;
+        for (; r + 3 * L < mine; r += 4 * L) {       // one warp may have a sub-partition: four rows' loads at once
+          double2 u[4], v[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            u[q] = x[r + q * L];
+            v[q] = y[r + q * L];
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            a0 = fma(u[q].x, v[q].x, fma(u[q].y, v[q].y, a0));
+            b0 = fma(u[q].x, v[q].y, fma(-u[q].y, v[q].x, b0));
+          }
+        }
+        for (; r < mine; r += L) {
+          const double2 u = x[r], v = y[r];
+          a0 = fma(u.x, v.x, fma(u.y, v.y, a0));
+          b0 = fma(u.x, v.y, fma(-u.y, v.x, b0));
+        }
+      }
+      const double2 t = group_sum(a0, b0, L, half);
+      if (on) {
+        for (int to = ln; to < C; to += L) {
+          *cl.map_shared_rank(&s_part[par][rank][k], to) = t;
+          if (rank == own) *cl.map_shared_rank(&s_row[par][k], to) = y[jl];
+        }
       }
     }
     cl.sync();
-    if (warp < 2) {
-      // the parts in CTA order: warp 0 the real parts, warp 1 the imaginary parts, lane = column
-      double v = 0.0;
-      if (lane >= j && lane < nc)
-        for (int c = 0; c < C; ++c) v += warp == 0 ? s_part[par][c][lane].x : s_part[par][c][lane].y;
-      s_tot[warp][lane] = v;
-    } else if (warp == 2) {
-      // alpha = row j of column j: |alpha|^2, |alpha| and its phase
-      const double2 al = s_row[par][j];
-      const double a2 = fma(al.x, al.x, al.y * al.y);
-      const double ra = a2 > 0.0 ? rsqrt(a2) : 0.0;
-      double aabs = a2 * ra;
-      aabs = fma(0.5 * ra, fma(-aabs, aabs, a2), aabs);
-      if (lane == 0) {
-        s_a2 = a2;
-        s_aabs = aabs;
-        s_ph = a2 > 0.0 ? make_double2(al.x * ra, al.y * ra) : make_double2(1.0, 0.0);
-      }
-    }
-    __syncthreads();
-    if (warp == 0) {
-      // nrm = ||x||, u_j = alpha - beta = phase (|alpha| + nrm), 2 / |u|^2 = 1 / (nrm (nrm + |alpha|)):
-      // w_k = (conj(phase) a_k,j + s_k / (nrm + |alpha|)) / nrm
-      const double n2 = s_tot[0][j] + s_a2;
-      const double2 ph = s_ph;
-      const bool some = n2 > 0.0 || n2 != n2;
-      const double rn = some ? rsqrt(n2) : 0.0;
-      double nrm = n2 * rn;
-      nrm = some ? fma(0.5 * rn, fma(-nrm, nrm, n2), nrm) : 0.0;
-      const double sum = s_aabs + nrm;
-      const double inv = some ? 1.0 / sum : 0.0;
-      const double2 yj = s_row[par][lane < nc ? lane : j];
-      const double sr = s_tot[0][lane], si = s_tot[1][lane];
-      const double cr = rn * ph.x, ci = rn * ph.y, ti = rn * inv;
-      s_w[lane] = make_double2(fma(cr, yj.x, fma(ci, yj.y, ti * sr)), fma(cr, yj.y, fma(-ci, yj.x, ti * si)));
-      if (lane == 0) {
-        s_u = make_double2(ph.x * sum, ph.y * sum);                                    // alpha - beta
-        s_scale[j] = make_double2(ph.x * inv, -ph.y * inv);                            // 1 / (alpha - beta)
-        s_taus[j] = some ? sum * rn : 0.0;
-        if (rank == own) s_p[(size_t)j * rc + jl] = some ? make_double2(-ph.x * nrm, -ph.y * nrm) : s_row[par][j];   // beta
-      }
-    }
-    __syncthreads();
-    const double2 uj = s_u;
+    double2 tot = make_double2(0.0, 0.0);
+    if (warp == PW) {
+      // alpha = row j of column j, nrm = ||x||: u_j = alpha - beta = phase (|alpha| + nrm), 2 / |u|^2 = 1 / (nrm (nrm +
+      // |alpha|)): w_k = (conj(phase) a_k,j + s_k / (nrm + |alpha|)) / nrm. Lane 0: alpha, lane 1: x
+      double v = lane < C ? s_part[par][lane][j].x : 0.0;
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int k = e == 0 ? k0 : k1;
-      if (k == j || k >= nc) continue;
-      double2* y = s_p + (size_t)k * rc;
-      const double2 w = s_w[k];
-      for (int r = from + lane; r < mine; r += 32) {
+      for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      const double2 al = s_row[par][j];
+      const double a2 = fma(al.x, al.x, al.y * al.y), n2 = v + a2;
+      const double q = lane == 0 ? a2 : n2;
+      const double ri = __double_as_longlong(q) == 0 ? 0.0 : inv_sqrt(q);
+      double rt = q * ri;
+      rt = fma(0.5 * ri, fma(-rt, rt, q), rt);
+      const double ra = __shfl_sync(0xffffffffu, ri, 0), rn = __shfl_sync(0xffffffffu, ri, 1);
+      const double aabs = __shfl_sync(0xffffffffu, rt, 0), nrm = __shfl_sync(0xffffffffu, rt, 1);
+      const bool some = __double_as_longlong(n2) != 0;
+      // an instruction of this warp takes 64 cycles whatever its lanes: the phase's two products and the ten at the end
+      // go to a lane each
+      const double pv = (lane == 0 ? al.x : al.y) * ra;
+      double px = __shfl_sync(0xffffffffu, pv, 0), py = __shfl_sync(0xffffffffu, pv, 1);
+      if (__double_as_longlong(a2) == 0) {
+        px = 1.0;
+        py = 0.0;
+      }
+      const double sum = aabs + nrm, inv = some ? inverse(sum) : 0.0;
+      const double f = lane < 2 ? rn : (lane < 4 ? sum : (lane < 6 ? inv : (lane < 8 ? rn : nrm)));
+      const double g = lane == 6 ? inv : (lane == 7 ? sum : ((lane & 1) ? py : px));
+      double v10 = f * g;
+      if (lane == 5 || lane >= 8) v10 = __hiloint2double(__double2hiint(v10) ^ 0x80000000, __double2loint(v10));
+      double* dst = lane < 2 ? &s_cr.x + lane                                    // conj(phase) / nrm
+                  : lane < 4 ? &s_u.x + (lane - 2)                               // alpha - beta
+                  : lane < 6 ? &s_scale[j].x + (lane - 4)                        // 1 / (alpha - beta)
+                  : lane == 6 ? &s_ti : lane == 7 ? &s_taus[j]
+                  : &s_p[(size_t)j * rc + max(0, jl)].x + (lane - 8);            // beta
+      if (lane < 8 || (lane < 10 && rank == own && some)) *dst = v10;
+    } else if (__any_sync(0xffffffffu, on && k > j)) {
+      // the parts, in the same order in every CTA
+      double a0 = 0, b0 = 0;
+      if (on)
+        for (int c = ln; c < C; c += L) {
+          const double2 t = s_part[par][c][k];
+          a0 += t.x;
+          b0 += t.y;
+        }
+      tot = group_sum(a0, b0, L, half);
+    }
+    __syncthreads();
+    if (on && k > j) {
+      const double2 cr = s_cr, yj = s_row[par][k];
+      const double ti = s_ti;
+      const double wx = fma(cr.x, yj.x, fma(cr.y, yj.y, ti * tot.x)), wy = fma(cr.x, yj.y, fma(-cr.y, yj.x, ti * tot.y));
+      int r = from + ln;
+      for (; r + 3 * L < mine; r += 4 * L) {
+        double2 u[4], v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          u[q] = x[r + q * L];
+          v[q] = y[r + q * L];
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          v[q].x = fma(-u[q].x, wx, fma(u[q].y, wy, v[q].x));
+          v[q].y = fma(-u[q].x, wy, fma(-u[q].y, wx, v[q].y));
+          y[r + q * L] = v[q];
+        }
+      }
+      for (; r < mine; r += L) {
         const double2 u = x[r];
         double2 v = y[r];
-        v.x = fma(-u.x, w.x, fma(u.y, w.y, v.x));
-        v.y = fma(-u.x, w.y, fma(-u.y, w.x, v.y));
+        v.x = fma(-u.x, wx, fma(u.y, wy, v.x));
+        v.y = fma(-u.x, wy, fma(-u.y, wx, v.y));
         y[r] = v;
       }
-      if (rank == own && lane == 0) {
-        const double2 yj = s_row[par][k];
-        y[jl].x = yj.x - (uj.x * w.x - uj.y * w.y);
-        y[jl].y = yj.y - (uj.x * w.y + uj.y * w.x);
+      if (rank == own && ln == 0) {
+        const double2 uj = s_u;
+        y[jl].x = yj.x - (uj.x * wx - uj.y * wy);
+        y[jl].y = yj.y - (uj.x * wy + uj.y * wx);
       }
     }
     __syncthreads();
   }
   // the panel's rows of R, the reflectors with their zeros and ones, tau
-  for (int k = warp; k < nc; k += PW) {
+  for (int k = warp; k < nc; k += PANEL_T / 32) {
     const double2 s = s_scale[k];
     double2* H = q.H + row0 + (size_t)(row0 + k) * q.m;
     for (int r = lane; r < mine; r += 32) {
@@ -301,7 +336,7 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel(const QRBlk* blk, int n_item
   }
   // zeros of R below the panel
   const int below = q.n - row0 - nc;
-  for (int idx = rank * PT + tid; idx < below * nc; idx += C * PT)
+  for (int idx = rank * PANEL_T + tid; idx < below * nc; idx += C * PANEL_T)
     q.R[row0 + nc + idx % below + (size_t)(row0 + idx / below) * q.n] = make_double2(0.0, 0.0);
   cl.sync();                               // no CTA leaves while another may still write to its shared memory
 }
@@ -512,7 +547,7 @@ ClusterTable g_tab[MAX_DEV];
 cudaLaunchConfig_t panel_cfg(int clusters, int c, size_t smem, cudaStream_t st, cudaLaunchAttribute* at) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(clusters * c, 1, 1);
-  cfg.blockDim = dim3(PT, 1, 1);
+  cfg.blockDim = dim3(PANEL_T, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -548,7 +583,7 @@ size_t up(size_t x) { return (x + 255) & ~size_t(255); }
 }  // namespace
 
 // CTAs per cluster for n matrices of at most m rows: the shortest estimate of a panel column's time, waves of clusters
-// times (76 cycles of FP64 work per row of a CTA, for the 16 columns a panel has right of a column on average, + 6000
+// times (76 cycles of FP64 work per row of a CTA, for the 16 columns a panel has right of a column on average, + 4000
 // cycles of exchange, scalars and barriers); 0: the panel does not fit
 int qr_block_cluster(int n, int m) {
   const ClusterTable& t = cluster_table();
@@ -557,7 +592,7 @@ int qr_block_cluster(int n, int m) {
   for (int c = 1; c <= MAX_C; ++c) {
     const int rc = (m + c - 1) / c;
     if (t.active[c] <= 0 || (size_t)rc * NB * sizeof(double2) > (size_t)PANEL_SMEM) continue;
-    const double v = (double)((n + t.active[c] - 1) / t.active[c]) * (76.0 * rc + 6000.0);
+    const double v = (double)((n + t.active[c] - 1) / t.active[c]) * (76.0 * rc + 4000.0);
     if (v < cost) {
       cost = v;
       best = c;
