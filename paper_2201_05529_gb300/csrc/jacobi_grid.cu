@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(CT, 1)
     if (blockIdx.x == 0 && ctid == 0) atomicOr(status, ST_CAPACITY);
     return;
   }
-  const int b = s_b, wpp = JW / b, lw = __ffs(wpp) - 1;      // warps per pair, its logarithm
+  const int b = s_b, lb = __ffs(b) - 1, wpp = JW >> lb, lw = __ffs(wpp) - 1;      // warps per pair; logarithms
   // CTAs that take part: as many as a round has tasks (and the passes over all columns can use)
   const int G = max(1, min((int)gridDim.x, max(s_most, min((s_cols + 15) / 16, 152))));
   if ((int)blockIdx.x >= G) return;
@@ -382,11 +382,14 @@ __global__ void __launch_bounds__(CT, 1)
         }
         const int w = lo, q = t - s_off[w];
         const int Ma = s_Ma[w], Na = s_Na[w], Vr = with_v ? Na : 0, ld = Ma + Vr;
-        const int nb = (Na + b - 1) / b, nbp = nb + (nb & 1);
-        if (round >= nbp - 1) continue;    // this item's tournament is over
+        const int nb = (Na + b - 1) >> lb, nbp = nb + (nb & 1), m1 = nbp - 1;
+        if (round >= m1) continue;    // this item's tournament is over
         int bi, bj;
         if (q == 0) { bi = nbp - 1; bj = round; }
-        else { bi = (round + q) % (nbp - 1); bj = (round - q + nbp - 1) % (nbp - 1); }
+        else {                             // (round +- q) mod (nbp - 1); a division takes as long as an inner product
+          bi = round + q < m1 ? round + q : round + q - m1;
+          bj = round >= q ? round - q : round - q + m1;
+        }
         double2 *A = s_A[w], *V = s_V[w];
         double *aux = s_aux[w], *sig = s_sig[w];
         // local column c: global column of block bi (c < b) or bj; -1 beyond the matrix
@@ -426,7 +429,7 @@ __global__ void __launch_bounds__(CT, 1)
         }
         if (tid == 0) S.cnt = 0;
         // the column warps share the 2 b columns evenly: JW / 2b warps per column, or two columns per warp
-        const int wpc = max(1, wpp >> 1), c0 = wpp > 1 ? wid / wpc : wid, rc0 = (wpp > 1 ? wid % wpc : 0) * 32 + lane;
+        const int lc = max(0, lw - 1), wpc = 1 << lc, c0 = wid >> lc, rc0 = (wid & (wpc - 1)) * 32 + lane;
         if (SM) {
           for (int c = c0; c < 2 * b && wid < JW; c += JW) {
             const int g = gcol(c);
@@ -485,10 +488,13 @@ __global__ void __launch_bounds__(CT, 1)
           // pair p's local columns: inside a block (round-robin over its b columns) or across the two
           auto pair_of = [&](int pp, int* i, int* j) {
             if (sr < n_inner) {
-              const int h = b / 2, blk = pp >= h, x = pp - blk * h;
+              const int h = b >> 1, blk = pp >= h, x = pp - blk * h;
               int u, v;
               if (x == 0) { u = b - 1; v = sr; }
-              else { u = (sr + x) % (b - 1); v = (sr - x + b - 1) % (b - 1); }
+              else {
+                u = sr + x < b - 1 ? sr + x : sr + x - (b - 1);
+                v = sr >= x ? sr - x : sr - x + b - 1;
+              }
               *i = blk * b + min(u, v);
               *j = blk * b + max(u, v);
             } else {
@@ -577,8 +583,7 @@ __global__ void __launch_bounds__(CT, 1)
             int redo = 0;
             if ((lead || lead_odd) && go) {
               const double rg = rho * g2, t2 = rho * rg, a1 = 1.0 + t2;
-              const double y0 = (double)(1.0f / (float)a1), e0 = fma(-a1, y0, 1.0);
-              const double c2 = fma(y0, fma(e0, e0, e0), y0);        // an FP32 seed, a third-order step: 1 / a1
+              const double c2 = inverse(a1);
               const double mine = odd ? be : al, his = odd ? al : be;
               const double nrm = c2 * fma(t2, his, fma(odd ? 2.0 : -2.0, rg, mine));
               // a quarter: two less in the exponent field
