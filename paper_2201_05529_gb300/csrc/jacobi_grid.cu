@@ -26,9 +26,11 @@
 //     no round can use leave at once, so small layers pay for small barriers.
 // Before (one 512-thread CTA per SM, b = 2, columns in L2, each pair's scalars on one lane in FP64 with two sqrt /
 // rsqrt chains, 5800 cycles; now 1900) -> with a grid barrier per round -> with the blocks' own counters and a pair's two
-// norms, scales and factors on two lanes: two 256 x 256 SVDs 112 ms (clusters) -> 31.6 -> 27.9, the three-site chain's
-// first eight steps 51.8 -> 34.6 -> 33.5 ms, the five-site chain's 219 -> 180 -> 150 ms, the 21-site chain's first four
-// on the tensor-core path 905 -> 651 (451 with the other kernels' later changes) -> 438 ms.
+// norms, scales and factors on two lanes -> with fixed-point sums, no divisions and a fitted choice of b: two 256 x 256
+// SVDs without QRs before them 112 ms (clusters) -> 31.6 -> 27.9 -> 27; the five-site chain's first eight steps 219 -> 180
+// -> 150 -> (with the new pivoted QR 131) 117 ms, the 16 chains' first four 300 -> 177 -> 176 -> (138) 118 ms, the 21-site
+// chain's first four on the tensor-core path 990 -> 451 -> 438 -> (417) 414 ms. A sweep now: 64 x 64 0.16 ms, two 136 x
+// 136 0.48, 64 of 80 x 80 0.72, two 256 x 256 with V 1.3.
 //
 // Sums are combined in a fixed order, so results are bitwise reproducible. Every barrier wait has a time
 // limit: on expiry the kernel records ST_TIMEOUT, raises an abort flag that releases every other CTA, and
@@ -155,16 +157,19 @@ __device__ __forceinline__ void store_relaxed(int* p, int v) {
 constexpr int MIN_SCALE_HI = (1023 - 64) << 20;    // below 2^-64 a squared scale is multiplied into its column
 
 // columns per block: the b in {1, 2, 4, 8} that fits cols_max columns and whose sweep is shortest by the cost of
-// its terms in cycles: per sub-round the scalars and reductions (2500 cycles, shared by the tasks of an SM) and 19
-// cycles per FP64 warp instruction of the SM's tasks; per round the transfer of a task's columns and its waits.
-// Costs estimated from the measured FP64 issue rate and barrier; the choice only moves a few percent around them.
+// its terms in cycles: per sub-round the scalars and reductions (2000 cycles, shared by the tasks of an SM) and 13.5
+// cycles per FP64 warp instruction of the SM's tasks; per round the waits and lookups (6100) and the transfer of a task's
+// columns (2.6 per row). The constants are fitted to the time of a sweep at every b, measured for 16 x 16, two 32 x 32, 64 x
+// 64 (1 and 24), 100 x 100 (2), 136 x 136 (2), 80 x 80 (64), 160 x 160 (10) and, with V, 128 x 128 and 256 x 256 (2): the
+// model finds the shortest one in each. An estimate from the issue rate alone (19 cycles, 2500 and 3500) took b = 2 for
+// ten 160 x 160 (1.31 ms a sweep, 0.75 at b = 8) and for one 64 x 64 (0.19, 0.16 at b = 4).
 // One warp computes it; every lane gets the result.
 __device__ int choose_block(const int* s_Na, const int* s_Ma, int n_work, int slots, int sms, int cols_max,
                             bool with_v, int lane) {
   int best = 1;
   float best_t = 3e38f;
   for (int b = 1; b <= JB && 2 * b <= cols_max; b <<= 1) {
-    int tasks = 0, rounds = 0, rows = 0, most_nb = 0;
+    int tasks = 0, rounds = 0, rows = 0, len = 0, most_nb = 0;
     for (int w = lane; w < n_work; w += 32) {
       if (s_Na[w] < 2) continue;
       const int nb = (s_Na[w] + b - 1) / b, nbp = nb + (nb & 1);
@@ -173,18 +178,20 @@ __device__ int choose_block(const int* s_Na, const int* s_Ma, int n_work, int sl
       rounds = max(rounds, nbp - 1);
       // FP64 operations per pair: 4 per row for the inner product, 8 per row (and row of V) for the rotation
       rows = max(rows, 12 * s_Ma[w] + (with_v ? 8 * s_Na[w] : 0));
+      len = max(len, s_Ma[w] + (with_v ? s_Na[w] : 0));
     }
     tasks = __reduce_add_sync(0xffffffffu, tasks);
     rounds = __reduce_max_sync(0xffffffffu, rounds);
     rows = __reduce_max_sync(0xffffffffu, rows);
+    len = __reduce_max_sync(0xffffffffu, len);
     most_nb = __reduce_max_sync(0xffffffffu, most_nb);
     if (tasks == 0) return 1;
     const float per_sm = (float)((tasks + sms - 1) / sms), waves = (float)((tasks + slots - 1) / slots);
-    const float fp = 19.f * b * (float)((rows + 31) / 32);
-    const float sub = fmaxf(waves * 2500.f + fp, per_sm * fp + 1500.f);
-    const float move = 1000.f + per_sm * b * (float)rows * 0.1f;
+    const float fp = 13.5f * b * (float)rows * (1.f / 32.f);
+    const float sub = fmaxf(waves * 2000.f + fp, per_sm * fp + 2000.f);
+    const float move = waves * 6100.f + per_sm * b * (float)len * 2.6f;
     // one block only: no cross pairs
-    const float t = most_nb < 2 ? (b - 1) * sub : rounds * ((float)b * sub + move + 2500.f) + (b - 1) * sub;
+    const float t = most_nb < 2 ? (b - 1) * sub : rounds * ((float)b * sub + move) + (b - 1) * sub;
     if (t < best_t) {
       best_t = t;
       best = b;
