@@ -449,9 +449,9 @@ def run_ours(args, rank, world, local):
         n_qr = (1 + RSVD_POWER) + (RSVD_POWER + 1)          # QR launches per layer
         qr_ms = stage[7] / K / n_layers / n_qr              # per launch
         achieved = (fl_qr / (K * n_layers * n_qr)) / (qr_ms / 1e3) / 1e12
-        traffic, tsrc = traffic_record(["hqr_grid.cu"], sketch_elements(blog) / (K * n_layers * n_qr))
-        roofline = {"bound": "alu", "kernel": "k_hqr_items: whole-GPU Householder QR (explicit Q) of the randomized "
-                                              "range finder's sketches Y (m x l) and Z (n x l) of every bond of a layer",
+        traffic, tsrc = traffic_record(["qr_block.cu", "tc_zgemm.cu"], sketch_elements(blog) / (K * n_layers * n_qr))
+        roofline = {"bound": "alu", "kernel": "blocked Householder QR (k_qr_panel on the FP64 pipe, the rest nine-slice tensor-core "
+                                              "products; explicit Q) of the range finder's sketches Y (m x l) and Z (n x l)",
                     "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s", "frac": achieved / fp64_peak,
                     "traffic": traffic, "traffic_source": tsrc,
                     "work": "16 (m l^2 - l^3 / 3) per m x l QR with its explicit Q (GVL, complex = 4 real), "
@@ -465,7 +465,7 @@ def run_ours(args, rank, world, local):
         # the sliced tensor-core products (the fast path's dense contractions)
         gemm_s = stage[8] / 1e3
         roofline["tensor_products"] = {
-            "kernel": "k_zgemm (+ k_zg_rowexp / k_zg_pack): D Omega, D^H Q, D Qz, D - Q Z^H, Q Wr, Qb Ur",
+            "kernel": "k_zgemm (+ k_zg_prep): D Omega, D^H Q, D Qz, D - Q Z^H, Q Wr, Qb Ur",
             "bound": "tensor", "achieved": fl_gemm / gemm_s / 1e12, "peak": bf16, "unit": "TFLOP/s",
             "frac": fl_gemm / gemm_s / 1e12 / bf16,
             "achieved_executed_bf16": 21.0 * fl_gemm / gemm_s / 1e12,

@@ -109,8 +109,9 @@ typedef struct {
                                      capacity, and keep the fastest (0: a fixed default order) */
   const char* tune_cache;         /* text file of tuned choices (read, appended), or NULL */
   int force_route;                /* 0: tuned or default; else 1 + qr + 4 k2 for every layer, with qr
-                                     0 whole-GPU / 1 cluster shared-memory / 2 cluster global-memory
-                                     pivoted QR, k2 0 whole-GPU / 1 one-CTA-per-block outer QR
+                                     1 the largest cluster per matrix / 2 clusters by the number of
+                                     matrices for the pivoted QR (0, a name of saved choices: as 1,
+                                     where a layer's columns fit one per warp), k2 0 whole-GPU / 1 one-CTA-per-block outer QR
                                      (PT_ERR_ARG where it does not fit) */
 } pt_options;
 
@@ -227,14 +228,18 @@ int pt_tebd_get_timing(pt_tebd_t h, double* ms9);
 /* Batched FP64 SVD (the one-sided Jacobi of the bond update, App. A.2) of `batch` complex
  * matrices A_b [m][n] row-major (device). Writes singular values sigma [batch][min(m,n)]
  * (descending), U [batch][m][min(m,n)] and V [batch][n][min(m,n)] (device, row-major), so
- * A_b = U diag(sigma) V^H. scratch: device workspace of pt_svd_scratch_bytes(m, n, batch) bytes.
+ * A_b = U diag(sigma) V^H. Larger matrices (min(m, n) from 96, or from 32 where the other side is four
+ * times as long) go through two QRs before the Jacobi; where those find NaN or the Jacobi then does not
+ * converge, the call repeats without them. scratch: device workspace of pt_svd_scratch_bytes(m, n, batch)
+ * bytes. PT_ERR_DEVICE_TIMEOUT: a bounded barrier wait.
  * Returns PT_ERR_SVD_NOCONV if a matrix did not converge within max_sweeps. */
 size_t pt_svd_scratch_bytes(int m, int n, int batch);
 int pt_svd_f64(const double* A, int m, int n, int batch, double* sigma, double* U, double* V,
                void* scratch, int max_sweeps, void* cuda_stream);
 
-/* Batched FP64 Householder QR with the explicit Q (the whole-GPU kernel of the outer-block
- * reductions, App. A.2, and of the fast path's range finder): A_b (m x n complex,
+/* Batched FP64 Householder QR with the explicit Q (of the outer-block reductions, App. A.2, and of
+ * the fast path's range finder: one CTA for a small matrix, else panels by clusters and tensor-core
+ * updates, the unblocked whole-GPU kernel where a panel does not fit): A_b (m x n complex,
  * column-major, 1 <= n <= m, b < batch, contiguous) is replaced by Q_b (m x n, orthonormal columns),
  * R_b (n x n, column-major, upper triangular) is written, A_b(in) = Q_b R_b. scratch: device workspace
  * of pt_qr_scratch_bytes(m, n, batch) bytes. Synchronous. Errors: PT_ERR_ARG, PT_ERR_CAPACITY
@@ -261,10 +266,10 @@ int pt_zgemm_sliced(int opA, int opB, int m, int n, int k, const double* A, int 
  * For callers that cannot allocate device memory: their device memory is owned by another pool
  * (a framework that reserves the GPU up front, a fixed-budget service), or a device allocation is
  * not acceptable where they run (cudaMalloc may synchronise the device and can fail mid-job).
- * Same batched FP64 Jacobi SVD and the same arguments and outputs as pt_svd_f64, minus the
- * scratch pointer: the workspace is a static device array of PT_SVD_NOALLOC_MAX_BYTES bytes that
- * every GPU which loads this library holds until the process exits. A problem whose workspace
- * (pt_svd_scratch_bytes(m, n, batch)) is larger is rejected with PT_ERR_CAPACITY. The first call on
+ * The batched FP64 Jacobi SVD without QRs before it, the same arguments and outputs as pt_svd_f64, minus
+ * the scratch pointer: the workspace is a static device array of PT_SVD_NOALLOC_MAX_BYTES bytes that
+ * every GPU which loads this library holds until the process exits. A problem whose workspace (16
+ * bytes per element of A and of a min(m, n) x min(m, n) factor, 20 per column, a few hundred per matrix) is larger is rejected with PT_ERR_CAPACITY. The first call on
  * a device looks up the array's device address with that device current and caches it per device
  * index (a cudaDeviceReset invalidates it). All calls share the one array: calls that overlap on the
  * GPU race and corrupt each other, so the caller must serialise them. Each call clears what must

