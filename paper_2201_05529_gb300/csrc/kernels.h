@@ -164,7 +164,8 @@ struct ZGemmItem {
   int skip_b;              // 1: B's are already in TB, or another item of the launch writes them there
   const double2* A2;       // rows a_split .. M - 1 of opA(A) come from A2 (same op and leading dimension); NULL: all from A
   int a_split;
-  long long split;         // > 0: each K chunk's product goes to C + chunk * split (chunks of zgemm9_chunks)
+  long long split;         // > 0: each K chunk's product goes to C + chunk * split (zgemm9_chunks of them)
+  int split_ks;            // the chunks' length in steps of 16 of K (0: the longest)
 };
 struct SvdQrHost {
   std::vector<QRItem> qr;
@@ -184,7 +185,8 @@ void launch_zgemm(const ZGemmItem* items, int n_items, int tile_cap, int m_cap_m
 // term, one FP64 rounding per 256-long chunk of K, the chunks added in FP64). Its operands' packed sizes, the
 // number of K chunks; unit_cap: output tiles (128 x 32), times the chunks where items are split
 size_t zgemm9_pack_bytes(int rows_cap, int k_cap, int which);
-int zgemm9_chunks(int k);
+constexpr int Z9_KSTEPS = 16;   // the longest chunk, in steps of 16 of K
+inline int zgemm9_chunks(int k) { return ((k < 1 ? 1 : k) + 16 * Z9_KSTEPS - 1) / (16 * Z9_KSTEPS); }
 void launch_zgemm9(const ZGemmItem* items, int n_items, long long unit_cap, int m_cap_max, int n_cap_max, int k_cap_max,
                    int* status, cudaStream_t st);
 // the most items one launch_zgemm takes

@@ -36,6 +36,7 @@ constexpr int PANEL_T = PT + 32;           // and a warp for the scalars
 constexpr int SMALL_N = 32;                // columns of a matrix that one CTA factors whole
 constexpr int MAX_C = 16;                  // CTAs per cluster
 constexpr int PANEL_SMEM = 200 * 1024;     // panel rows of one CTA (227 KB less the exchange buffers)
+constexpr int MAX_PARTS = 16;               // K chunks of a product W, unless chunks of the longest kind are more
 constexpr int WT_ROWS = 8;                 // rows of W per block of k_qr_wt, one warp each
 
 // lane 0 ends with the total of a, lane 16 with the total of b
@@ -56,6 +57,26 @@ __device__ __forceinline__ double2 group_sum(double a, double b, int L, bool hal
   return half ? make_double2(other, s) : make_double2(s, other);
 }
 
+// Length of the K chunks of W = A^H V (steps of 16) for n_items products of `cols` rows: the shortest estimate, waves of
+// units over the SMs times (steps + 2.5 for a unit's start and epilogue). 256-long chunks alone leave few units for few
+// matrices and a second, nearly empty wave for others (160 units of ten 2048 x 160 on 152 SMs): two 256 x 256 QRs 2.54 ->
+// 2.36 ms, ten 1120 x 160 3.22 -> 3.05, the 21-site chain's first four steps 410 -> 388.
+__device__ __forceinline__ int split_steps(int n_items, int cols, int k, int sms) {
+  const int ks = (k + 15) / 16, tiles = n_items * ((cols + 127) / 128);
+  int best = Z9_KSTEPS;
+  float cost = 3e38f;
+  for (int c = Z9_KSTEPS; c >= 1; --c) {
+    const int parts = (ks + c - 1) / c;
+    if (parts > MAX_PARTS && c < Z9_KSTEPS) break;
+    const float t = (float)((tiles * parts + sms - 1) / sms) * ((float)min(c, ks) + 2.5f);
+    if (t < cost) {
+      cost = t;
+      best = c;
+    }
+  }
+  return best;
+}
+
 __device__ __forceinline__ bool live(const QRItem& q) { return q.m > 0 && q.n > 0 && q.n <= q.m; }
 
 }  // namespace
@@ -64,7 +85,7 @@ __device__ __forceinline__ bool live(const QRItem& q) { return q.m > 0 && q.n > 
 // one thread per (matrix, panel). ops: per panel n each of forward W and S (one product: the rows of [A2, V_p]^H V_p),
 // forward update, backward W, backward update.
 __global__ void k_qrb_plan(Tables T, const BondWork* work, const QRItem* list, QRBlk* blk, int n_items, int panels,
-                           ZGemmItem* ops, int* status) {
+                           ZGemmItem* ops, int sms, int* status) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n_items * panels) return;
   const int i = idx % n_items, p = idx / n_items;
@@ -110,6 +131,7 @@ __global__ void k_qrb_plan(Tables T, const BondWork* work, const QRItem* list, Q
       it.cap_n = NB;
       it.cap_k = B.m_cap;
       it.split = (long long)it.ldc * NB;
+      it.split_ks = split_steps(n_items, M, rows, sms);
       return it;
     };
     auto outer = [&](double2* C, int N) {
@@ -344,7 +366,7 @@ __global__ void __launch_bounds__(PANEL_T, 1) k_qr_panel(const QRBlk* blk, int n
 // X = W T (forward) or W T^H (backward) from the parts of W, eight rows per block, one warp per row: x_k = tau_k (w_k -
 // sum_{i < k} x_i S_ik), or from the last column up with conj(S_ki). Forward also adds S's parts, the rows below
 // W's (kept for backward). S is scaled by tau_i first, so a step of the solve is four FP64 operations of a warp.
-__global__ void __launch_bounds__(32 * WT_ROWS) k_qr_wt(const QRBlk* blk, int n_items, int p, int backward) {
+__global__ void __launch_bounds__(32 * WT_ROWS) k_qr_wt(const QRBlk* blk, const ZGemmItem* ops, int p, int backward) {
   __shared__ double2 s_s[NB][NB + 1];
   __shared__ double2 s_w[WT_ROWS][NB + 1];
   const int i = blockIdx.y;
@@ -355,7 +377,7 @@ __global__ void __launch_bounds__(32 * WT_ROWS) k_qr_wt(const QRBlk* blk, int n_
   const int n_rows = backward ? q.n - row0 : q.n - row0 - NB;
   const int r0 = blockIdx.x * WT_ROWS;
   if (r0 >= n_rows && (backward || blockIdx.x > 0)) return;
-  const int nch = (((q.m - row0 + 15) / 16) + 15) / 16;        // K chunks of 256
+  const int ks = ops[i].split_ks, nch = ((q.m - row0 + 15) / 16 + ks - 1) / ks;      // W's K chunks
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const size_t ldw = B.n_cap + NB, chunk = ldw * NB;
   double2* S = B.S + (size_t)p * NB * NB;
@@ -608,7 +630,7 @@ size_t qr_block_bytes(int m, int n, QRBlk* B, char* base) {
     o += up(bytes);
     return r;
   };
-  const size_t ch = zgemm9_chunks(m), pn = (n + NB - 1) / NB;
+  const size_t ch = std::max(zgemm9_chunks(m), std::min(MAX_PARTS, (m + 15) / 16)), pn = (n + NB - 1) / NB;
   QRBlk b{};
   b.m_cap = m;
   b.n_cap = n;
@@ -637,9 +659,13 @@ size_t qr_block_ops(int n_items, int n_cap) { return (size_t)4 * n_items * ((n_c
 void launch_qr_block(const Tables& T, const BondWork* work, const QRItem* list, const QRBlkList& L, int* status,
                      cudaStream_t st) {
   const int n = L.n_items, panels = (L.n_cap + NB - 1) / NB;
-  k_qrb_plan<<<(n * panels + 127) / 128, 128, 0, st>>>(T, work, list, L.blk, n, panels, L.ops, status);
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  k_qrb_plan<<<(n * panels + 127) / 128, 128, 0, st>>>(T, work, list, L.blk, n, panels, L.ops, std::max(1, sms), status);
   const int rc = (L.m_cap + L.cluster - 1) / L.cluster;
-  const long long ch = zgemm9_chunks(L.m_cap);
+  const long long ch = std::max(zgemm9_chunks(L.m_cap), MAX_PARTS);
+
   auto tiles = [](int m, int k) { return (long long)((m + 127) / 128) * ((k + 31) / 32); };
   for (int p = 0; p < panels; ++p) {
     cudaLaunchAttribute at[1];
@@ -648,7 +674,7 @@ void launch_qr_block(const Tables& T, const BondWork* work, const QRItem* list, 
     const ZGemmItem* o = L.ops + (size_t)p * 4 * n;
     const int trail = std::max(0, L.n_cap - (p + 1) * NB), rows = std::max(1, L.m_cap - p * NB);
     launch_zgemm9(o, n, tiles(trail + NB, 1) * ch * n, trail + NB, NB, L.m_cap, status, st);
-    k_qr_wt<<<dim3(std::max(1, (trail + WT_ROWS - 1) / WT_ROWS), n), 32 * WT_ROWS, 0, st>>>(L.blk, n, p, 0);
+    k_qr_wt<<<dim3(std::max(1, (trail + WT_ROWS - 1) / WT_ROWS), n), 32 * WT_ROWS, 0, st>>>(L.blk, o, p, 0);
     if (trail > 0) launch_zgemm9(o + n, n, tiles(rows, trail) * n, rows, trail, NB, status, st);
   }
   k_qr_identity<<<dim3(std::min(64, (L.m_cap * std::min(L.n_cap, 64) + 255) / 256), n), 256, 0, st>>>(L.blk, n);
@@ -656,7 +682,7 @@ void launch_qr_block(const Tables& T, const BondWork* work, const QRItem* list, 
     const ZGemmItem* o = L.ops + (size_t)p * 4 * n;
     const int cols = L.n_cap - p * NB, rows = std::max(1, L.m_cap - p * NB);
     launch_zgemm9(o + 2 * n, n, tiles(cols, 1) * ch * n, cols, NB, L.m_cap, status, st);
-    k_qr_wt<<<dim3((cols + WT_ROWS - 1) / WT_ROWS, n), 32 * WT_ROWS, 0, st>>>(L.blk, n, p, 1);
+    k_qr_wt<<<dim3((cols + WT_ROWS - 1) / WT_ROWS, n), 32 * WT_ROWS, 0, st>>>(L.blk, o + 2 * n, p, 1);
     launch_zgemm9(o + 3 * n, n, tiles(rows, cols) * n, rows, cols, NB, status, st);
   }
 }

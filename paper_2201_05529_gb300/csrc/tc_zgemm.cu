@@ -55,7 +55,7 @@ struct Z6 {
   }
 };
 struct Z9 {
-  static constexpr int NS = 9, NLEV = 8, TN = 32, KC = 16;
+  static constexpr int NS = 9, NLEV = 8, TN = 32, KC = Z9_KSTEPS;
   // two words: levels 0..3 in units of 2^-35, the rest in units of 2^-70, one FP64 addition
   static __device__ __forceinline__ double value(const float (&f)[NLEV][8], int j, int e, bool neg) {
     const long long h = level_sum<0, 3, 35, 0>(f, j), l = level_sum<4, 7, 70, 65>(f, j);
@@ -240,7 +240,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) k_zgemm(const ZGemmItem* item
     if (blockIdx.x == 0 && tid == 0) atomicOr(status, ST_CAPACITY);
     return;
   }
-  auto n_chunks = [](const ZGemmItem& it) { return it.split > 0 ? cdiv(cdiv(it.K, ZG::KSTEP), KC) : 1; };
+  auto chunk_ks = [](const ZGemmItem& it) { return it.split_ks > 0 ? min(it.split_ks, KC) : KC; };
+  auto n_chunks = [&](const ZGemmItem& it) { return it.split > 0 ? cdiv(cdiv(it.K, ZG::KSTEP), chunk_ks(it)) : 1; };
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   for (int i = tid; i < n_items; i += blockDim.x) {
     const ZGemmItem& it = items[i];
@@ -301,8 +302,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) k_zgemm(const ZGemmItem* item
     U.rt = tile / nt_b;
     U.ct = tile % nt_b;
     const int n_ks = cdiv(U.it->K, ZG::KSTEP);
-    U.ks_from = U.it->split > 0 ? U.chunk * KC : 0;
-    U.ks_to = U.it->split > 0 ? min(n_ks, U.ks_from + KC) : n_ks;
+    U.ks_from = U.it->split > 0 ? U.chunk * chunk_ks(*U.it) : 0;
+    U.ks_to = U.it->split > 0 ? min(n_ks, U.ks_from + chunk_ks(*U.it)) : n_ks;
     return U;
   };
   bool ok = true;
@@ -435,7 +436,6 @@ size_t zgemm9_pack_bytes(int rows_cap, int k_cap, int which) {
                   which == 0 ? 0 : 3 * Z9::NS).total;
 }
 
-int zgemm9_chunks(int k) { return cdiv(cdiv(std::max(1, k), ZG::KSTEP), Z9::KC); }
 
 int zgemm_max_items() { return MAX_ITEMS; }
 
