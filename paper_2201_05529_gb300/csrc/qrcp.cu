@@ -219,7 +219,7 @@ __device__ __forceinline__ void qrcp_run(const BondWork& W, int Ma, int Na, int 
       // the instructions of a sub-partition: ten per row and about twelve besides, three per reduction step
       int best = 0x7fffffff;
 #pragma unroll
-      for (int lg = 2; lg <= 5; ++lg) {
+      for (int lg = GL ? 4 : 2; lg <= 5; ++lg) {          // from L2 in runs of 256 bytes or more
         const int warps = ((((na << lg) + 31) >> 5) + 3) >> 2;
         const int cost = warps * (10 * ((rows + (1 << lg) - 1) >> lg) + 3 * lg + 12);
         if (cost < best) {
@@ -239,12 +239,25 @@ __device__ __forceinline__ void qrcp_run(const BondWork& W, int Ma, int Na, int 
       const bool on = l >= 0 && l != own;
       double2* a = on ? colp(l) : nullptr;
       double sr = 0, si = 0;
-      if (on)
-        for (int r = j + 1 + ln; r < Ma; r += L) {
+      if (on) {
+        int r = j + 1 + ln;
+        for (; r + 3 * L < Ma; r += 4 * L) {      // four rows' loads in flight
+          double2 v[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) v[q] = ld(a + r + q * L);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const double2 u = hv[r + q * L];
+            sr = fma(u.x, v[q].x, fma(u.y, v[q].y, sr));
+            si = fma(u.x, v[q].y, fma(-u.y, v[q].x, si));
+          }
+        }
+        for (; r < Ma; r += L) {
           const double2 u = hv[r], v = ld(a + r);
           sr = fma(u.x, v.x, fma(u.y, v.y, sr));
           si = fma(u.x, v.y, fma(-u.y, v.x, si));
         }
+      }
       // real parts to the lower half of the group, imaginary parts to the upper, then both to all
       const bool up = ln >= (L >> 1);
       double s = (up ? si : sr) + __shfl_xor_sync(0xffffffffu, up ? sr : si, L >> 1);
@@ -264,7 +277,21 @@ __device__ __forceinline__ void qrcp_run(const BondWork& W, int Ma, int Na, int 
         aj = ld(a + j);
         const double wr = fma(vj.x, aj.x, fma(vj.y, aj.y, sr)), wi = fma(vj.x, aj.y, fma(-vj.y, aj.x, si));
         const double tr = kap * wr, ti = kap * wi;
-        for (int r = j + 1 + ln; r < Ma; r += L) {
+        int r = j + 1 + ln;
+        for (; r + 3 * L < Ma; r += 4 * L) {
+          double2 v[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) v[q] = ld(a + r + q * L);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const double2 u = hv[r + q * L];
+            v[q].x = fma(-u.x, tr, fma(u.y, ti, v[q].x));
+            v[q].y = fma(-u.x, ti, fma(-u.y, tr, v[q].y));
+            st(a + r + q * L, v[q]);
+            nn = fma(v[q].x, v[q].x, fma(v[q].y, v[q].y, nn));
+          }
+        }
+        for (; r < Ma; r += L) {
           const double2 u = hv[r];
           double2 v = ld(a + r);
           v.x = fma(-u.x, tr, fma(u.y, ti, v.x));
@@ -460,14 +487,17 @@ long long qr_x_elems(int c, int m_cap, int n_cap) {
 
 // CTAs per matrix for n_work matrices: the shortest estimate of a step, the waves of clusters times (4000 cycles of
 // latency + the arithmetic of a third of a matrix of half the capacities, ten instructions of 19 cycles per 32 entries,
-// over the cluster). Whether a matrix stays in shared memory is seen on the device from its live size.
+// over the cluster), for matrices of equal size and for a quarter of them large (a correlation front): the waves of both
+// are added. Equal sizes alone took 10 CTAs for a layer of ten with two of 592 x 592 (280000 cycles a step). Whether a
+// matrix stays in shared memory is seen on the device from its live size.
 int qr_pick_cluster(int n_work, int m_cap, int n_cap) {
   const QrClusters& t = qr_clusters();
   int best = 0;
   double cost = 1e300;
   for (int c = 1; c <= QR_MAX_C; ++c) {
     if (t.active[c] <= 0 || qr_x_elems(c, m_cap, n_cap) < 0) continue;
-    const double v = (double)((n_work + t.active[c] - 1) / t.active[c]) *
+    const int quarter = (n_work + 3) / 4;
+    const double v = (double)((n_work + t.active[c] - 1) / t.active[c] + (quarter + t.active[c] - 1) / t.active[c]) *
                      (4000.0 + 19.0 * 10.0 / 32.0 / 3.0 * (0.5 * n_cap) * (0.5 * m_cap) / c);
     if (v < cost) {
       cost = v;
