@@ -391,15 +391,17 @@ __global__ void __launch_bounds__(32 * WT_ROWS) k_qr_wt(const QRBlk* blk, const 
     return v;
   };
   // s_s[c][k]: tau_c S_ck (forward, k > c) or tau_c conj(S_kc) (backward, k < c)
-  for (int e = tid; e < NB * NB; e += blockDim.x) {
-    const int a = e % NB, b = e / NB;          // S_ab, a < b
-    if (a >= b || b >= nc) continue;
+  // S_ab, a < b: a warp takes column 16 + i and column 15 - i (an FP64 instruction takes as long
+  // for half a warp's lanes)
+  for (int e = tid; e < NB * NB / 2; e += blockDim.x) {
+    const int l = e % NB, d = NB / 2 + e / NB, a = l < d ? l : NB - 1 - l, b = l < d ? d : NB - 1 - d;
+    if (l == d || b >= nc) continue;
     double2 v;
     if (backward) {
-      v = S[e];
+      v = S[a + b * NB];
     } else {
       v = sum(max(0, n_rows) + a + (size_t)b * ldw);
-      if (blockIdx.x == 0) S[e] = v;
+      if (blockIdx.x == 0) S[a + b * NB] = v;
     }
     const double t = q.tau[row0 + (backward ? b : a)];
     if (backward) s_s[b][a] = make_double2(v.x * t, -v.y * t);
