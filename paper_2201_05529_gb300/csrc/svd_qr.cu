@@ -167,9 +167,10 @@ size_t svd_qr_layout(int Ma, int Na, int batch, SvdQr* out, char* base) {
 
 // From 96 columns on, or from 32 where the matrix is at least four times as long; the blocked QR's panel has to fit and
 // the two products of every matrix have to go into one launch. Measured with the direct call beside it, singular values
-// over four decades: 64 x 64 2.9 against 3.5 ms, 96 x 96 4.9 / 6.7, four 128 x 128 7.2 / 10.2, 256 x 256 20.3 / 31.2, two
-// 256 x 64 3.1 / 4.9, two 1000 x 40 2.4 / 4.8; with random entries, columns graded over four decades, the Jacobi alone is
-// quick as well: 64 x 64 2.9 / 2.1, ten 160 x 160 14.5 / 15.3, two 256 x 256 15.6 / 15.5.
+// over four decades: 96 x 96 4.0 against 5.5 ms, four 128 x 128 6.2 / 8.7, 256 x 256 14.8 / 24.7, two 256 x 64 2.7 / 4.6,
+// two 1000 x 40 2.0 / 4.5 (64 x 64 gained a fifth with QRs of 2.9 ms). With random entries and columns graded over four
+// decades the Jacobi alone is quick as well: 96 x 96 4.0 / 3.0, ten 160 x 160 10.2 / 10.3, two 256 x 256 14.3 / 13.9; a
+// line further down would lose more there than a bond's matrix gains.
 bool svd_qr_fits(int Ma, int Na, int batch) {
   return (Na >= 96 || (Na >= 32 && Ma / 4 >= Na)) && 2LL * batch <= zgemm_max_items() &&
          qr_block_cluster(batch, Ma) > 0 && qr_block_cluster(batch, Na) > 0;
