@@ -174,8 +174,9 @@ __global__ void k_qrb_plan(Tables T, const BondWork* work, const QRItem* list, Q
 // reflector's scalars from those of s_j; then they apply w_k = tau u^H a_k to their column. An FP64 instruction takes 64
 // cycles of a sub-partition whatever its lanes: so columns share warps where there are many (L = 4 or 8: fewer
 // reduction steps than a warp per column has), the scalars' square roots go to two lanes of one instruction and start from
-// FP32. Cycles per reflector besides the rows' arithmetic: 15000 with all of it done by every warp for its own columns ->
-// 6000 with one warp for the sums over CTAs and the scalars of all columns -> 4000 so.
+// FP32. Two matrices of 256 rows on 16 CTAs each: 10400 cycles per reflector with one warp for the sums over CTAs and the
+// scalars of all columns (which had come down from ~15000 besides the rows' arithmetic, all of it done by every warp for
+// its own columns), 7100 so; ten of 1120 rows, mostly the rows' arithmetic, 292 us a panel.
 __global__ void __launch_bounds__(PANEL_T, 1) k_qr_panel(const QRBlk* blk, int n_items, int p, int rc_cap, int* status) {
   extern __shared__ __align__(16) double2 s_p[];
   __shared__ double2 s_part[2][MAX_C][NB];
