@@ -253,8 +253,10 @@ int pt_qr_f64(double* A, int m, int n, int batch, double* R, void* scratch, void
  * (in complex elements) and batch stride (in complex elements); op: 0 as stored, 1 transposed,
  * 2 conjugate transposed. Arithmetic: each row of opA(A) and column of opB(B) is scaled by a power
  * of two and cut into six BF16 fixed-point slices; slice products accumulate in FP32 on the
- * tcgen05 tensor cores (exactly for the two leading levels) and are summed in FP64, so C is
- * accurate to ~1e-12 of max|row of opA(A)| x max|column of opB(B)|. scratch: device workspace of
+ * tcgen05 tensor cores (exactly for the two leading levels) and are summed as 64-bit integers, so C is
+ * accurate to ~1e-12 of max|row of opA(A)| x max|column of opB(B)|; where an entry's terms add up
+ * coherently down to their last slices (constant operands), the FP32 accumulation truncates to
+ * 1.2e-10 k of that. scratch: device workspace of
  * pt_zgemm_scratch_bytes(m, n, k, batch) bytes. Synchronous. Errors: PT_ERR_ARG (bad sizes, op or
  * leading dimension, batch > 1024), PT_ERR_DEVICE_TIMEOUT (a bounded pipeline wait expired). */
 size_t pt_zgemm_scratch_bytes(int m, int n, int k, int batch);

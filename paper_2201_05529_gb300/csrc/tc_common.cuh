@@ -352,16 +352,41 @@ __device__ __forceinline__ double fixed_to_double(long long n, int e, int lsb) {
   return ldexp((double)n, e - lsb);
 }
 
+// the largest sum of a level's slice pairs over `terms` products, in units of 2^(-7 (L + 2)): |a_0| <= 2^7, |a_i| <= 2^6
+__host__ __device__ constexpr long long level_max(int L, int NS, long long terms) {
+  long long n = 0;
+  for (int s = 0; s <= L; ++s)
+    if (s < NS && L - s < NS) n += (s == 0 ? 128 : 64) * (s == L ? 128 : 64);
+  return n * terms;
+}
+// the same of levels L .. NS - 1 together, in units of 2^-u
+__host__ __device__ constexpr double levels_max(int L, int NS, long long terms, int u) {
+  double n = 0;
+  for (int t = L; t < NS; ++t) {
+    double v = (double)level_max(t, NS, terms);
+    for (int q = 7 * (t + 2); q < u; ++q) v *= 2;
+    for (int q = u; q < 7 * (t + 2); ++q) v /= 2;
+    n += v;
+  }
+  return n;
+}
+
 // the sum of levels FROM .. TO of an entry's accumulators (slice width 7) as an integer multiple of 2^-LSB: level L holds
-// integer multiples of 2^(-7 (L + 2)) below 2^24 of them. LAST > 0: the last level, shared by several, is rounded to
-// multiples of 2^-LAST, which fit 32 bits.
-template <int FROM, int TO, int LSB, int LAST, int NLEV>
+// integer multiples of 2^(-7 (L + 2)), of TERMS products a pair. LAST > 0: the last level, shared by several, is rounded to
+// multiples of 2^-LAST. A 32-bit conversion clamps, so it is taken only where the digits' largest sum fits (entries of
+// coherent operands come near it; the 64-bit one costs 1 % of a 300 x 70 x 530 or 16384 x 64 x 64 product).
+template <int FROM, int TO, int LSB, int LAST, int NS, int TERMS, int NLEV>
 __device__ __forceinline__ long long level_sum(const float (&f)[NLEV][8], int j) {
+  static_assert(levels_max(FROM, NS, TERMS, LSB) < 9e18, "the sum fits 63 bits");
   long long n = 0;
 #pragma unroll
   for (int L = FROM; L <= TO; ++L) {
-    const int u = LAST > 0 && L == TO ? LAST : 7 * (L + 2);
-    n += (long long)__float2int_rn(f[L][j] * __uint_as_float((uint32_t)(127 + u) << 23)) * (1ll << (LSB - u));
+    const bool last = LAST > 0 && L == TO;
+    const int u = last ? LAST : 7 * (L + 2);
+    const float x = f[L][j] * __uint_as_float((uint32_t)(127 + u) << 23);
+    const double most = last ? levels_max(L, NS, TERMS, u) : (double)level_max(L, NS, TERMS);
+    // less 2^12 for what the accumulation's own rounding adds
+    n += (most < 2147483648.0 - 4096.0 ? (long long)__float2int_rn(x) : __float2ll_rn(x)) * (1ll << (LSB - u));
   }
   return n;
 }

@@ -17,7 +17,8 @@
 // pairs (s, t) accumulate in TMEM by level min(s + t, 3), real and imaginary parts separately
 // (Re = Ar Br - Ai Bi via the MMA's negate-A bit, Im = Ar Bi + Ai Br); the epilogue adds the
 // levels as 64-bit integers and applies 2^(e_row + e_col). The result is accurate to ~1e-12 of the scale
-// of the rows and columns it combines (per 512-long chunk of K).
+// of the rows and columns it combines (per 512-long chunk of K); where the terms of an entry add up coherently, in the
+// slices too (constant operands), the FP32 accumulation of the deeper levels truncates to 1.2e-10 of K times that scale.
 //
 // Data flow: one preparation launch (row exponents, then the 12 slice planes in the tcgen05
 // K-major no-swizzle layout: A in 128-row tiles, B in 64-column tiles, one 16-element K step per
@@ -50,15 +51,16 @@ constexpr int ZBITS = 7;                      // slice width
 struct Z6 {
   static constexpr int NS = 6, NLEV = 4, TN = TNB, KC = 32;
   static __device__ __forceinline__ double value(const float (&f)[NLEV][8], int j, int e, bool neg) {
-    const long long n = level_sum<0, 3, 46, 42>(f, j);
-    return fixed_to_double(neg ? -n : n, e, 46);
+    // the last level as it stands in FP32: its multiples of 2^-49
+    const long long n = level_sum<0, 3, 49, 49, NS, 2 * 16 * KC>(f, j);
+    return fixed_to_double(neg ? -n : n, e, 49);
   }
 };
 struct Z9 {
   static constexpr int NS = 9, NLEV = 8, TN = 32, KC = Z9_KSTEPS;
   // two words: levels 0..3 in units of 2^-35, the rest in units of 2^-70, one FP64 addition
   static __device__ __forceinline__ double value(const float (&f)[NLEV][8], int j, int e, bool neg) {
-    const long long h = level_sum<0, 3, 35, 0>(f, j), l = level_sum<4, 7, 70, 65>(f, j);
+    const long long h = level_sum<0, 3, 35, 0, NS, 2 * 16 * KC>(f, j), l = level_sum<4, 7, 70, 65, NS, 2 * 16 * KC>(f, j);
     return fixed_to_double(neg ? -h : h, e, 35) + fixed_to_double(neg ? -l : l, e, 70);
   }
 };
