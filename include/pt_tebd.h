@@ -230,7 +230,8 @@ int pt_tebd_get_timing(pt_tebd_t h, double* ms9);
  * (descending), U [batch][m][min(m,n)] and V [batch][n][min(m,n)] (device, row-major), so
  * A_b = U diag(sigma) V^H. Larger matrices (min(m, n) from 96, or from 32 where the other side is four
  * times as long) go through two QRs before the Jacobi; where those find NaN or the Jacobi then does not
- * converge, the call repeats without them. scratch: device workspace of pt_svd_scratch_bytes(m, n, batch)
+ * converge, the call repeats without them. Squares of the entries have to stay in FP64's range
+ * (largest entry between about 1e-135 and 1e150); within it the scale does not matter. scratch: device workspace of pt_svd_scratch_bytes(m, n, batch)
  * bytes. PT_ERR_DEVICE_TIMEOUT: a bounded barrier wait.
  * Returns PT_ERR_SVD_NOCONV if a matrix did not converge within max_sweeps. */
 size_t pt_svd_scratch_bytes(int m, int n, int batch);

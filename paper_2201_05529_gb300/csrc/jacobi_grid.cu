@@ -113,6 +113,11 @@ __device__ __forceinline__ int pair_exponent(double al, double be, double qx, do
   return (exponent_of(al) + exponent_of(be) - exponent_of(qx) - exponent_of(qy) + 3) >> 1;
 }
 
+// Squared norms, inner products and thresholds of an item are in units of 2^norm_exponent(||A||_F^2), so that |gamma|^2 and
+// norm^2 stay in range whatever the matrix' scale (without, columns of norm 1e-76 or 1e76 were left as they were)
+__device__ __forceinline__ int norm_exponent(double fro2) { return max(-1022, min(1022, exponent_of(fro2))); }
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }       // |e| <= 1022
+
 // x in units of 2^(E - 57), truncated; 0 if not finite or out of range
 __device__ __forceinline__ long long to_fixed(double x, int E) {
   const long long b = __double_as_longlong(x);
@@ -143,7 +148,7 @@ __device__ __forceinline__ float scale_pow2(float f, int k) {
 }
 
 // shared-memory tables of a launch over n items
-__host__ __device__ constexpr int header_bytes(int n) { return (48 * n + 4 * (4 * n + 1) + 15) & ~15; }
+__host__ __device__ constexpr int header_bytes(int n) { return (48 * n + 4 * (5 * n + 1) + 15) & ~15; }
 
 __device__ __forceinline__ int load_acquire(const int* p) {
   int v;
@@ -205,8 +210,8 @@ __device__ int choose_block(const int* s_Na, const int* s_Ma, int n_work, int sl
 // One-sided Jacobi over all matrices of a layer in FP64. with_v: accumulate the right factor V from V = I.
 // tol_scale: a pair rotates while |a_i^H a_j| > tol_scale * unit roundoff * |a_i| |a_j| (0: the row count m).
 // Columns whose squared norm is at floor2 ||A||_F^2 or below are not rotated: they cannot become orthogonal
-// relative to their own norm and carry no information at that precision. Squared column norms live in aux, squared
-// scales in sig, rotation counters in info[4..5], sweeps go to info[3]. SM: the columns fit in shared memory (cols_max
+// relative to their own norm and carry no information at that precision. Squared column norms (in the item's unit) live
+// in aux, squared scales in sig, rotation counters in info[4..5], sweeps go to info[3]. SM: the columns fit in shared memory (cols_max
 // of them); otherwise a pair's columns are read from and written to L2 (b = 1).
 template <bool SM>
 __global__ void __launch_bounds__(CT, 1)
@@ -231,7 +236,7 @@ __global__ void __launch_bounds__(CT, 1)
     if (blockIdx.x == 0 && ctid == 0) atomicOr(status, ST_CAPACITY);
     return;
   }
-  double* s_fro = (double*)s_raw;                    // ||A||_F^2 per item
+  double* s_fro = (double*)s_raw;                    // ||A||_F^2 per item, in units of 2^s_exp
   double2** s_A = (double2**)(s_fro + n_work);       // the items' buffers (the work list itself is behind two loads)
   double2** s_V = s_A + n_work;
   double** s_aux = (double**)(s_V + n_work);
@@ -241,6 +246,7 @@ __global__ void __launch_bounds__(CT, 1)
   int* s_Ma = s_Na + n_work;                         // rows
   int* s_off = s_Ma + n_work;                        // [n_work + 1] prefix of the sweep's tasks per round
   int* s_act = s_off + n_work + 1;
+  int* s_exp = s_act + n_work;                       // norm_exponent of ||A||_F^2
   const int hdr = header_bytes(n_work);
   const int slot_bytes = (dyn_bytes - hdr) / n_grp & ~15;
   double2* s_col = (double2*)(s_raw + hdr + (size_t)grp * slot_bytes);
@@ -340,7 +346,11 @@ __global__ void __launch_bounds__(CT, 1)
     double acc = 0;
     for (int k = lane; k < s_Na[w]; k += 32) acc += __ldcg(work[w].aux + k);
     acc = wsum(acc);
-    if (lane == 0) s_fro[w] = acc;
+    if (lane == 0) {
+      const int e = norm_exponent(acc);
+      s_fro[w] = acc * pow2(-e);
+      s_exp[w] = e;
+    }
   }
   // the rounds of the next sweep, the longest tournament among the active items (0: all converged), and the prefix of
   // the active items' task counts
@@ -399,6 +409,8 @@ __global__ void __launch_bounds__(CT, 1)
         }
         double2 *A = s_A[w], *V = s_V[w];
         double *aux = s_aux[w], *sig = s_sig[w];
+        const int ex = s_exp[w];
+        const double unit = pow2(-ex);
         // local column c: global column of block bi (c < b) or bj; -1 beyond the matrix
         auto gcol = [&](int c) {
           const int g = (c < b ? bi * b + c : bj * b + c - b);
@@ -479,7 +491,7 @@ __global__ void __launch_bounds__(CT, 1)
               for (int k = 0; k < wpc; ++k) s += S.part[tid * wpc + k][0];
             else
               s = S.part[tid & (JW - 1)][tid / JW];
-            S.nrm[tid] = s * S.q[tid];
+            S.nrm[tid] = s * unit * S.q[tid];
           }
           slot_sync(grp);
         }
@@ -529,7 +541,7 @@ __global__ void __launch_bounds__(CT, 1)
                 gr = fma(u.x, v.x, fma(u.y, v.y, gr));
                 gim = fma(u.x, v.y, fma(-u.y, v.x, gim));
               }
-              const int E = pair_exponent(S.nrm[li], S.nrm[lj], S.q[li], S.q[lj]);
+              const int E = pair_exponent(S.nrm[li], S.nrm[lj], S.q[li], S.q[lj]) + ex;
               __syncwarp();
               const long long sr_ = lane_sum(to_fixed(gr, E)), si_ = lane_sum(to_fixed(gim, E));
               if (lane < 2) S.part[wid][lane] = __longlong_as_double(lane == 0 ? sr_ : si_);
@@ -647,8 +659,8 @@ __global__ void __launch_bounds__(CT, 1)
                 sa += S.part[p * wpp + k][0];
                 sb += S.part[p * wpp + k][1];
               }
-              S.nrm[li] = sa * S.q[li];
-              S.nrm[lj] = sb * S.q[lj];
+              S.nrm[li] = sa * unit * S.q[li];
+              S.nrm[lj] = sb * unit * S.q[lj];
             }
             slot_sync(grp);
           }
