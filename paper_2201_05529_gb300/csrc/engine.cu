@@ -1713,7 +1713,7 @@ static size_t svd_layout(int m, int n, int batch, size_t* offs) {
   offs[5] = take(sizeof(int));                                // status, and the barrier's words at + 8 ints
   offs[6] = take(sizeof(BondWork) * (size_t)batch);           // work items
   offs[7] = take(sizeof(double) * (size_t)Na * batch);        // column norms
-  offs[8] = take(ptk::svd_qr_fits(Ma, Na, batch) ? ptk::svd_qr_layout(Ma, Na, batch, nullptr, nullptr) : 0);
+  offs[8] = take(ptk::svd_qr_shape(Ma, Na, batch) ? ptk::svd_qr_layout(Ma, Na, batch, nullptr, nullptr) : 0);
   return o;
 }
 

@@ -68,6 +68,7 @@ struct QRBlkList {
   int cluster = 0;         // qr_block_cluster(n_items, m_cap)
 };
 int qr_block_cluster(int n_items, int m_cap);
+constexpr int QR_BLOCK_MAX_ROWS = 6400;      // the longest panel that the largest cluster holds
 size_t qr_block_bytes(int m, int n, QRBlk* B, char* base);
 size_t qr_block_ops(int n_items, int n_cap);
 // the whole factorisation of small matrices, one CTA each (items' live shapes at most m_cap x n_cap)
@@ -114,6 +115,8 @@ struct SvdQr {
   size_t per_blk, per_a, per_b;
 };
 struct SvdQrHost;
+// by shape alone (the workspace's size follows it); and whether the current device takes the panels' clusters
+bool svd_qr_shape(int Ma, int Na, int batch);
 bool svd_qr_fits(int Ma, int Na, int batch);
 size_t svd_qr_layout(int Ma, int Na, int batch, SvdQr* out, char* base);
 void launch_svd_qr(const double2* A, int m, int n, int batch, const BondWork* items, double2* wA, double2* wV,

@@ -36,6 +36,7 @@ constexpr int PANEL_T = PT + 32;           // and a warp for the scalars
 constexpr int SMALL_N = 32;                // columns of a matrix that one CTA factors whole
 constexpr int MAX_C = 16;                  // CTAs per cluster
 constexpr int PANEL_SMEM = 200 * 1024;     // panel rows of one CTA (227 KB less the exchange buffers)
+static_assert(QR_BLOCK_MAX_ROWS == MAX_C * (PANEL_SMEM / (NB * (int)sizeof(double2))), "rows of the largest cluster");
 constexpr int MAX_PARTS = 16;               // K chunks of a product W, unless chunks of the longest kind are more
 constexpr int WT_ROWS = 8;                 // rows of W per block of k_qr_wt, one warp each
 

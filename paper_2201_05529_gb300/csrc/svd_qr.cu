@@ -171,9 +171,12 @@ size_t svd_qr_layout(int Ma, int Na, int batch, SvdQr* out, char* base) {
 // two 1000 x 40 2.0 / 4.5 (64 x 64 gained a fifth with QRs of 2.9 ms). With random entries and columns graded over four
 // decades the Jacobi alone is quick as well: 96 x 96 4.0 / 3.0, ten 160 x 160 10.2 / 10.3, two 256 x 256 14.3 / 13.9; a
 // line further down would lose more there than a bond's matrix gains.
+bool svd_qr_shape(int Ma, int Na, int batch) {
+  return (Na >= 96 || (Na >= 32 && Ma / 4 >= Na)) && 2LL * batch <= zgemm_max_items() && Ma <= QR_BLOCK_MAX_ROWS;
+}
+
 bool svd_qr_fits(int Ma, int Na, int batch) {
-  return (Na >= 96 || (Na >= 32 && Ma / 4 >= Na)) && 2LL * batch <= zgemm_max_items() &&
-         qr_block_cluster(batch, Ma) > 0 && qr_block_cluster(batch, Na) > 0;
+  return svd_qr_shape(Ma, Na, batch) && qr_block_cluster(batch, Ma) > 0 && qr_block_cluster(batch, Na) > 0;
 }
 
 void launch_svd_qr(const double2* A, int m, int n, int batch, const BondWork* items, double2* wA, double2* wV,
