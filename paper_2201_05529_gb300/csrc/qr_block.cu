@@ -20,6 +20,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <mutex>
 
 #include "kernels.h"
 
@@ -562,9 +563,10 @@ __global__ void k_qr_identity(const QRBlk* blk, int n_items) {
 
 namespace {
 
-// clusters of c CTAs (one CTA per SM) that fit the device at the same time, c = 1 .. MAX_C; 0: not launchable
+// clusters of c CTAs (one CTA per SM) that fit the device at the same time, c = 1 .. MAX_C; 0: not launchable. Filled once
+// per device, by one thread while the others wait
 struct ClusterTable {
-  bool done = false;
+  std::once_flag once;
   int active[MAX_C + 1] = {};
 };
 constexpr int MAX_DEV = 64;
@@ -589,7 +591,7 @@ const ClusterTable& cluster_table() {
   int dev = 0;
   cudaGetDevice(&dev);
   ClusterTable& t = g_tab[std::max(0, std::min(dev, MAX_DEV - 1))];
-  if (!t.done) {
+  std::call_once(t.once, [&t] {
     cudaFuncSetAttribute(k_qr_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, PANEL_SMEM);
     cudaFuncSetAttribute(k_qr_panel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     for (int c = 1; c <= MAX_C; ++c) {
@@ -599,8 +601,7 @@ const ClusterTable& cluster_table() {
       if (cudaOccupancyMaxActiveClusters(&n, k_qr_panel, &cfg) == cudaSuccess) t.active[c] = n;
       cudaGetLastError();
     }
-    t.done = true;
-  }
+  });
   return t;
 }
 

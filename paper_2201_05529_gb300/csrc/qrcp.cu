@@ -13,6 +13,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <mutex>
 
 #include "kernels.h"
 
@@ -440,7 +441,7 @@ namespace {
 constexpr int QR_SMEM = 208 * 1024;          // 227 KB less the static arrays
 constexpr int QR_MAX_DEV = 64;
 struct QrClusters {
-  bool done = false;
+  std::once_flag once;                       // filled by one thread while the others wait
   int active[QR_MAX_C + 1] = {};             // clusters of c CTAs the device holds at once
 };
 QrClusters g_qr_tab[QR_MAX_DEV];
@@ -464,7 +465,7 @@ const QrClusters& qr_clusters() {
   int dev = 0;
   cudaGetDevice(&dev);
   QrClusters& t = g_qr_tab[std::max(0, std::min(dev, QR_MAX_DEV - 1))];
-  if (!t.done) {
+  std::call_once(t.once, [&t] {
     cudaFuncSetAttribute(k_qrcp_cl, cudaFuncAttributeMaxDynamicSharedMemorySize, QR_SMEM);
     cudaFuncSetAttribute(k_qrcp_cl, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     for (int c = 1; c <= QR_MAX_C; ++c) {
@@ -474,8 +475,7 @@ const QrClusters& qr_clusters() {
       if (cudaOccupancyMaxActiveClusters(&n, k_qrcp_cl, &cfg) == cudaSuccess) t.active[c] = n;
       cudaGetLastError();
     }
-    t.done = true;
-  }
+  });
   return t;
 }
 

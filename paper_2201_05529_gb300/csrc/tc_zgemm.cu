@@ -31,6 +31,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <mutex>
 
 #include "kernels.h"
 #include "tc_common.cuh"
@@ -445,7 +446,7 @@ int zgemm_tile_cap(int m_cap, int n_cap) { return cdiv(std::max(1, m_cap), TMA) 
 
 namespace {
 constexpr int ZMAX_DEV = 64;
-bool g_zattr_done[ZMAX_DEV][2] = {};
+std::once_flag g_zattr[ZMAX_DEV][2];        // the shared-memory limit is set once per device
 
 template <class Z>
 void launch_prep(const ZGemmItem* items, int n_items, int m_cap_max, int n_cap_max, int k_cap_max, int mode, int* status,
@@ -464,10 +465,10 @@ void launch_gemm(const ZGemmItem* items, int n_items, long long unit_cap, int* s
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (dev >= 0 && dev < ZMAX_DEV && !g_zattr_done[dev][Z::NS == 9]) {
-    cudaFuncSetAttribute(k_zgemm<Z>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    g_zattr_done[dev][Z::NS == 9] = true;
-  }
+  if (dev >= 0 && dev < ZMAX_DEV)
+    std::call_once(g_zattr[dev][Z::NS == 9], [smem] {
+      cudaFuncSetAttribute(k_zgemm<Z>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    });
   const int grid = (int)std::max<long long>(1, std::min<long long>(sms > 0 ? sms : 152, unit_cap));
   k_zgemm<Z><<<grid, GEMM_THREADS, smem, st>>>(items, n_items, status);
 }
