@@ -291,6 +291,10 @@ int pt_svd_f64_noalloc(const double* A, int m, int n, int batch, double* sigma, 
  * cases the context stays usable. device_status (may be NULL) receives the device status bits.
  * Uses static device variables only and synchronises the device. */
 int pt_selftest_grid_barrier(int withheld_block, double limit_ms, int* device_status);
+/* pt_svd_f64 without QRs before it, its Jacobi launched with `ctas` CTAs (0: one per SM) and a wait limit of
+ * limit_ms (0: the usual one; at most 10000) beside the part that grows with the work of a sweep. */
+int pt_selftest_svd(const double* A, int m, int n, int batch, double* sigma, double* U, double* V, void* scratch,
+                    int ctas, double limit_ms, void* cuda_stream);
 
 #ifdef __cplusplus
 }

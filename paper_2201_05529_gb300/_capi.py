@@ -30,6 +30,7 @@ EXPORTS = [
     "pt_tebd_sync", "pt_tebd_destroy", "pt_tebd_last_error", "pt_tebd_set_timing",
     "pt_tebd_get_timing", "pt_svd_scratch_bytes", "pt_svd_f64", "pt_svd_f64_noalloc",
     "pt_zgemm_scratch_bytes", "pt_zgemm_sliced", "pt_qr_scratch_bytes", "pt_qr_f64", "pt_selftest_grid_barrier",
+    "pt_selftest_svd",
 ]
 
 
@@ -125,6 +126,8 @@ lib.pt_svd_f64_noalloc.argtypes = [C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_vo
 NOALLOC_MAX_BYTES = 16 << 20     # PT_SVD_NOALLOC_MAX_BYTES
 
 
+lib.pt_selftest_svd.argtypes = [C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
+                                C.c_int, C.c_double, C.c_void_p]
 lib.pt_selftest_grid_barrier.argtypes = [C.c_int, C.c_double, C.POINTER(C.c_int)]
 lib.pt_selftest_grid_barrier.restype = C.c_int
 
@@ -482,6 +485,15 @@ def selftest_grid_barrier(withheld_block=-1, limit_ms=1.0):
     st = C.c_int(0)
     rc = lib.pt_selftest_grid_barrier(int(withheld_block), float(limit_ms), C.byref(st))
     return rc, st.value
+
+
+def selftest_svd(A, sigma, U, V, scratch, ctas=0, limit_ms=0.0, stream=None):
+    """pt_selftest_svd: the direct Jacobi SVD (tensors as svd_f64's) launched with `ctas` CTAs and a wait limit of limit_ms;
+    returns the code without raising."""
+    b, m, n = A.shape
+    st = stream if stream is not None else current_stream_handle()
+    return lib.pt_selftest_svd(C.c_void_p(A.data_ptr()), m, n, b, C.c_void_p(sigma.data_ptr()), C.c_void_p(U.data_ptr()),
+                               C.c_void_p(V.data_ptr()), C.c_void_p(scratch.data_ptr()), int(ctas), float(limit_ms), st)
 
 
 def tune_cache_lookup(path, key):

@@ -1900,14 +1900,14 @@ int pt_zgemm_sliced(int opA, int opB, int m, int n, int k, const double* A, int 
   return PT_OK;
 }
 
-int pt_svd_f64(const double* A, int m, int n, int batch, double* sigma, double* U, double* V,
-               void* scratch, int max_sweeps, void* cuda_stream) {
+// direct: without the two QRs
+static int svd_f64(const double* A, int m, int n, int batch, double* sigma, double* U, double* V, void* scratch,
+                   int max_sweeps, cudaStream_t st, bool direct, const ptk::JacobiTune& tune) {
   if (!A || m < 1 || n < 1 || batch < 1 || !sigma || !U || !V || !scratch) {
     g_err = "pt_svd_f64: bad arguments";
     return PT_ERR_ARG;
   }
   if (max_sweeps <= 0) max_sweeps = 60;
-  cudaStream_t st = (cudaStream_t)cuda_stream;
   size_t offs[9];
   svd_layout(m, n, batch, offs);
   char* base = (char*)scratch;
@@ -1955,7 +1955,7 @@ int pt_svd_f64(const double* A, int m, int n, int batch, double* sigma, double* 
     } else {
       const int gx = (int)std::min<size_t>(256, ((size_t)m * n + 255) / 256);
       ptk::k_svd_load<<<dim3(gx, batch), 256, 0, st>>>((const double2*)A, m, n, batch, wA, sA);
-      ptk::launch_svd_jacobi(items, batch, Ma, Na, max_sweeps, status, (unsigned*)(status + 8), st);
+      ptk::launch_svd_jacobi(items, batch, Ma, Na, max_sweeps, status, (unsigned*)(status + 8), st, tune);
       const int gs = (int)std::min<size_t>(256, ((size_t)(m + n + 1) * Na + 255) / 256);
       ptk::k_svd_store<<<dim3(gs, batch), 256, 0, st>>>(wA, wV, sig, perm, m, n, batch, sA, sV, sigma,
                                                         (double2*)U, (double2*)V);
@@ -1966,7 +1966,7 @@ int pt_svd_f64(const double* A, int m, int n, int batch, double* sigma, double* 
     const cudaError_t es = cudaStreamSynchronize(st);
     return e == cudaSuccess ? es : e;
   };
-  const bool pre = ptk::svd_qr_fits(Ma, Na, batch);
+  const bool pre = !direct && ptk::svd_qr_fits(Ma, Na, batch);
   int hs = 0;
   cudaError_t e = attempt(pre, &hs);
   // an infinity turns into NaN in a reflector, not everywhere in a rotation: such input gets the direct call's answer
@@ -1992,6 +1992,24 @@ int pt_svd_f64(const double* A, int m, int n, int batch, double* sigma, double* 
     return PT_ERR_CAPACITY;
   }
   return PT_OK;
+}
+
+int pt_svd_f64(const double* A, int m, int n, int batch, double* sigma, double* U, double* V, void* scratch, int max_sweeps,
+               void* cuda_stream) {
+  return svd_f64(A, m, n, batch, sigma, U, V, scratch, max_sweeps, (cudaStream_t)cuda_stream, false, ptk::JacobiTune{});
+}
+
+int pt_selftest_svd(const double* A, int m, int n, int batch, double* sigma, double* U, double* V, void* scratch, int ctas,
+                    double limit_ms, void* cuda_stream) {
+  int dev = 0, khz = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev);
+  if (ctas < 0 || limit_ms < 0.0 || limit_ms > 10000.0 || khz <= 0) {
+    g_err = "pt_selftest_svd: bad arguments";
+    return PT_ERR_ARG;
+  }
+  return svd_f64(A, m, n, batch, sigma, U, V, scratch, 0, (cudaStream_t)cuda_stream, true,
+                 ptk::JacobiTune{ctas, (long long)(limit_ms * khz)});
 }
 
 }  // extern "C"

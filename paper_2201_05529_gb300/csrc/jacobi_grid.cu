@@ -230,6 +230,7 @@ __global__ void __launch_bounds__(CT, 1)
   };
   __shared__ Slot s_slot[JG];
   __shared__ int s_b, s_rounds, s_fit, s_most, s_cols;
+  __shared__ long long s_limit;            // wait limit: the launch's, and what a sweep can take
   const int ctid = threadIdx.x, grp = ctid / JT, tid = ctid % JT, lane = tid & 31, wid = tid >> 5, cwid = ctid >> 5;
   Slot& S = s_slot[grp];
   if (n_work > MAX_ITEMS) {
@@ -272,19 +273,26 @@ __global__ void __launch_bounds__(CT, 1)
     rows = __reduce_max_sync(0xffffffffu, rows);
     const int fit = SM ? (rows > 0 ? slot_bytes / (16 * rows) : 2) : 2;
     const int b = SM ? choose_block(s_Na, s_Ma, n_work, n_grp * gridDim.x, gridDim.x, fit, with_v != 0, lane) : 1;
-    int most = 0, cols = 0;
+    int most = 0, cols = 0, nbs = 0;
     for (int w = lane; w < n_work; w += 32) {
       const int nb = (s_Na[w] + b - 1) / b, nbp = nb + (nb & 1);
       if (s_Na[w] >= 2) most += nbp / 2;
       cols += s_Na[w];
+      nbs = max(nbs, nbp);
     }
     most = __reduce_add_sync(0xffffffffu, most);
     cols = __reduce_add_sync(0xffffffffu, cols);
+    nbs = __reduce_max_sync(0xffffffffu, nbs);
     if (lane == 0) {
       s_fit = fit;
       s_b = b;
       s_most = most;
       s_cols = cols;
+      // a CTA without tasks (its items have converged) waits for a whole sweep of the others: rounds x a slot's tasks x up
+      // to 2 b sub-rounds of b pairs, at most 64 cycles per row and pair (twelve FP64 instructions of two slots at the issue
+      // rate are 24, columns from memory 15) and what does not depend on the rows
+      const long long turns = most / (n_grp * (int)gridDim.x) + 1;
+      s_limit = gs.limit + nbs * turns * 2 * b * (64LL * b * rows + 20000);
     }
   }
   __syncthreads();
@@ -296,7 +304,7 @@ __global__ void __launch_bounds__(CT, 1)
   // CTAs that take part: as many as a round has tasks (and the passes over all columns can use)
   const int G = max(1, min((int)gridDim.x, max(s_most, min((s_cols + 15) / 16, 152))));
   if ((int)blockIdx.x >= G) return;
-  auto barrier = [&]() { return grid_barrier(gs, status, G); };
+  auto barrier = [&]() { return grid_barrier(GridSync{gs.count, gs.abort, s_limit}, status, G); };
   // V = I, zero counters, unit scales, column norms
   {
     const int gt = blockIdx.x * CT + ctid, ngt = G * CT;
@@ -427,7 +435,7 @@ __global__ void __launch_bounds__(CT, 1)
             for (int it = 1; load_acquire(ver + blk) < need; ++it) {
               if ((it & 63) != 0) continue;
               if (*(volatile int*)gs.abort) lost = true;
-              else if (clock64() - t0 > gs.limit) {
+              else if (clock64() - t0 > s_limit) {
                 atomicOr(status, ST_TIMEOUT);
                 atomicExch(gs.abort, 1);
                 lost = true;
@@ -820,10 +828,11 @@ int jacobi_grid_blocks() {
 }
 
 void launch_jacobi_grid(const BondWork* work, int n_work, int blocks, int rows_cap, int max_sweeps, unsigned* sync3,
-                        int* status, cudaStream_t st, int on_b, int with_v, double tol_scale, double floor2) {
+                        int* status, cudaStream_t st, int on_b, int with_v, double tol_scale, double floor2,
+                        long long wait_cycles) {
   // the barrier's arrival counter and the abort flag start at zero for every launch
   cudaMemsetAsync(sync3, 0, 3 * sizeof(unsigned), st);
-  GridSync gs{sync3, (int*)(sync3 + 2), GRID_WAIT_LIMIT_CYCLES};
+  GridSync gs{sync3, (int*)(sync3 + 2), wait_cycles > 0 ? wait_cycles : GRID_WAIT_LIMIT_CYCLES};
   int n_grp = 1;
   const int hdr = jacobi_smem(n_work, 1 << 20, &n_grp), smem = jacobi_smem(n_work, rows_cap, &n_grp);
   cudaLaunchConfig_t cfg = {};
@@ -843,10 +852,11 @@ void launch_jacobi_grid(const BondWork* work, int n_work, int blocks, int rows_c
 // Whole GPU against one cluster per matrix: two 256 x 256 matrices 113 ms in two 16-CTA clusters (32 of 152 SMs),
 // see the head of this file; the cluster kernel takes what one launch of this one does not.
 void launch_svd_jacobi(const BondWork* items, int batch, int Ma, int Na, int max_sweeps, int* status, unsigned* sync3,
-                       cudaStream_t st) {
+                       cudaStream_t st, const JacobiTune& tune) {
   const int blocks = batch <= MAX_ITEMS ? jacobi_grid_blocks() : 0;
   if (blocks > 0) {
-    launch_jacobi_grid(items, batch, blocks, Ma + Na, max_sweeps, sync3, status, st, /*on_b=*/0, /*with_v=*/1, 0.0);
+    launch_jacobi_grid(items, batch, tune.ctas > 0 ? tune.ctas : blocks, Ma + Na, max_sweeps, sync3, status, st, /*on_b=*/0,
+                       /*with_v=*/1, 0.0, JACOBI_FLOOR2, tune.wait_cycles);
   } else {
     const int cl = jacobi_cluster_size(std::max(1, std::min(16, (Na / 2 + 7) / 8)));
     launch_jacobi_cluster(items, batch, cl, max_sweeps, status, st);

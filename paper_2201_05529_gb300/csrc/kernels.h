@@ -91,15 +91,20 @@ int jacobi_grid_blocks();
 constexpr double JACOBI_FLOOR2 = 1.232595164407831e-32;      // squared noise floor: u^2 = 2^-106
 // on_b: 0 = the matrix in A, 1 = B = R^H of the pivoted QR (Na x info[8]), 2 = R^H of the range finder's l x l
 // factor R in G64 (l = info[9]), formed and overwritten by its left vectors in V; with_v: accumulate V; tol_scale: rotation threshold in units of the unit roundoff (0: the
-// row count); floor2: columns at floor2 ||A||_F^2 or below (squared norms) are left as they are
+// row count); wait_cycles: the part of the waits' limit that does not grow with a sweep (0: the usual one); floor2: columns at floor2 ||A||_F^2 or below (squared norms) are left as they are
 void launch_jacobi_grid(const BondWork* work, int n_work, int blocks, int rows_cap, int max_sweeps, unsigned* sync3,
                         int* status, cudaStream_t st, int on_b, int with_v, double tol_scale,
-                        double floor2 = JACOBI_FLOOR2);
+                        double floor2 = JACOBI_FLOOR2, long long wait_cycles = 0);
 
 // the standalone batched SVD's Jacobi (k_svd_load before it, k_svd_store after it) on Ma x Na matrices: the whole
-// GPU where it can be co-scheduled and a launch takes the batch, else one cluster per matrix; sync3 as above
+// GPU where it can be co-scheduled and a launch takes the batch, else one cluster per matrix; sync3 as above; tune: the
+// CTAs and the wait limit of a diagnostic call (0: the usual ones)
+struct JacobiTune {
+  int ctas = 0;
+  long long wait_cycles = 0;
+};
 void launch_svd_jacobi(const BondWork* items, int batch, int Ma, int Na, int max_sweeps, int* status, unsigned* sync3,
-                       cudaStream_t st);
+                       cudaStream_t st, const JacobiTune& tune = JacobiTune{});
 
 // the standalone SVD after two QRs (svd_qr.cu): its workspaces (of size svd_qr_layout), the host copies of its lists
 // (kept until the stream is synchronised); items: n x n matrices in SvdQr::T with V in wV
