@@ -827,7 +827,7 @@ int jacobi_grid_blocks() {
   return a >= 1 && b >= 1 ? sms : 0;
 }
 
-void launch_jacobi_grid(const BondWork* work, int n_work, int blocks, int rows_cap, int max_sweeps, unsigned* sync3,
+cudaError_t launch_jacobi_grid(const BondWork* work, int n_work, int blocks, int rows_cap, int max_sweeps, unsigned* sync3,
                         int* status, cudaStream_t st, int on_b, int with_v, double tol_scale, double floor2,
                         long long wait_cycles) {
   // the barrier's arrival counter and the abort flag start at zero for every launch
@@ -845,22 +845,25 @@ void launch_jacobi_grid(const BondWork* work, int n_work, int blocks, int rows_c
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, smem > hdr ? k_jacobi_grid<true> : k_jacobi_grid<false>, work, n_work, max_sweeps, gs,
+  return cudaLaunchKernelEx(&cfg, smem > hdr ? k_jacobi_grid<true> : k_jacobi_grid<false>, work, n_work, max_sweeps, gs,
                      status, on_b, with_v, tol_scale, floor2, n_grp, smem);
 }
 
 // Whole GPU against one cluster per matrix: two 256 x 256 matrices 113 ms in two 16-CTA clusters (32 of 152 SMs),
-// see the head of this file; the cluster kernel takes what one launch of this one does not.
+// see the head of this file; the cluster kernel takes what one launch of this one does not, and what is left of a device
+// that cannot hold all of its CTAs at once (a context with fewer SMs than the device says).
 void launch_svd_jacobi(const BondWork* items, int batch, int Ma, int Na, int max_sweeps, int* status, unsigned* sync3,
                        cudaStream_t st, const JacobiTune& tune) {
   const int blocks = batch <= MAX_ITEMS ? jacobi_grid_blocks() : 0;
   if (blocks > 0) {
-    launch_jacobi_grid(items, batch, tune.ctas > 0 ? tune.ctas : blocks, Ma + Na, max_sweeps, sync3, status, st, /*on_b=*/0,
-                       /*with_v=*/1, 0.0, JACOBI_FLOOR2, tune.wait_cycles);
-  } else {
-    const int cl = jacobi_cluster_size(std::max(1, std::min(16, (Na / 2 + 7) / 8)));
-    launch_jacobi_cluster(items, batch, cl, max_sweeps, status, st);
+    const bool clean = cudaPeekAtLastError() == cudaSuccess;
+    const cudaError_t e = launch_jacobi_grid(items, batch, tune.ctas > 0 ? tune.ctas : blocks, Ma + Na, max_sweeps, sync3,
+                                             status, st, /*on_b=*/0, /*with_v=*/1, 0.0, JACOBI_FLOOR2, tune.wait_cycles);
+    if (e != cudaErrorCooperativeLaunchTooLarge || !clean) return;
+    cudaGetLastError();                    // this launch's, refused before anything ran
   }
+  const int cl = jacobi_cluster_size(std::max(1, std::min(16, (Na / 2 + 7) / 8)));
+  launch_jacobi_cluster(items, batch, cl, max_sweeps, status, st);
 }
 
 }  // namespace ptk

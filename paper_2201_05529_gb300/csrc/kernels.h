@@ -92,8 +92,8 @@ constexpr double JACOBI_FLOOR2 = 1.232595164407831e-32;      // squared noise fl
 // on_b: 0 = the matrix in A, 1 = B = R^H of the pivoted QR (Na x info[8]), 2 = R^H of the range finder's l x l
 // factor R in G64 (l = info[9]), formed and overwritten by its left vectors in V; with_v: accumulate V; tol_scale: rotation threshold in units of the unit roundoff (0: the
 // row count); wait_cycles: the part of the waits' limit that does not grow with a sweep (0: the usual one); floor2: columns at floor2 ||A||_F^2 or below (squared norms) are left as they are
-void launch_jacobi_grid(const BondWork* work, int n_work, int blocks, int rows_cap, int max_sweeps, unsigned* sync3,
-                        int* status, cudaStream_t st, int on_b, int with_v, double tol_scale,
+cudaError_t launch_jacobi_grid(const BondWork* work, int n_work, int blocks, int rows_cap, int max_sweeps,
+                               unsigned* sync3, int* status, cudaStream_t st, int on_b, int with_v, double tol_scale,
                         double floor2 = JACOBI_FLOOR2, long long wait_cycles = 0);
 
 // the standalone batched SVD's Jacobi (k_svd_load before it, k_svd_store after it) on Ma x Na matrices: the whole

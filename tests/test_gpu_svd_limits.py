@@ -1,5 +1,6 @@
 """The launch of the whole-GPU Jacobi behind the standalone SVD: CTAs whose matrices have converged wait for a whole sweep
-of the others, which may take longer than the wait limit; the limit grows with a sweep's work."""
+of the others, which may take longer than the wait limit; the limit grows with a sweep's work. Where the device cannot
+hold the launch's CTAs at once, one cluster per matrix does the work."""
 import numpy as np
 import pytest
 
@@ -44,3 +45,12 @@ def test_a_sweep_may_take_longer_than_the_wait_limit(capi):
     A = rng.standard_normal((2, 256, 256)) + 1j * rng.standard_normal((2, 256, 256))
     A[0] = np.diag(np.arange(256, 0, -1.0))
     _check(capi, A, limit_ms=0.2)
+
+
+@pytest.mark.parametrize("m,n,batch", [(1, 1, 1), (9, 7, 3), (70, 130, 2), (100, 100, 1)])
+def test_a_refused_cooperative_launch_falls_back_to_clusters(capi, m, n, batch):
+    """More CTAs than the device holds: the launch is refused on the host, before anything runs."""
+    rng = np.random.default_rng(m + n)
+    A = rng.standard_normal((batch, m, n)) + 1j * rng.standard_normal((batch, m, n))
+    _check(capi, A, ctas=100000)
+    _check(capi, A)
