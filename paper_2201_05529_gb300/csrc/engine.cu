@@ -175,6 +175,8 @@ struct pt_tebd {
       p = nullptr;
     }
     if (p) allocs.push_back({p, bytes});
+    // the caller decides what a refused request means: its error does not stay for a later check
+    else if (cudaPeekAtLastError() == cudaErrorMemoryAllocation) cudaGetLastError();
     return p;
   }
 
