@@ -59,6 +59,14 @@ __device__ __forceinline__ double2 group_sum(double a, double b, int L, bool hal
   return half ? make_double2(other, s) : make_double2(s, other);
 }
 
+// 1 where 1 / (nrm sum), sum = |alpha| + nrm, has no FP64 value (||x||^2 below 2^-1024; its factors have one), as the trip count
+// of a loop around the rare arithmetic (behind a short if the compiler issues it always, 64 cycles an instruction).
+__device__ __forceinline__ int no_value(double ti) {
+  int n = __double2hiint(ti) >= 0x7ff00000;
+  asm("" : "+r"(n));
+  return n;
+}
+
 // Length of the K chunks of W = A^H V (steps of 16) for n_items products of `cols` rows: the shortest estimate, waves of
 // units over the SMs times (steps + 2.5 for a unit's start and epilogue). 256-long chunks alone leave few units for few
 // matrices and a second, nearly empty wave for others (160 units of ten 2048 x 160 on 152 SMs): two 256 x 256 QRs 2.54 ->
@@ -184,7 +192,7 @@ __global__ void __launch_bounds__(PANEL_T, 1) k_qr_panel(const QRBlk* blk, int n
   __shared__ double2 s_part[2][MAX_C][NB];
   __shared__ double2 s_row[2][NB];
   __shared__ double2 s_u, s_cr, s_scale[NB];
-  __shared__ double s_ti, s_taus[NB];
+  __shared__ double s_ti, s_rn, s_inv, s_taus[NB];
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), C = (int)cl.num_blocks();
   const int i = blockIdx.x / C;
@@ -299,6 +307,8 @@ __global__ void __launch_bounds__(PANEL_T, 1) k_qr_panel(const QRBlk* blk, int n
                   : lane == 6 ? &s_ti : lane == 7 ? &s_taus[j]
                   : &s_p[(size_t)j * rc + max(0, jl)].x + (lane - 8);            // beta
       if (lane < 8 || (lane < 10 && rank == own && some)) *dst = v10;
+      if (lane == 10) s_rn = rn;
+      if (lane == 11) s_inv = inv;
     } else if (__any_sync(0xffffffffu, on && k > j)) {
       // the parts, in the same order in every CTA
       double a0 = 0, b0 = 0;
@@ -313,7 +323,13 @@ __global__ void __launch_bounds__(PANEL_T, 1) k_qr_panel(const QRBlk* blk, int n
     __syncthreads();
     if (on && k > j) {
       const double2 cr = s_cr, yj = s_row[par][k];
-      const double ti = s_ti;
+      double ti = s_ti;
+#pragma unroll 1
+      for (int q = no_value(ti); q > 0; --q) {
+        tot.x = s_rn * (s_inv * tot.x);
+        tot.y = s_rn * (s_inv * tot.y);
+        ti = 1.0;
+      }
       const double wx = fma(cr.x, yj.x, fma(cr.y, yj.y, ti * tot.x)), wy = fma(cr.x, yj.y, fma(-cr.y, yj.x, ti * tot.y));
       int r = from + ln;
       for (; r + 3 * L < mine; r += 4 * L) {
@@ -501,12 +517,21 @@ __global__ void __launch_bounds__(PT, 1) k_qr_small(const QRItem* items, int n_i
       const bool some = n2 > 0.0 || n2 != n2;
       const double sum = aabs + nrm, inv = some ? 1.0 / sum : 0.0;
       const double cr = rn * ph.x, ci = rn * ph.y, ti = rn * inv;
-      for (int k = j + 1 + lane; k < n; k += 32) {
-        const double2 yj = s_p[j + (size_t)k * m], t = s_tot[k];
-        const double2 w = make_double2(fma(cr, yj.x, fma(ci, yj.y, ti * t.x)), fma(cr, yj.y, fma(-ci, yj.x, ti * t.y)));
+      auto row_j = [&](int k, double2 yj, double2 w) {
         s_w[k] = w;
         const double ux = ph.x * sum, uy = ph.y * sum;
         s_p[j + (size_t)k * m] = make_double2(yj.x - (ux * w.x - uy * w.y), yj.y - (ux * w.y + uy * w.x));
+      };
+      if (!no_value(ti)) {
+        for (int k = j + 1 + lane; k < n; k += 32) {
+          const double2 yj = s_p[j + (size_t)k * m], t = s_tot[k];
+          row_j(k, yj, make_double2(fma(cr, yj.x, fma(ci, yj.y, ti * t.x)), fma(cr, yj.y, fma(-ci, yj.x, ti * t.y))));
+        }
+      } else {
+        for (int k = j + 1 + lane; k < n; k += 32) {
+          const double2 yj = s_p[j + (size_t)k * m], t = make_double2(rn * (inv * s_tot[k].x), rn * (inv * s_tot[k].y));
+          row_j(k, yj, make_double2(fma(cr, yj.x, fma(ci, yj.y, t.x)), fma(cr, yj.y, fma(-ci, yj.x, t.y))));
+        }
       }
       if (lane == 0) {
         s_s = make_double2(ph.x * inv, -ph.y * inv);
