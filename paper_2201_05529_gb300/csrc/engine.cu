@@ -554,6 +554,10 @@ HostMpo fuse(const HostMpo& in, const cplx* LP) {
 // caches the choice in a text file (one line per layer shape: key, QR route, outer-QR route,
 // timings), keyed by GPU name, driver version, compute capability, precision and the layer's
 // capacities. A layer whose key is cached is not timed again.
+// of the kernels behind the choices: raised when one is replaced, so that timings of what is gone are not reused
+// (1, not in the key: the whole-GPU pivoted QR and the unblocked outer QR; 2: clusters only, blocked QR)
+constexpr int TUNE_GENERATION = 2;
+
 std::string tune_key(pt_tebd* h, const std::vector<BondWork>& v, int k_cap, int m_cap) {
   int dev = 0, drv = 0;
   cudaGetDevice(&dev);
@@ -570,8 +574,8 @@ std::string tune_key(pt_tebd* h, const std::vector<BondWork>& v, int k_cap, int 
     mL = std::max(mL, std::max(W.mL_cap, W.nR_cap));
   }
   char buf[512];
-  snprintf(buf, sizeof buf, "%s|drv%d|sm%d%d|p%d|n%zu|k%d|m%d|c%lld|b%d", name.c_str(), drv, prop.major,
-           prop.minor, (int)h->opt.precision, v.size(), k_cap, m_cap, cols, mL);
+  snprintf(buf, sizeof buf, "%s|drv%d|sm%d%d|p%d|n%zu|k%d|m%d|c%lld|b%d|g%d", name.c_str(), drv, prop.major,
+           prop.minor, (int)h->opt.precision, v.size(), k_cap, m_cap, cols, mL, TUNE_GENERATION);
   return buf;
 }
 
