@@ -295,6 +295,9 @@ int pt_selftest_grid_barrier(int withheld_block, double limit_ms, int* device_st
  * limit_ms (0: the usual one; at most 10000) beside the part that grows with the work of a sweep. */
 int pt_selftest_svd(const double* A, int m, int n, int batch, double* sigma, double* U, double* V, void* scratch,
                     int ctas, double limit_ms, void* cuda_stream);
+/* The kernels' reciprocal square root and reciprocal of n values (device), beside CUDA's: out [4][n] (device) gets
+ * theirs, rsqrt(v), theirs, 1 / v. */
+int pt_selftest_reciprocals(const double* v, int n, double* out, void* cuda_stream);
 
 #ifdef __cplusplus
 }

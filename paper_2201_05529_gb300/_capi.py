@@ -30,7 +30,7 @@ EXPORTS = [
     "pt_tebd_sync", "pt_tebd_destroy", "pt_tebd_last_error", "pt_tebd_set_timing",
     "pt_tebd_get_timing", "pt_svd_scratch_bytes", "pt_svd_f64", "pt_svd_f64_noalloc",
     "pt_zgemm_scratch_bytes", "pt_zgemm_sliced", "pt_qr_scratch_bytes", "pt_qr_f64", "pt_selftest_grid_barrier",
-    "pt_selftest_svd",
+    "pt_selftest_svd", "pt_selftest_reciprocals",
 ]
 
 
@@ -126,6 +126,7 @@ lib.pt_svd_f64_noalloc.argtypes = [C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_vo
 NOALLOC_MAX_BYTES = 16 << 20     # PT_SVD_NOALLOC_MAX_BYTES
 
 
+lib.pt_selftest_reciprocals.argtypes = [C.c_void_p, C.c_int, C.c_void_p, C.c_void_p]
 lib.pt_selftest_svd.argtypes = [C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
                                 C.c_int, C.c_double, C.c_void_p]
 lib.pt_selftest_grid_barrier.argtypes = [C.c_int, C.c_double, C.POINTER(C.c_int)]
@@ -485,6 +486,12 @@ def selftest_grid_barrier(withheld_block=-1, limit_ms=1.0):
     st = C.c_int(0)
     rc = lib.pt_selftest_grid_barrier(int(withheld_block), float(limit_ms), C.byref(st))
     return rc, st.value
+
+
+def selftest_reciprocals(v, out, stream=None):
+    """pt_selftest_reciprocals: out [4, n] = the kernels' 1 / sqrt(v), CUDA's, the kernels' 1 / v, CUDA's (float64 tensors)."""
+    st = stream if stream is not None else current_stream_handle()
+    _check(lib.pt_selftest_reciprocals(C.c_void_p(v.data_ptr()), int(v.numel()), C.c_void_p(out.data_ptr()), st), None)
 
 
 def selftest_svd(A, sigma, U, V, scratch, ctas=0, limit_ms=0.0, stream=None):

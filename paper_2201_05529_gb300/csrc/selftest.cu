@@ -1,4 +1,4 @@
-// Diagnostic: the bounded grid barrier's failure path, exercised without a GPU fault.
+// Diagnostics: the bounded grid barrier's failure path, exercised without a GPU fault; the kernels' own reciprocals.
 //
 // Every spin-wait of the path's cooperative kernels (the Jacobi rounds, the pivoted-QR steps) has
 // a time limit after which the waiting CTA records ST_TIMEOUT, raises the launch's abort flag and
@@ -22,7 +22,25 @@ __global__ void k_barrier_selftest(GridSync gs, int* status, int withheld) {
     if (!grid_barrier(gs, status)) return;
 }
 
+// inv_sqrt, rsqrt, inverse and 1 / v of n values
+__global__ void k_reciprocals_selftest(const double* v, int n, double* out) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const double x = v[i];
+    out[i] = inv_sqrt(x);
+    out[(size_t)n + i] = rsqrt(x);
+    out[(size_t)2 * n + i] = inverse(x);
+    out[(size_t)3 * n + i] = 1.0 / x;
+  }
+}
+
 }  // namespace ptk
+
+extern "C" int pt_selftest_reciprocals(const double* v, int n, double* out, void* cuda_stream) {
+  if (!v || n < 1 || !out) return PT_ERR_ARG;
+  ptk::k_reciprocals_selftest<<<152, 256, 0, (cudaStream_t)cuda_stream>>>(v, n, out);
+  if (cudaGetLastError() != cudaSuccess) return PT_ERR_CUDA;
+  return cudaStreamSynchronize((cudaStream_t)cuda_stream) == cudaSuccess ? PT_OK : PT_ERR_CUDA;
+}
 
 extern "C" int pt_selftest_grid_barrier(int withheld_block, double limit_ms, int* device_status) {
   using namespace ptk;
