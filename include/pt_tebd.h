@@ -270,8 +270,8 @@ int pt_zgemm_sliced(int opA, int opB, int m, int n, int k, const double* A, int 
  * (a framework that reserves the GPU up front, a fixed-budget service), or a device allocation is
  * not acceptable where they run (cudaMalloc may synchronise the device and can fail mid-job).
  * The batched FP64 Jacobi SVD without QRs before it, the same arguments and outputs as pt_svd_f64, minus
- * the scratch pointer: the workspace is a static device array of PT_SVD_NOALLOC_MAX_BYTES bytes that
- * every GPU which loads this library holds until the process exits. A problem whose workspace (16
+ * the scratch pointer: the workspace is a static device array of PT_SVD_NOALLOC_MAX_BYTES bytes (and 1/32
+ * more for what the limit does not count) that every GPU which loads this library holds until the process exits. A problem whose workspace (16
  * bytes per element of A and of a min(m, n) x min(m, n) factor, 20 per column, a few hundred per matrix) is larger is rejected with PT_ERR_CAPACITY. The first call on
  * a device looks up the array's device address with that device current and caches it per device
  * index (a cudaDeviceReset invalidates it). All calls share the one array: calls that overlap on the

@@ -90,8 +90,9 @@ void launch_jacobi_cluster(const BondWork* work, int n_work, int cluster, int ma
 int jacobi_grid_blocks();
 constexpr double JACOBI_FLOOR2 = 1.232595164407831e-32;      // squared noise floor: u^2 = 2^-106
 // on_b: 0 = the matrix in A, 1 = B = R^H of the pivoted QR (Na x info[8]), 2 = R^H of the range finder's l x l
-// factor R in G64 (l = info[9]), formed and overwritten by its left vectors in V; with_v: accumulate V; tol_scale: rotation threshold in units of the unit roundoff (0: the
-// row count); wait_cycles: the part of the waits' limit that does not grow with a sweep (0: the usual one); floor2: columns at floor2 ||A||_F^2 or below (squared norms) are left as they are
+// factor R in G64 (l = info[9]), formed and overwritten by its left vectors in V; with_v: accumulate V; tol_scale: rotation
+// threshold in units of the unit roundoff (0: the row count); floor2: columns at floor2 ||A||_F^2 or below (squared norms)
+// are left as they are; wait_cycles: the part of the waits' limit that does not grow with a sweep (0: the usual one)
 cudaError_t launch_jacobi_grid(const BondWork* work, int n_work, int blocks, int rows_cap, int max_sweeps,
                                unsigned* sync3, int* status, cudaStream_t st, int on_b, int with_v, double tol_scale,
                         double floor2 = JACOBI_FLOOR2, long long wait_cycles = 0);
@@ -169,7 +170,6 @@ struct ZGemmItem {
   int* flag;               // set to 1 when a product entry is not finite (NULL: not reported)
   int acc;                 // 0: C = opA(A) opB(B); -1: C = C - opA(A) opB(B)
   int skip_a;              // 1: A's slice planes and row exponents are already in TA (packed earlier)
-  int skip_b;              // 1: B's are already in TB, or another item of the launch writes them there
   const double2* A2;       // rows a_split .. M - 1 of opA(A) come from A2 (same op and leading dimension); NULL: all from A
   int a_split;
   long long split;         // > 0: each K chunk's product goes to C + chunk * split (zgemm9_chunks of them)

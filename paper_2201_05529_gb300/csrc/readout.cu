@@ -205,7 +205,7 @@ void launch_observe(const Tables& T, int n_chains, int n_max, int gx_m, const do
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cl * 2 * n_chains, 1, 1);
   cfg.blockDim = dim3(RD_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = 2 * sizeof(double2) * (size_t)ld;
+  cfg.dynamicSmemBytes = 2 * sizeof(double2) * (size_t)ld;      // at most 16 KB: init takes no bond above 512 (4 chi <= 2048)
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;

@@ -14,14 +14,14 @@
 // level-0 and level-1 sums of a chunk stay integers below 2^24: the tensor cores' FP32 accumulation
 // is exact there, the deeper levels carry only their own rounding, and the chunks are added in
 // FP64 in the output. Products of slice
-// pairs (s, t) accumulate in TMEM by level min(s + t, 3), real and imaginary parts separately
-// (Re = Ar Br - Ai Bi via the MMA's negate-A bit, Im = Ar Bi + Ai Br); the epilogue adds the
+// pairs (s, t) accumulate in TMEM by level min(s + t, 3), real and imaginary parts side by side
+// (B's planes as (-Bi, Br, Bi): Ar (Br, Bi) and Ai (-Bi, Br), one MMA each); the epilogue adds the
 // levels as 64-bit integers and applies 2^(e_row + e_col). The result is accurate to ~1e-12 of the scale
 // of the rows and columns it combines (per 512-long chunk of K); where the terms of an entry add up coherently, in the
 // slices too (constant operands), the FP32 accumulation of the deeper levels truncates to 1.2e-10 of K times that scale.
 //
-// Data flow: one preparation launch (row exponents, then the 12 slice planes in the tcgen05
-// K-major no-swizzle layout: A in 128-row tiles, B in 64-column tiles, one 16-element K step per
+// Data flow: one preparation launch (row exponents, then the slice planes in the tcgen05
+// K-major layout with the 32-byte swizzle: A in 128-row tiles, B in 64-column tiles, one 16-element K step per
 // block, so one cp.async.bulk stages each), then one persistent GEMM launch (one CTA per SM) that
 // walks the live 128 x 64 output tiles of all items with a two-stage bulk-copy / MMA pipeline.
 // Every mbarrier wait is bounded: on expiry the kernel records ST_TIMEOUT in *status, waits
@@ -82,10 +82,10 @@ __device__ __forceinline__ bool item_fits(const ZGemmItem& it) {
 }  // namespace
 
 // Operand preparation, both passes in one launch: a block takes PREP_ROWS rows of opA(A) (blockIdx.x < n_a) or
-// columns of opB(B) of one item, finds each one's exponent e (max |entry| < 2^e), then writes the 12 slice
-// planes: one thread per (row, 8-element K group), 16 bytes per plane, consecutive rows in consecutive
+// columns of opB(B) of one item, finds each one's exponent e (max |entry| < 2^e), then writes the slice planes
+// (A: 2 per slice, B: 3): one thread per (row, 8-element K group), 16 bytes per plane, consecutive rows in consecutive
 // 16-byte slots. Eight rows per block, or 32 where K is at most 64 (a block of eight would have work for 64 threads). The second read of the block's rows comes from L1 or L2.
-// Bound by the integer pipes and the planes' writes (24 bytes per element). Integer arithmetic throughout
+// Bound by the integer pipes and the planes' writes (24 bytes per element of A, 36 of B). Integer arithmetic throughout
 // (tc_common.cuh): with the slices cut by FP64 rint and ldexp in a launch per operand after another for the
 // exponents, the preparation of ten 1120 x 160 x 1120 products took 4.75 ms of the call's 5.68; now ~0.16 of 0.58.
 // mode 0: B, and A unless the item marks it as packed; mode 1: A alone, marked or not.
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(PREP_THREADS) k_zg_prep(const ZGemmItem* items
   const int which = (int)blockIdx.x < n_a ? 0 : 1;
   const int blk = which == 0 ? blockIdx.x : blockIdx.x - n_a, nblk = which == 0 ? n_a : gridDim.x - n_a;
   constexpr int ZNS = Z::NS;
-  if (!item_live(it) || (which == 0 && it.skip_a > 0 && mode == 0) || (which == 1 && it.skip_b > 0)) return;
+  if (!item_live(it) || (which == 0 && it.skip_a > 0 && mode == 0)) return;
   if (!item_fits(it)) {
     if (blk == 0 && threadIdx.x == 0) atomicOr(status, ST_CAPACITY);
     return;
